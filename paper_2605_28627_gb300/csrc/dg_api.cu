@@ -121,7 +121,7 @@ static dg_status checked(Ctx* c, cudaStream_t s) {
 static void release(Ctx* c) {
   if (!c) return;
   if (c->graph) cudaGraphExecDestroy(c->graph);
-  void* bufs[] = {c->d_modal, c->d_D, c->d_metrics, c->d_J, c->d_X, c->d_mms, c->d_Uf, c->d_gf, c->d_lgb, c->d_facegeo, c->d_metrics_f, c->d_facegeo_f,
+  void* bufs[] = {c->d_modal, c->d_jx, c->d_ejx, c->d_D, c->d_metrics, c->d_J, c->d_X, c->d_mms, c->d_Uf, c->d_gf, c->d_lgb, c->d_facegeo, c->d_metrics_f, c->d_facegeo_f,
                   c->d_grad, c->d_fstar, c->d_red, c->d_w, c->d_clock, c->d_U, c->d_G,
                   c->d_adj_qbar, c->d_adj_gbar, c->d_adj_gtil, c->d_adj_fseed, c->d_adj_face, c->d_adj_mu,
                   c->d_adj_stage, c->d_adj_work, c->d_adj_mx, c->d_adj_lgf, c->d_fv_pin, c->d_fv_tab, c->d_fv_iJb, c->d_fv_S, c->d_fv_M, c->d_fv_Fb};
@@ -338,6 +338,9 @@ static dg_status init_impl(const dg_mesh* mesh, const dg_params* prm, int device
        (!alloc((void**)&c->d_Uf, sizeof(double) * E * 6 * 5 * NN, "alloc face states") ||
         !alloc((void**)&c->d_gf, sizeof(double) * E * 6 * 12 * NN, "alloc face gradients") ||
         !alloc((void**)&c->d_lgb, sizeof(double) * (2 * NN + 5 * c->n), "alloc Gauss basis"))) ||
+      (prm->precision != DG_FP32OP && prm->nodes != DG_NODES_LG &&
+       (!alloc((void**)&c->d_jx, sizeof(long long) * E * 10 * P, "alloc metrics (fixed point)") ||
+        !alloc((void**)&c->d_ejx, sizeof(float4) * E, "alloc metric exponents"))) ||
       (prm->precision == DG_FP32OP &&
        (!alloc((void**)&c->d_metrics_f, sizeof(float) * E * 10 * P, "alloc metrics (fp32)") ||
         !alloc((void**)&c->d_facegeo_f, sizeof(float) * c->nfaces * 4 * NN, "alloc facegeo (fp32)"))))
@@ -417,6 +420,7 @@ static dg_status init_impl(const dg_mesh* mesh, const dg_params* prm, int device
   if (err == cudaSuccess) err = setup_kernels(c->N);
   if (err == cudaSuccess) err = build_geometry(*c, d_xgeo, mesh->ngeo, d_bad, s);
   if (err == cudaSuccess && prm->nodes == DG_NODES_LG) err = gauss_geometry(*c, d_bad, s);
+  if (err == cudaSuccess && c->d_jx) err = launch_fx_metrics(*c, s);
   if (err == cudaSuccess && prm->source == DG_SOURCE_MMS) err = launch_mms_phase(*c, s);
   if (err == cudaSuccess && prm->precision == DG_FP32OP) {
     err = launch_to_float(c->d_metrics, c->d_metrics_f, (size_t)E * 10 * P, s);

@@ -15,7 +15,7 @@
 #include <string>
 #include <vector>
 
-#include "dg_stage.cuh"
+#include "dg_volume_fx.cuh"
 
 namespace dg {
 
@@ -26,6 +26,8 @@ struct MemberDev {
   double* clock;              // {t, dt} of this member
   const R* metrics;
   const double* metrics64;
+  const i64* jx;              // fixed-point metric terms and their exponents (FP64)
+  const float4* ejx;
   R* grad;
   R* fstar;
   const R* facegeo;
@@ -71,8 +73,12 @@ k_volume_ens(const MemberDev<R>* __restrict__ mem, int nmem, const int2* __restr
     const int2 tl = tiles[t];
     const MemberDev<R>& m = mem[dg_idx(tl.x, nmem, kSiteEnsMember)];
     StageArgs a{m.U, m.U, m.G, nullptr, m.clock, c_stage, A, B, 1};
-    volume_body<N, R, EPB>(a, m.metrics, m.metrics64, m.grad, m.fstar, m.elem_face, m.mms, Dg, m.E, m.gas,
-                           m.inv_w0, tl.y);
+    if constexpr (sizeof(R) == 8)
+      volume_body_f64<N, EPB>(a, m.metrics, m.jx, m.ejx, m.grad, m.fstar, m.elem_face, m.mms, Dg, m.E, m.gas, m.inv_w0,
+                              tl.y);
+    else
+      volume_body<N, R, EPB>(a, m.metrics, m.metrics64, m.grad, m.fstar, m.elem_face, m.mms, Dg, m.E, m.gas,
+                             m.inv_w0, tl.y);
     __syncthreads();
   }
 }
@@ -98,14 +104,14 @@ struct GroupPlan {
 template <int N, typename R, int EPB>
 static cudaError_t set_vol_attr() {
   return cudaFuncSetAttribute(k_volume_ens<N, R, EPB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)volume_smem_bytes<N, R, EPB>());
+                              (int)volume_op_smem_bytes<N, R, EPB>());
 }
 
 template <int N, typename R>
 struct Epb2 {   // the doubled tile, if it still fits a block (<= 1024 threads, <= 227 KB smem)
   static constexpr int base = default_epb((N + 1) * (N + 1) * (N + 1));
   static constexpr int P = (N + 1) * (N + 1) * (N + 1);
-  static constexpr bool ok = 2 * base * P <= 1024 && volume_smem_bytes<N, R, 2 * base>() + 64 <= 227 * 1024;
+  static constexpr bool ok = 2 * base * P <= 1024 && volume_op_smem_bytes<N, R, 2 * base>() + 4096 <= 227 * 1024;
   static constexpr int value = ok ? 2 * base : base;
 };
 
@@ -137,10 +143,10 @@ static cudaError_t launch_group_stage(const Group& g, int k, const double* A, co
       mem, nmem, g.d_elem_tiles[0], g.n_elem_tiles[0], g.d_D);
   k_face_ens<N, R><<<g.plan.face_grid, 128, 0, s>>>(mem, nmem, g.d_face_tiles, g.n_face_tiles);
   if (ch == 0)
-    k_volume_ens<N, R, e0><<<g.plan.vol_grid, VShape<N, e0>::THREADS, volume_smem_bytes<N, R, e0>(), s>>>(
+    k_volume_ens<N, R, e0><<<g.plan.vol_grid, VShape<N, e0>::THREADS, volume_op_smem_bytes<N, R, e0>(), s>>>(
         mem, nmem, g.d_elem_tiles[0], g.n_elem_tiles[0], g.d_D, C[k], A[k], B[k]);
   else
-    k_volume_ens<N, R, e1><<<g.plan.vol_grid, VShape<N, e1>::THREADS, volume_smem_bytes<N, R, e1>(), s>>>(
+    k_volume_ens<N, R, e1><<<g.plan.vol_grid, VShape<N, e1>::THREADS, volume_op_smem_bytes<N, R, e1>(), s>>>(
         mem, nmem, g.d_elem_tiles[1], g.n_elem_tiles[1], g.d_D, C[k], A[k], B[k]);
   return cudaGetLastError();
 }
@@ -265,6 +271,8 @@ static void fill_member(MemberDev<R>& m, Ctx* c, double* U, double* G, double* c
   m.clock = clock;
   m.metrics = (const R*)(sizeof(R) == 8 ? (const void*)c->d_metrics : (const void*)c->d_metrics_f);
   m.metrics64 = c->d_metrics;
+  m.jx = c->d_jx;
+  m.ejx = c->d_ejx;
   m.grad = (R*)c->d_grad;
   m.fstar = (R*)c->d_fstar;
   m.facegeo = (const R*)(sizeof(R) == 8 ? (const void*)c->d_facegeo : (const void*)c->d_facegeo_f);

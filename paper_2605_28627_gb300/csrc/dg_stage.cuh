@@ -508,12 +508,14 @@ __device__ __forceinline__ void mms_source(const Gas& g, const double* __restric
 
 // LIST: the element slots come from a.list (the DG elements when FV sub-cell
 // elements exist); without it slot = element, as in every other launch.
+// state (FP64, block-shared [EPB], or null): only the elements whose entry is 2
+// are worked on (those that the fixed-point body left).
 template <int N, typename R, int EPB_, bool LIST = false>
 __device__ __forceinline__ void volume_body(const StageArgs& a, const R* __restrict__ metrics,
                                             const double* __restrict__ iJ64, const R* __restrict__ grad,
                                             const R* __restrict__ fstar, const int* __restrict__ elem_face,
                                             const double* __restrict__ mms, const double* __restrict__ Dg, int E,
-                                            const Gas& g, double inv_w0d, int blk) {
+                                            const Gas& g, double inv_w0d, int blk, const int* state = nullptr) {
   using S = VShape<N, EPB_>;
   constexpr int n = S::n, P = S::P, NN = S::NN, EPB = S::EPB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -544,7 +546,7 @@ __device__ __forceinline__ void volume_body(const StageArgs& a, const R* __restr
       if (e >= E) return;   // the whole block, before any barrier
     }
   }
-  const bool active = e < E;
+  const bool active = e < E && (state == nullptr || state[le] == 2);
   __shared__ double s_tc[3];          // sin, cos of pi t (manufactured source); B_s dt (FP32 operator)
   if (threadIdx.x == 0) {
     if (g.source == DG_SOURCE_MMS) sincospi(a.clock[0] + a.c_stage * a.clock[1], &s_tc[0], &s_tc[1]);
@@ -799,7 +801,7 @@ __device__ __forceinline__ void volume_body(const StageArgs& a, const R* __restr
       } else {
         le2 = t / (P / 2); w2 = t - le2 * (P / 2); take = t < EPB * (P / 2);
       }
-      if (take && blk * EPB + le2 < nslot) {
+      if (take && blk * EPB + le2 < nslot && (state == nullptr || state[le2] == 2)) {
         const int hi = w2 / stride;
         const int ia = w2 - hi * stride + stride * (hi % H + n * (hi / H));   // node with r < n/2
         const int ib = ia + H * stride;                                          // its partner

@@ -1,23 +1,28 @@
 // Single-context launcher of the volume kernel (body in dg_stage.cuh): split-form
 // flux differencing, viscous volume term, surface integral, Jacobian, source
 // and LSERK stage update, one element per block (several for small N).
-#include "dg_stage.cuh"
+#include "dg_volume_fx.cuh"
 
 namespace dg {
 
 // LIST: the DG elements of a context with FV sub-cell elements (FP64 only).
 template <int N, typename R, bool LIST>
-__global__ void __launch_bounds__(VShape<N>::THREADS, vol_min_blocks<N, R>())
+__global__ void __launch_bounds__(VShape<N>::THREADS, sizeof(R) == 8 ? fx_min_blocks<N>() : vol_min_blocks<N, R>())
 k_volume2(StageArgs a, const R* __restrict__ metrics, const double* __restrict__ iJ64,
-          const R* __restrict__ grad, const R* __restrict__ fstar, const int* __restrict__ elem_face,
-          const double* __restrict__ mms, const double* __restrict__ Dg, int E, Gas g, double inv_w0) {
-  volume_body<N, R, VShape<N>::EPB, LIST>(a, metrics, iJ64, grad, fstar, elem_face, mms, Dg, E, g, inv_w0,
-                                          blockIdx.x);
+          const i64* __restrict__ jx, const float4* __restrict__ ejx, const R* __restrict__ grad,
+          const R* __restrict__ fstar, const int* __restrict__ elem_face, const double* __restrict__ mms,
+          const double* __restrict__ Dg, int E, Gas g, double inv_w0) {
+  if constexpr (sizeof(R) == 8)
+    volume_body_f64<N, VShape<N>::EPB, LIST>(a, metrics, jx, ejx, grad, fstar, elem_face, mms, Dg, E, g, inv_w0,
+                                             blockIdx.x);
+  else
+    volume_body<N, R, VShape<N>::EPB, LIST>(a, metrics, iJ64, grad, fstar, elem_face, mms, Dg, E, g, inv_w0,
+                                            blockIdx.x);
 }
 
 template <int N, typename R>
 static size_t volume2_smem() {
-  return volume_smem_bytes<N, R, VShape<N>::EPB>();
+  return volume_op_smem_bytes<N, R, VShape<N>::EPB>();
 }
 
 template <int N, typename R, bool LIST>
@@ -34,7 +39,7 @@ cudaError_t volume2_launch(const Ctx& c, const StageArgs& a0, cudaStream_t s) {
   StageArgs a = a0;
   a.nfaces = c.nfaces;
   k_volume2<N, R, LIST><<<blocks, S::THREADS, volume2_smem<N, R>(), s>>>(
-      a, metrics, c.d_metrics, (const R*)c.d_grad, (const R*)c.d_fstar, c.d_elem_face, c.d_mms, c.d_D, c.E, c.gas,
+      a, metrics, c.d_metrics, c.d_jx, c.d_ejx, (const R*)c.d_grad, (const R*)c.d_fstar, c.d_elem_face, c.d_mms, c.d_D, c.E, c.gas,
       1.0 / c.w[0]);
   return cudaGetLastError();
 }
@@ -85,6 +90,16 @@ cudaError_t setup_volume(int N) {
     case 9: return setup_any<9>();
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t launch_fx_metrics(const Ctx& c, cudaStream_t s) {
+  switch (c.N) {
+#define DG_FXM(n) case n: k_fx_metrics<n><<<c.E, 256, 0, s>>>(c.d_metrics, c.d_jx, c.d_ejx); break;
+    DG_FXM(1) DG_FXM(2) DG_FXM(3) DG_FXM(4) DG_FXM(5) DG_FXM(6) DG_FXM(7) DG_FXM(8) DG_FXM(9)
+#undef DG_FXM
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
 }
 
 // Host reader of this file's bounds-check error word (0 in normal builds).

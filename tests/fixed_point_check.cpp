@@ -1,0 +1,148 @@
+// Host build of the fixed-point arithmetic (csrc/dg_fixed.cuh) against long
+// double: error statistics for tests/test_fixed_point.py.
+#include <algorithm>
+#include <cmath>
+#include <cstdlib>
+
+#include "../paper_2605_28627_gb300/csrc/dg_fixed.cuh"
+
+using namespace dg;
+using L = long double;
+
+static double uniform(double a, double b) { return a + (b - a) * drand48(); }
+static int expo(double x) {
+  int e;
+  frexp(x, &e);
+  return e;
+}
+template <class T>
+static T ratio_log(T a, T b) {   // atanh(f)/f, f = (a - b)/(a + b)
+  const T f = (a - b) / (a + b), u = f * f;
+  if (u < T(1e-4)) return 1 + u * (T(1) / 3 + u * (T(1) / 5 + u * (T(1) / 7 + u * (T(1) / 9 + u / 11))));
+  const T z = a / b;
+  return std::log(z) / (2 * ((z - 1) / (z + 1)));
+}
+template <class T>
+static void flux(T ra, T rb, const T* ua, const T* ub, T ba, T bb, const T* sn, T ig, T* F) {
+  T su[3], un = 0, sk = 0;
+  for (int a = 0; a < 3; ++a) {
+    su[a] = ua[a] + ub[a];
+    un += su[a] * sn[a];
+    sk += ua[a] * ua[a] + ub[a] * ub[a];
+  }
+  const T X = (ra + rb) / ratio_log(ra, rb) * un, Y = (ra + rb) / (ba + bb);
+  F[0] = X;
+  F[4] = X * (ratio_log(ba, bb) / (ba + bb) * ig - sk);
+  for (int a = 0; a < 3; ++a) {
+    F[1 + a] = X * su[a] + Y * sn[a];
+    F[4] += su[a] * F[1 + a];
+  }
+}
+
+extern "C" {
+
+// Pairs with density in [r0, r1], pressure in [p0, p1], velocities below um,
+// metric terms below jm (axis: one component only), gamma.  out[0..2]: rms
+// error of the fixed-point mass, momentum and energy flux over the rms flux,
+// out[3..5]: the same of FP64, out[6]: largest |F| as log2, out[7]: pairs
+// outside the range.
+void check_pairs(int count, double r0, double r1, double p0, double p1, double um, double jm, int axis, double gamma,
+                 double* out) {
+  srand48(11);
+  const double ig = 1.0 / (gamma - 1.0), jl = axis ? jm : 3 * jm, bmax = r1 / (8 * p0);
+  FxExp e{expo(r1), expo(um), expo(bmax), expo(jl), 0, 0, 0, 0};
+  const double bmin = std::max(r0 / (8 * p1), ldexp(1.0, e.b - 4));
+  e.lr = (float)(log2(r1) - e.r + 1e-3);
+  e.lu = (float)(log2(um) - e.u + 1e-3);
+  e.lj = (float)(log2(jl) - e.j + 1e-3);
+  e.lb = (float)(log2(bmin) - e.b - 1e-3);
+  const int eD = 5, eg = expo(ig);
+  const FxAlign al = fx_align(e, eg, (float)(log2(ig) - eg + 1e-3), eD);
+  const Fx G = fx_split(fx_from(ig, 62 - eg));
+  double ef[3] = {0}, ed[3] = {0}, sc[3] = {0}, big = 0;
+  long outside = 0;
+  for (int t = 0; t < count; ++t) {
+    // both nodes anywhere in the range, close together, or equal
+    const double ra = uniform(r0, r1), pa = uniform(p0, p1), near = t % 3 == 1 ? 1e-2 : 1e-5;
+    double rb = t % 3 == 0 ? uniform(r0, r1) : std::min(r1, std::max(r0, ra * (1 + uniform(-near, near))));
+    double pb = t % 3 == 0 ? uniform(p0, p1) : std::min(p1, std::max(p0, pa * (1 + uniform(-near, near))));
+    if (t % 7 == 0) { rb = ra; pb = pa; }
+    double ua[3], ub[3], na[3], nb[3], sn[3];
+    for (int a = 0; a < 3; ++a) {
+      const bool on = !axis || a == 0;
+      ua[a] = uniform(-um, um); ub[a] = uniform(-um, um);
+      na[a] = on ? uniform(-jm, jm) : 0; nb[a] = on ? uniform(-jm, jm) : 0;
+      sn[a] = na[a] + nb[a];
+    }
+    const double ba = 0.125 * ra / pa, bb = 0.125 * rb / pb;
+    const i64 xr[2] = {fx_from(ra, 60 - e.r), fx_from(rb, 60 - e.r)}, xb[2] = {fx_from(ba, 60 - e.b), fx_from(bb, 60 - e.b)};
+    const i64 least = (i64)1 << 56;
+    if (std::min(std::min(xr[0], xr[1]), std::min(xb[0], xb[1])) < least || ba < bmin || bb < bmin) { ++outside; continue; }
+    i64 su[3], n2[3];
+    double ka = 0, kb = 0;
+    for (int a = 0; a < 3; ++a) {
+      su[a] = fx_from(ua[a], 60 - e.u) + fx_from(ub[a], 60 - e.u);
+      n2[a] = fx_from(na[a], 60 - e.j) + fx_from(nb[a], 60 - e.j);
+      ka += ua[a] * ua[a]; kb += ub[a] * ub[a];
+    }
+    i64 F[5];
+    fx_pair(xr[0], xr[1], xb[0], xb[1], su[0], su[1], su[2], fx_from(ka, 58 - 2 * e.u) + fx_from(kb, 58 - 2 * e.u), n2[0],
+            n2[1], n2[2], G, al, F, [](i64 a, i64 b, i64 c, i64 d, i64 y, i64 u, i64 v) {
+              return fx_means_long(a, b, c, d, y, u, v, [](double p, double q) { return ratio_log<double>(p, q); });
+            });
+    L la[3], lb[3], ln[3], R[5];
+    for (int a = 0; a < 3; ++a) { la[a] = ua[a]; lb[a] = ub[a]; ln[a] = (L)na[a] + nb[a]; }
+    flux<L>(ra, rb, la, lb, ba, bb, ln, ig, R);
+    double D[5];
+    flux<double>(ra, rb, ua, ub, ba, bb, sn, ig, D);
+    for (int v = 0; v < 5; ++v) {
+      const int q = (v == 0 ? al.q0 - 2 : (v < 4 ? al.qm - 3 : al.qe - 4)) - (kFxQD - eD - 64);
+      const double d = (double)(std::ldexp((L)F[v], -q) - R[v]), s = (double)R[v];
+      const int c = v == 0 ? 0 : (v < 4 ? 1 : 2);   // the momentum as one vector
+      ef[c] += d * d;
+      ed[c] += (double)((D[v] - R[v]) * (D[v] - R[v]));
+      sc[c] += s * s;
+      big = std::max(big, std::fabs((double)F[v]));
+    }
+  }
+  for (int c = 0; c < 3; ++c) {
+    out[c] = std::sqrt(ef[c] / sc[c]);
+    out[3 + c] = std::sqrt(ed[c] / sc[c]);
+  }
+  out[6] = std::log2(big);
+  out[7] = (double)outside;
+}
+
+// Largest relative error of 2^119 / S over S in [2^57, 2^61).
+double check_rcp(int count) {
+  srand48(12);
+  double worst = 0;
+  for (int t = 0; t < count; ++t) {
+    const i64 S = t < 16 ? ((i64)1 << (57 + t % 4)) + t / 4 : (i64)ldexp(1 + drand48(), 57 + t % 4);
+    const Fx s = fx_split(S);
+    const L y = std::ldexp((L)1, 119) / (L)S;
+    worst = std::max(worst, (double)std::fabs(((L)fx_rcp_full(s, fx_rcp(s)) - y) / y));
+  }
+  return worst;
+}
+
+// Conversions: worst error of fx_from in units of its last bit, of fx_to and
+// fx_to2 relative to the value.
+void check_conversions(int count, double* out) {
+  srand48(13);
+  out[0] = out[1] = out[2] = 0;
+  for (int t = 0; t < count; ++t) {
+    double x = t < 4 ? (t & 1 ? -0.0 : 0.0) : ldexp(drand48() - 0.5, (int)(drand48() * 70) - 68);
+    if (t == 4) x = 5e-324;
+    out[0] = std::max(out[0], (double)std::fabs((L)fx_from(x, 60) - std::ldexp((L)x, 60)));
+    const i64 X = (i64)ldexp(drand48() - 0.5, (int)(drand48() * 63)) ^ (i64)(lrand48() & 0xff);
+    if (X) out[1] = std::max(out[1], (double)std::fabs(((L)fx_to(X, 9) - std::ldexp((L)X, -9)) / std::ldexp((L)X, -9)));
+    const i64 c = (i64)ldexp(drand48() - 0.5, 63);
+    {
+      const L v = std::ldexp((L)X + std::ldexp((L)c, -32), -9);
+      if (std::fabs(v) > 65536) out[2] = std::max(out[2], (double)std::fabs(((L)fx_to2<32>(X, c, 9) - v) / v));
+    }
+  }
+  if (fx_to(0, 9) != 0.0 || fx_to2<32>(0, 0, 9) != 0.0) out[1] = 1;
+}
+}

@@ -1,0 +1,62 @@
+"""The fixed-point arithmetic of the FP64 kernels, built for the host: its
+conversions, reciprocal and two-point flux against long double.
+
+Bars: a conversion to fixed point truncates to one unit of 2^-60; back to
+FP64 it rounds to nearest (2^-53, and 2^-32 units, of the 96-bit
+sums' last word); the reciprocal is good to 2^-55; the flux stays below 2^60.5, so
+that the sums with a row of D cannot overflow, and its error is no larger than
+that of the same formula in FP64 over the whole admitted range of the data."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("fx") / "fixed_point_check.so")
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-fwrapv", "-shared", "-fPIC", "-o", so,
+                           os.path.join(HERE, "fixed_point_check.cpp")])
+    L = C.CDLL(so)
+    L.check_rcp.restype = C.c_double
+    L.check_pairs.argtypes = [C.c_int] + [C.c_double] * 6 + [C.c_int, C.c_double, C.c_void_p]
+    return L
+
+
+def test_conversions(lib):
+    out = np.zeros(3)
+    lib.check_conversions(200000, out.ctypes.data_as(C.c_void_p))
+    assert out[0] < 1.0 and out[1] <= 2.0 ** -53 and out[2] <= 2.0 ** -52.9, out
+
+
+def test_reciprocal(lib):
+    assert lib.check_rcp(200000) < 2.0 ** -55
+
+
+# density, pressure, velocity, metric terms, one-component metrics, gamma:
+# random states of the parity tests, low Mach numbers, the density wave, Mach 2
+# and 30, densities over the whole admitted range, gamma near 1 and large
+@pytest.mark.parametrize("r0,r1,p0,p1,um,jm,axis,gamma", [
+    (0.8, 1.2, 0.8, 1.2, 0.5, 1.0, 0, 1.4),
+    (0.99, 1.01, 71.0, 72.0, 1.0, 0.01, 1, 1.4),
+    (0.9999, 1.0001, 714285.0, 714286.0, 1.0, 0.3, 0, 1.4),
+    (1.9, 2.1, 1.0, 1.001, 1.01, 0.004, 0, 1.4),
+    (0.5, 1.5, 0.8, 2.0, 3.0, 1.0, 1, 1.4),
+    (1.0, 1.1, 0.9, 1.0, 35.0, 2e-9, 0, 1.4),
+    (1.0, 7.9, 1.0, 6.0, 1.0, 1.0, 1, 1.4),
+    (0.126, 1.0, 0.1, 1.0, 0.3, 50.0, 0, 1.4),
+    (1e-7, 1.2e-7, 1e20, 1.1e20, 1e13, 1e6, 1, 1.05),
+    (0.8, 1.2, 0.8, 1.2, 0.5, 1.0, 1, 3.0),
+])
+def test_two_point_flux(lib, r0, r1, p0, p1, um, jm, axis, gamma):
+    out = np.zeros(8)
+    n = 20000
+    lib.check_pairs(n, r0, r1, p0, p1, um, jm, axis, gamma, out.ctypes.data_as(C.c_void_p))
+    fixed, fp64 = out[:3], out[3:6]
+    assert out[7] < 0.8 * n
+    assert out[6] < 60.5, out[6]
+    assert (fixed <= fp64).all(), (fixed, fp64)

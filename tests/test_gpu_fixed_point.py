@@ -1,0 +1,95 @@
+"""FP64 operator on LGL nodes: block fixed point against the oracle where its
+range and its branches end -- densities varying by more than the series of the
+logarithmic means take (ratio 1.13 and 1.67), by about the admitted factor of
+8 to 16 and beyond it (those elements run in FP64), blocks that hold elements
+of both kinds, velocities of zero and of Mach 17, low Mach numbers and states
+of far-off scales.
+
+Bar: R(U) within 1e-12 of max |R| per variable and ten RK steps within 1e-10,
+as for the parity tests.  The momentum of R comes from the variation of the
+pressure while the rounding of the metric terms (1e-13 between the two codes)
+multiplies its mean, so the bar grows with their quotient (2.5 for the ranges
+0.8 to 1.2, 5.5 for the low Mach number).  Meshes above the node count of the
+latency kernels, with ragged last blocks."""
+import numpy as np
+import pytest
+
+from workloads import box_mesh, random_state
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+SIZE = {1: 13, 2: 9, 3: 7, 4: 3, 5: 3, 7: 2, 8: 2}
+
+
+def _cuda(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def _err(got, ref):
+    d = np.abs(got - ref).reshape(ref.shape[0], 5, -1).max(axis=(0, 2))
+    return d / np.abs(ref).reshape(ref.shape[0], 5, -1).max(axis=(0, 2))
+
+
+STATES = {
+    "means by long series": dict(rho=(0.75, 1.0), p=(0.75, 1.0)),
+    "means by logarithm": dict(rho=(0.3, 1.0), p=(0.4, 1.0)),
+    "edge of the range": dict(rho=(0.08, 1.0), p=(0.8, 1.0)),
+    "FP64 elements": dict(rho=(0.03, 1.0), p=(0.8, 1.2)),
+    "at rest": dict(vel=0.0),
+    "Mach 17": dict(vel=20.0),
+    "low Mach": dict(vel=0.5, p=(1.0e5, 1.2e5)),
+    "far-off scales": dict(rho=(0.8e-9, 1.2e-9), vel=1e8, p=(0.8e7, 1.2e7)),
+}
+
+
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 7, 8])
+@pytest.mark.parametrize("kind", list(STATES))
+def test_time_derivative(orc, N, kind):
+    import paper_2605_28627_gb300 as dg
+    mesh = box_mesh(SIZE[N], min(N, 4), deform="sinprod", rotate_seed=400 + N)
+    mu = 0.02 * (STATES[kind].get("rho", (1, 1))[1] * STATES[kind].get("vel", 0.5) if kind == "far-off scales" else 1.0)
+    o, s = orc.Oracle(mesh, N, mu=mu), dg.Solver(mesh, N, mu=mu)
+    U = random_state(mesh.n_elems, N, seed=500 + N, **STATES[kind])
+    err = _err(s.time_derivative(_cuda(U)).cpu().numpy(), o.time_derivative(U))
+    p = STATES[kind].get("p", (0.8, 1.2))
+    assert (err < 1e-12 * max(1.0, 0.5 * (p[0] + p[1]) / (p[1] - p[0]))).all(), err
+
+
+@pytest.mark.parametrize("N", [1, 3, 4, 7])
+def test_blocks_of_both_kinds(orc, N):
+    """Every third element outside the fixed-point range, R(U) and RK steps in
+    place (each element is written by one of the two bodies)."""
+    import paper_2605_28627_gb300 as dg
+    mesh = box_mesh(SIZE[N], min(N, 4), deform="sinprod", rotate_seed=420 + N)
+    o, s = orc.Oracle(mesh, N, mu=0.01), dg.Solver(mesh, N, mu=0.01)
+    U = random_state(mesh.n_elems, N, seed=520 + N)
+    W = random_state(mesh.n_elems, N, seed=521 + N, rho=(0.03, 1.0))
+    U[::3] = W[::3]
+    err = _err(s.time_derivative(_cuda(U)).cpu().numpy(), o.time_derivative(U))
+    assert (err < 1e-12).all(), err
+    Ud = _cuda(U)
+    s.rk_step(Ud, torch.empty_like(Ud), 0.0, 2e-5, 10)
+    ref = o.rk_steps(U, 0.0, 2e-5, 10)
+    assert np.abs(Ud.cpu().numpy() - ref).max() / np.abs(ref).max() < 1e-10
+
+
+def test_non_finite_state_stays_local():
+    """A NaN gives NaN in its element and leaves elements that do not touch it
+    as they are, bit for bit; so does an infinity."""
+    import paper_2605_28627_gb300 as dg
+    N = 3
+    mesh = box_mesh(7, 3, deform="sinprod", rotate_seed=430)
+    s = dg.Solver(mesh, N, mu=0.01)
+    U = _cuda(random_state(mesh.n_elems, N, seed=530))
+    R = s.time_derivative(U)
+    e = 100
+    near = {e} | set(int(x) for x in mesh.face_nbr[e, :, 0])
+    near |= {int(x) for a in list(near) for x in mesh.face_nbr[a, :, 0]}
+    far = [x for x in range(mesh.n_elems) if x not in near]
+    for bad in (float("nan"), float("inf")):
+        V = U.clone()
+        V[e, 4, 1, 2, 1] = bad
+        Rv = s.time_derivative(V)
+        assert not bool(torch.isfinite(Rv[e]).all())
+        assert torch.equal(Rv[far], R[far])
