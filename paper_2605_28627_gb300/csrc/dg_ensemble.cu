@@ -15,6 +15,7 @@
 #include <string>
 #include <vector>
 
+#include "dg_lift_fx.cuh"
 #include "dg_volume_fx.cuh"
 
 namespace dg {
@@ -50,7 +51,11 @@ k_lift_ens(const MemberDev<R>* __restrict__ mem, int nmem, const int2* __restric
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int2 tl = tiles[t];
     const MemberDev<R>& m = mem[dg_idx(tl.x, nmem, kSiteEnsMember)];
-    lift_body<N, R, EPB>(m.U, m.metrics, m.elem_nbr, m.elem_face, Dg, m.grad, m.E, m.gas, m.inv_w0, tl.y);
+    if constexpr (sizeof(R) == 8)
+      lift_body_fx<N, EPB>(m.U, m.metrics, m.jx, m.ejx, m.elem_nbr, m.elem_face, Dg, m.grad, m.E, m.gas, m.inv_w0,
+                           tl.y);
+    else
+      lift_body<N, R, EPB>(m.U, m.metrics, m.elem_nbr, m.elem_face, Dg, m.grad, m.E, m.gas, m.inv_w0, tl.y);
     __syncthreads();
   }
 }
@@ -139,7 +144,7 @@ static cudaError_t launch_group_stage(const Group& g, int k, const double* A, co
   const int ch = g.plan.epb_choice;
   // lifting always uses the default tile (its tile table is choice 0)
   const int nmem = (int)g.members.size();
-  k_lift_ens<N, R, e0><<<g.plan.lift_grid, Shape<N, e0>::THREADS, lift_smem_bytes<N, R, e0>(), s>>>(
+  k_lift_ens<N, R, e0><<<g.plan.lift_grid, Shape<N, e0>::THREADS, lift_op_smem_bytes<N, R, e0>(), s>>>(
       mem, nmem, g.d_elem_tiles[0], g.n_elem_tiles[0], g.d_D);
   k_face_ens<N, R><<<g.plan.face_grid, 128, 0, s>>>(mem, nmem, g.d_face_tiles, g.n_face_tiles);
   if (ch == 0)
@@ -154,7 +159,7 @@ static cudaError_t launch_group_stage(const Group& g, int k, const double* A, co
 template <int N, typename R>
 static cudaError_t setup_group() {
   cudaError_t e = cudaFuncSetAttribute(k_lift_ens<N, R, Shape<N>::EPB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)lift_smem_bytes<N, R, Shape<N>::EPB>());
+                                       (int)lift_op_smem_bytes<N, R, Shape<N>::EPB>());
   if (e == cudaSuccess) e = set_vol_attr<N, R, Shape<N>::EPB>();
   if (e == cudaSuccess) e = set_vol_attr<N, R, Epb2<N, R>::value>();
   return e;

@@ -1,6 +1,6 @@
 // Single-context launchers of the lifting and face-flux kernels (bodies in
 // dg_stage.cuh): one thread per volume node (lifting) or face node (face flux).
-#include "dg_stage.cuh"
+#include "dg_lift_fx.cuh"
 
 namespace dg {
 
@@ -14,6 +14,17 @@ k_lift(const double* __restrict__ U, const R* __restrict__ metrics, const int* _
        const int* __restrict__ elem_face, const double* __restrict__ Dg, R* __restrict__ grad, int E, Gas g,
        double inv_w0, const double* __restrict__ mvirt, int n_mortar) {
   lift_body<N, R, Shape<N>::EPB, MORTAR>(U, metrics, elem_nbr, elem_face, Dg, grad, E, g, inv_w0, blockIdx.x,
+                                         mvirt, n_mortar);
+}
+template <int N>
+constexpr int lift_fx_min_blocks() { return Shape<N>::THREADS <= 512 ? 1024 / Shape<N>::THREADS : 1; }
+template <int N, bool MORTAR>
+__global__ void __launch_bounds__(Shape<N>::THREADS, lift_fx_min_blocks<N>())
+k_lift_fx(const double* __restrict__ U, const double* __restrict__ metrics, const i64* __restrict__ jx,
+          const float4* __restrict__ ejx, const int* __restrict__ elem_nbr, const int* __restrict__ elem_face,
+          const double* __restrict__ Dg, double* __restrict__ grad, int E, Gas g, double inv_w0,
+          const double* __restrict__ mvirt, int n_mortar) {
+  lift_body_fx<N, Shape<N>::EPB, MORTAR>(U, metrics, jx, ejx, elem_nbr, elem_face, Dg, grad, E, g, inv_w0, blockIdx.x,
                                          mvirt, n_mortar);
 }
 
@@ -43,6 +54,21 @@ static cudaError_t lift_NR(const Ctx& c, const double* U, cudaStream_t s) {
   if (c.M > 0) {   // the mortar sides' neighbour states first
     cudaError_t e = launch_mortar_lift(c, U, s);
     if (e != cudaSuccess) return e;
+  }
+  if constexpr (sizeof(R) == 8) {
+    if (c.d_jx) {   // absent in an FP32-operator context, whose diagnostics lift in FP64
+      if (c.M > 0)
+        k_lift_fx<N, true><<<blocks, S::THREADS, lift_fx_smem_bytes<N, S::EPB>(), s>>>(
+            U, c.d_metrics, c.d_jx, c.d_ejx, c.d_elem_nbr, c.d_elem_face, c.d_D, (double*)c.d_grad, c.E, c.gas,
+            1.0 / c.w[0], c.d_mortar_virt, c.M);
+      else
+        k_lift_fx<N, false><<<blocks, S::THREADS, lift_fx_smem_bytes<N, S::EPB>(), s>>>(
+            U, c.d_metrics, c.d_jx, c.d_ejx, c.d_elem_nbr, c.d_elem_face, c.d_D, (double*)c.d_grad, c.E, c.gas,
+            1.0 / c.w[0], nullptr, 0);
+      return cudaGetLastError();
+    }
+  }
+  if (c.M > 0) {
     k_lift<N, R, true><<<blocks, S::THREADS, lift_smem_bytes<N, R, S::EPB>(), s>>>(
         U, metrics, c.d_elem_nbr, c.d_elem_face, c.d_D, (R*)c.d_grad, c.E, c.gas, 1.0 / c.w[0], c.d_mortar_virt, c.M);
     return cudaGetLastError();
@@ -115,6 +141,12 @@ static cudaError_t setup_lift_N() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_lift<N, double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)lift_smem_bytes<N, double, Shape<N>::EPB>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_lift_fx<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)lift_fx_smem_bytes<N, Shape<N>::EPB>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_lift_fx<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)lift_fx_smem_bytes<N, Shape<N>::EPB>());
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_lift<N, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)lift_smem_bytes<N, float, Shape<N>::EPB>());
