@@ -15,6 +15,7 @@
 #include <string>
 #include <vector>
 
+#include "dg_face_fx.cuh"
 #include "dg_lift_fx.cuh"
 #include "dg_volume_fx.cuh"
 
@@ -66,7 +67,10 @@ k_face_ens(const MemberDev<R>* __restrict__ mem, int nmem, const int2* __restric
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int2 tl = tiles[t];
     const MemberDev<R>& m = mem[dg_idx(tl.x, nmem, kSiteEnsMember)];
-    face_body<N, R>(m.U, m.grad, m.faces, m.facegeo, m.fstar, m.F, m.E, m.gas, (long)tl.y * 128 + threadIdx.x);
+    if constexpr (sizeof(R) == 8)
+      face_body_fx<N>(m.U, m.grad, m.faces, m.facegeo, m.fstar, m.F, m.E, m.gas, (long)tl.y * 128 + threadIdx.x);
+    else
+      face_body<N, R>(m.U, m.grad, m.faces, m.facegeo, m.fstar, m.F, m.E, m.gas, (long)tl.y * 128 + threadIdx.x);
   }
 }
 

@@ -1,5 +1,6 @@
 // Single-context launchers of the lifting and face-flux kernels (bodies in
 // dg_stage.cuh): one thread per volume node (lifting) or face node (face flux).
+#include "dg_face_fx.cuh"
 #include "dg_lift_fx.cuh"
 
 namespace dg {
@@ -42,7 +43,8 @@ k_face(const double* __restrict__ U, const R* __restrict__ grad, const FaceInfo*
     if (fv_mask[dg_idx(fi.master >> 3, E, kSiteFaceElems)] || fv_mask[dg_idx(fi.slave >> 3, E, kSiteFaceElems)])
       return;
   }
-  face_body<N, R>(U, grad, faces, facegeo, fstar, F, E, g, gid);
+  if constexpr (sizeof(R) == 8) face_body_fx<N>(U, grad, faces, facegeo, fstar, F, E, g, gid);
+  else face_body<N, R>(U, grad, faces, facegeo, fstar, F, E, g, gid);
 }
 
 // ---------------------------------------------------------------------------
