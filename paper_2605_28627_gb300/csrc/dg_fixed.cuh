@@ -143,28 +143,47 @@ DG_HD double fx_from_bits(i64 b) {
 // x 2^q truncated to an integer, |x 2^q| < 2^62, integer instructions only.
 DG_HD i64 fx_from(double x, int q) {
   const i64 b = fx_bits(x);
-  const int hi = (int)((u64)b >> 32);
-  const int ex = (hi >> 20) & 0x7ff;
-  u64 m = (((u64)b & 0xfffffffffffffull) | 0x10000000000000ull) << 9;   // 62 bits
-  int r = 1075 + 9 - q - ex;                                              // right shift, >= 0
-  m >>= r < 63 ? r : 63;
+  const int hi = fx_high(b);
+  const u64 m = (((u64)b & 0xfffffffffffffull) | 0x10000000000000ull) << 9;   // 62 bits
+  const unsigned r = (unsigned)(1084 - q - ((hi >> 20) & 0x7ff));              // right shift, >= 0
+#ifdef __CUDA_ARCH__
+  i64 v;
+  asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(r));                       // 0 for r > 63
+#else
+  const i64 v = r < 64 ? (i64)(m >> r) : 0;
+#endif
   const i64 s = (i64)(hi >> 31);
-  return ((i64)m ^ s) - s;
+  return (v ^ s) - s;
 }
 
-// X 2^(-q) as a double, rounded to nearest (ties away); the result must be normal or zero.
+// x 2^q to the nearest integer, |x 2^q| < 2^61: tables.
+DG_HD i64 fx_round(double x, int q) { return (fx_from(x, q + 1) + 1) >> 1; }
+
+// X 2^(-q) as a double, rounded to nearest (ties away; a negative X by at most
+// one unit of X more); the result must be normal or zero.
 DG_HD double fx_to(i64 x, int q) {
-  const u64 a = x < 0 ? (u64)0 - (u64)x : (u64)x;
+  uint32_t h = (uint32_t)fx_high(x), l = (uint32_t)(u64)x;
+  const uint32_t sg = (uint32_t)((int)h >> 31);
+  const u64 t = (((u64)(h ^ sg) << 32) | (l ^ sg)) + (sg & 1u);
+  h = (uint32_t)(t >> 32);
+  l = (uint32_t)t;
+  int e = 1085 - q;
+  if (h == 0) {
+    h = l;
+    l = 0;
+    e -= 32;
+  }
 #ifdef __CUDA_ARCH__
-  const int z = __clzll((i64)a);
+  const int z = __clz((int)h);
+  const uint32_t nh = __funnelshift_l(l, h, z), nl = z < 32 ? l << z : 0u;
+  const uint32_t lo = __funnelshift_r(nl, nh, 11);
 #else
-  const int z = a ? __builtin_clzll(a) : 64;
+  const int z = h ? __builtin_clz(h) : 32;
+  const uint32_t nh = z & 31 ? (h << (z & 31)) | (l >> (32 - (z & 31))) : h, nl = z < 32 ? l << z : 0u;
+  const uint32_t lo = (nl >> 11) | (nh << 21);
 #endif
-  const u64 n = a << (z & 63);
-  const u64 m = (n >> 11) + ((n >> 10) & 1);
-  u64 bits = ((u64)(uint32_t)(1085 - z - q) << 52) + m;
-  bits = a ? bits : 0;
-  return fx_from_bits((i64)(bits | ((u64)x & 0x8000000000000000ull)));
+  const u64 r = ((u64)((nh >> 11) + ((uint32_t)(e - z) << 20)) << 32 | lo) + ((nl >> 10) & 1u);
+  return fx_from_bits((i64)(nh ? r | ((u64)(sg & 0x80000000u) << 32) : 0));
 }
 
 // (p + c 2^(-CB)) 2^(-q) as a double, rounded (to 2^-96 of the leading bit's
@@ -179,12 +198,14 @@ DG_HD double fx_to2(i64 p, i64 c, int q) {
   l ^= sg;
   f ^= sg;
   int z0 = 0;
-  if (h == 0) {
-    h = l;
-    l = f;
-    f = 0;
-    z0 = 32;
-  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+    if (h == 0) {
+      h = l;
+      l = f;
+      f = 0;
+      z0 += 32;
+    }
 #ifdef __CUDA_ARCH__
   const int z = __clz((int)h);
   const uint32_t nh = __funnelshift_l(l, h, z), nl = __funnelshift_l(f, l, z);
@@ -193,7 +214,7 @@ DG_HD double fx_to2(i64 p, i64 c, int q) {
   const uint32_t nh = z & 31 ? (h << (z & 31)) | (l >> (32 - (z & 31))) : h;
   const uint32_t nl = z & 31 ? (l << (z & 31)) | (f >> (32 - (z & 31))) : l;
 #endif
-  if (h == 0) return 0.0;   // below the unit of p
+  if (h == 0) return 0.0;
   const u64 n = ((u64)nh << 32) | nl;
   const u64 m = (n >> 11) + ((n >> 10) & 1);
   const u64 bits = ((u64)(uint32_t)(1085 - z - z0 - q) << 52) + m;
@@ -246,7 +267,7 @@ constexpr int kFxQ = 60;
 // the next product fill 62 bits whatever the element's values (sums of few
 // products then lose little to rounding), down by s* to align two terms (one
 // of each two is zero); bits after the point of the five components, as summed
-// with D at 58 - e_D and with the factors 1/4, 1/8, 1/16 of D taken in (see
+// with D at 60 - e_D and with the factors 1/4, 1/8, 1/16 of D taken in (see
 // fx_pair).
 struct alignas(16) FxAlign {
   int ky, ku, kx, k4;       // 1/(b_a + b_b), {u}.n, xf and y4 in the momentum flux
@@ -254,7 +275,11 @@ struct alignas(16) FxAlign {
   int sz1, sz2, se1, se2;
   int q0, qm, qe, pad;
 };
-constexpr int kFxQD = 58;   // bits of D, less e_D
+// Bits of D, less e_D (with 58, truncated, the representation of D was the
+// largest error of R; 61 would let the sums of nine terms overflow), and what
+// line sums shift up by to keep 62 - e_D as their scale.
+constexpr int kFxQD = 60;
+constexpr int kFxUpD = 62 - kFxQD;
 DG_HD int fx_floor(float x) { return (int)x - (x < (float)(int)x ? 1 : 0); }
 DG_HD float fx_log2_sum(float a, float b) {   // log2(2^a + 2^b), rounded up
   const float m = a > b ? a : b, d = a > b ? b - a : a - b;
@@ -380,7 +405,7 @@ DG_HD FxMeans fx_means_long(i64 ra, i64 rb, i64 ba, i64 bb, i64 yb, i64 Ur, i64 
 // Bounds: sums of two velocities and of two metric terms are below 2^61 (the
 // latter also summed over l), so a product sum stays below 2^63 in p and c; xf
 // stays below 2^59, M below 2^60 and E below 2^60.4, so that nine terms of a row of D,
-// with 58 - e_D bits, fit in c between two fx_fold.  Factors are shifted up
+// with 60 - e_D bits, fit in c between two fx_fold.  Factors are shifted up
 // before a product rather than the product after it, where the low * low part
 // that fx_add leaves out would count.
 template <class LONG>

@@ -79,7 +79,7 @@ __device__ __forceinline__ void lift_body_fx(const double* __restrict__ U, const
   double phi[4] = {0, 0, 0, 0};
   double qn[5] = {1, 0, 0, 0, 0};
   if constexpr (NI == 1) load_nbr(threadIdx.x, qn);
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) sD[t] = fx_split(fx_from(Dg[t], kFxQD - eD));
+  for (int t = threadIdx.x; t < n * n; t += blockDim.x) sD[t] = fx_split(fx_round(Dg[t], kFxQD - eD));
   for (int t = threadIdx.x; t < EPB * 2; t += blockDim.x) s_mx[t >> 1][t & 1] = 0;
   if (active) {
     double q[5];
@@ -143,7 +143,7 @@ __device__ __forceinline__ void lift_body_fx(const double* __restrict__ U, const
       const i64 own[4] = {p0.x, p0.y, p1.x, p1.y};
       const int eu2 = expo(s_mx[le2][0]), et2 = expo(s_mx[le2][1]);
       if (eu2 < 90 && et2 < 90 && ejx[blk * EPB + le2].x < 90.0f) {
-        const Fx hx = fx_split(fx_from(hs, kFxQD - eD));
+        const Fx hx = fx_split(fx_round(hs, kFxQD - eD));
 #pragma unroll
         for (int a = 0; a < 4; ++a)
           sj[a * NN] = fx_mul<0>(fx_split(fx_from(__longlong_as_double(sj[a * NN]), kFxQ - (a < 3 ? eu2 : et2)) - own[a]), hx);
@@ -208,7 +208,7 @@ __device__ __forceinline__ void lift_body_fx(const double* __restrict__ U, const
       fx_add(s[3], D, fx_split(p1.y));
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a) dd[a][d] = fx_end<4>(s[a]);
+    for (int a = 0; a < 4; ++a) dd[a][d] = fx_end<kFxUpD>(s[a]);
   }
   // g_l = (1/J) sum_d Ja^d_l dd_d
   const i64* mt = jx + (size_t)e * 10 * P + id;

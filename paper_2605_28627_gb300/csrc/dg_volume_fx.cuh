@@ -34,7 +34,7 @@ constexpr int fx_min_blocks() {
   return threads <= 512 ? (768 / threads > 1 ? 768 / threads : 2) : 1;
 }
 
-// Shared memory: the Fx table of D (58 - e_D bits), then per element, in words
+// Shared memory: the Fx table of D (60 - e_D bits), then per element, in words
 // of 8 bytes: (rho, b), (|u|^2, u), (v, w) as pairs (6 P), the viscous sums (4
 // P), and the metric terms of the three directions as a pair and a single with
 // the exchange buffers (pairs F0 F1, F2 F3 and F4), which the viscous fluxes
@@ -162,7 +162,7 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
   for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
     const double d = Dg[t];
     // the corners carry the viscous part of the surface term, as in volume_body
-    sD[t] = fx_split(fx_from(t == 0 ? d + inv_w0 : (t == n * n - 1 ? d - inv_w0 : d), kFxQD - eD));
+    sD[t] = fx_split(fx_round(t == 0 ? d + inv_w0 : (t == n * n - 1 ? d - inv_w0 : d), kFxQD - eD));
   }
   for (int t = threadIdx.x; t < EPB * kMxCount; t += blockDim.x) s_mx[t / kMxCount][t % kMxCount] = 0;
   // state by bulk copy into the region of the metric terms and fluxes
@@ -283,7 +283,7 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
     // viscous line sums (with the viscous part of the surface term)
     const int ek = ((__double2hiint(g.kappa) >> 20) & 0x7ff) - 1022;
     const int q1 = 56 - ex.g - ex.e.u, q2 = 59 - ex.t - ek;
-    const int qv = 52 - ex.g - ex.e.j - eD, qe = (q1 < q2 ? q1 : q2) - 6 - ex.e.j - eD;
+    const int qv = kFxQD - 6 - ex.g - ex.e.j - eD, qe = (q1 < q2 ? q1 : q2) - (64 - kFxQD) - ex.e.j - eD;
 #pragma unroll 1
     for (int c = 0; c < 4; ++c) {
       i64 p = 0, f = 0;

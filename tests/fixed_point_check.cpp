@@ -140,7 +140,9 @@ void check_conversions(int count, double* out) {
     const i64 c = (i64)ldexp(drand48() - 0.5, 63);
     {
       const L v = std::ldexp((L)X + std::ldexp((L)c, -32), -9);
-      if (std::fabs(v) > 65536) out[2] = std::max(out[2], (double)std::fabs(((L)fx_to2<32>(X, c, 9) - v) / v));
+      // 2^-32 units of the one's complement apart
+      const double err = (double)(std::fabs((L)fx_to2<32>(X, c, 9) - v) - std::ldexp((L)1, -41));
+      if (v != 0) out[2] = std::max(out[2], err / (double)std::fabs(v));
     }
   }
   if (fx_to(0, 9) != 0.0 || fx_to2<32>(0, 0, 9) != 0.0) out[1] = 1;
