@@ -338,7 +338,7 @@ static dg_status init_impl(const dg_mesh* mesh, const dg_params* prm, int device
        (!alloc((void**)&c->d_Uf, sizeof(double) * E * 6 * 5 * NN, "alloc face states") ||
         !alloc((void**)&c->d_gf, sizeof(double) * E * 6 * 12 * NN, "alloc face gradients") ||
         !alloc((void**)&c->d_lgb, sizeof(double) * (2 * NN + 5 * c->n), "alloc Gauss basis"))) ||
-      (prm->precision != DG_FP32OP && prm->nodes != DG_NODES_LG &&
+      (prm->precision != DG_FP32OP &&
        (!alloc((void**)&c->d_jx, sizeof(long long) * E * 10 * P, "alloc metrics (fixed point)") ||
         !alloc((void**)&c->d_ejx, sizeof(float4) * E, "alloc metric exponents"))) ||
       (prm->precision == DG_FP32OP &&

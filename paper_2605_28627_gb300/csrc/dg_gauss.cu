@@ -13,6 +13,7 @@
 // Gauss points of each face.  Both sides of a face see the same face values of
 // the polynomial, and its discrete metric identities keep a uniform flow
 // uniform.  FP64 only.
+#include "dg_face_fx.cuh"
 #include "dg_gauss.cuh"
 
 #include <cmath>
@@ -335,6 +336,21 @@ __device__ __forceinline__ void state_phi(const Q* q, int st, const Gas& g, R ph
   ph[3] = p * ir * gsel<R>(g.inv_R, g.f_inv_R);
 }
 
+}  // namespace dg
+#include "dg_gauss_fx.cuh"
+namespace dg {
+
+// Blocks per SM that the registers of the fixed-point kernels must allow: 32
+// warps and 64 registers for the volume kernel and for the lifting at N >= 5
+// (N = 7: lifting 1011 -> 898 us, volume 676 -> 486 us against 16 warps and 128
+// registers), 16 warps for the lifting below (N = 4: 223 us against 252).
+template <int N>
+constexpr int lift_lg_fx_min_blocks() {
+  return Shape<N>::THREADS <= 512 ? (N >= 5 ? 1024 : 512) / Shape<N>::THREADS : 1;
+}
+template <int N>
+constexpr int volume_lg_fx_min_blocks() { return Shape<N>::THREADS <= 512 ? 1024 / Shape<N>::THREADS : 1; }
+
 template <int N, int EPB, typename R = double>
 constexpr size_t lift_lg_smem() {
   constexpr int n = N + 1, P = n * n * n, NN = n * n;
@@ -347,12 +363,15 @@ constexpr size_t lift_lg_smem() {
 // face values Uf, the metric terms, face geometry, g and its face values gf).
 // MORTAR: a face whose neighbour entry is negative is a mortar side,
 // whose neighbour face state is mvirt[-1 - entry][5][NN] in its own point order.
+// state (block-shared [EPB], or null): only the elements whose entry is 2 are
+// worked on (those that the fixed-point body left).
 template <int N, int EPB, bool MORTAR = false, typename R = double>
-__global__ void __launch_bounds__(Shape<N, EPB>::THREADS)
-k_lift_lg(const double* __restrict__ U, const R* __restrict__ Uf, const R* __restrict__ metrics,
-          const R* __restrict__ facegeo, const int* __restrict__ elem_face, const int* __restrict__ elem_nbr,
-          const double* __restrict__ tab, R* __restrict__ grad, R* __restrict__ gf, int E, int F, Gas g,
-          const double* __restrict__ mvirt, int n_mortar) {
+__device__ __forceinline__ void lift_lg_body(const double* __restrict__ U, const R* __restrict__ Uf,
+                                             const R* __restrict__ metrics, const R* __restrict__ facegeo,
+                                             const int* __restrict__ elem_face, const int* __restrict__ elem_nbr,
+                                             const double* __restrict__ tab, R* __restrict__ grad, R* __restrict__ gf,
+                                             int E, int F, const Gas& g, const double* __restrict__ mvirt, int n_mortar,
+                                             const int* state = nullptr) {
   using S = Shape<N, EPB>;
   constexpr int n = S::n, P = S::P, NN = n * n, PER = 16 * P + 72 * NN;
   extern __shared__ __align__(16) unsigned char lift_lg_raw[];
@@ -360,7 +379,7 @@ k_lift_lg(const double* __restrict__ U, const R* __restrict__ Uf, const R* __res
   __shared__ R sDw[n * n], sT[4 * n];   // weak D; l(-1)/w, l(+1)/w, l(-1), l(+1)
   const int le = threadIdx.x / P, id = threadIdx.x - le * P;
   const int e = blockIdx.x * EPB + le;
-  const bool active = e < E;
+  const bool active = e < E && (state == nullptr || state[le] == 2);
   R* sphi = sm + le * PER;     // [4][P]
   R* sprod = sphi + 4 * P;     // [12][P]
   R* sS = sprod + 12 * P;      // [6][12][NN]: phi* (n_l sJ) with the outward normal
@@ -471,6 +490,32 @@ k_lift_lg(const double* __restrict__ U, const R* __restrict__ Uf, const R* __res
   }
 }
 
+template <int N, int EPB, bool MORTAR, typename R>
+__global__ void __launch_bounds__(Shape<N, EPB>::THREADS)
+k_lift_lg(const double* __restrict__ U, const R* __restrict__ Uf, const R* __restrict__ metrics,
+          const R* __restrict__ facegeo, const int* __restrict__ elem_face, const int* __restrict__ elem_nbr,
+          const double* __restrict__ tab, R* __restrict__ grad, R* __restrict__ gf, int E, int F, Gas g,
+          const double* __restrict__ mvirt, int n_mortar) {
+  lift_lg_body<N, EPB, MORTAR, R>(U, Uf, metrics, facegeo, elem_face, elem_nbr, tab, grad, gf, E, F, g, mvirt,
+                                  n_mortar);
+}
+// FP64 operator: fixed point, then FP64 for the elements out of its range.
+template <int N, int EPB, bool MORTAR>
+__global__ void __launch_bounds__(Shape<N, EPB>::THREADS, lift_lg_fx_min_blocks<N>())
+k_lift_lg_fx(const double* __restrict__ U, const double* __restrict__ Uf, const double* __restrict__ metrics,
+             const i64* __restrict__ jx, const float4* __restrict__ ejx, const double* __restrict__ facegeo,
+             const int* __restrict__ elem_face, const int* __restrict__ elem_nbr, const double* __restrict__ tab,
+             double* __restrict__ grad, double* __restrict__ gf, int E, int F, Gas g,
+             const double* __restrict__ mvirt, int n_mortar) {
+  __shared__ int s_state[EPB];
+  if (lift_lg_fx<N, EPB, MORTAR>(U, Uf, jx, ejx, facegeo, elem_face, elem_nbr, tab, grad, gf, E, F, g, mvirt, n_mortar,
+                                 s_state)) {
+    __syncthreads();
+    lift_lg_body<N, EPB, MORTAR, double>(U, Uf, metrics, facegeo, elem_face, elem_nbr, tab, grad, gf, E, F, g, mvirt,
+                                         n_mortar, s_state);
+  }
+}
+
 // Surface flux at the Gauss face points of each master face, from both sides'
 // face values of the state and of the lifted gradients.
 // FVSKIP: faces with an FV sub-cell element on either side are left to the FV
@@ -511,6 +556,14 @@ k_face_lg(const R* __restrict__ Uf, const R* __restrict__ gf, const FaceInfo* __
   }
   const R* gM = gf + ((size_t)eM * 6 + fM) * 12 * NN + pq;
   const R* gS = gf + ((size_t)eS * 6 + fS) * 12 * NN + pq2;
+  if constexpr (sizeof(R) == 8) {
+    if (g.surf_flux == DG_FLUX_LLF) {
+      const double* fg = facegeo + (size_t)f * 4 * NN + pq;
+      const double nv[3] = {fg[0], fg[NN], fg[2 * NN]};
+      face_point_fx(dL, dR, gM, gS, NN, nv, fg[3 * NN], g, fstar + (size_t)f * 5 * NN + pq, NN);
+      return;
+    }
+  }
 #pragma unroll
   for (int r = 0; r < 12; ++r) {
     gL[r] = gM[r * NN];
@@ -534,11 +587,13 @@ constexpr size_t volume_lg_smem() {
 // R: the operator type (metric terms, gradients, surface fluxes and the
 // arithmetic of the residual); the state, 1/J of the final scaling and the RK
 // update are FP64 (metrics64: the FP64 metric array, row 9 = 1/J).
+// state as in lift_lg_body.
 template <int N, int EPB, bool LIST, typename R = double>
-__global__ void __launch_bounds__(Shape<N, EPB>::THREADS)
-k_volume_lg(StageArgs a, const R* __restrict__ metrics, const double* __restrict__ metrics64,
-            const R* __restrict__ grad, const R* __restrict__ fstar, const int* __restrict__ elem_face,
-            const double* __restrict__ mms, const double* __restrict__ tab, int E, Gas g) {
+__device__ __forceinline__ void volume_lg_body(const StageArgs& a, const R* __restrict__ metrics,
+                                               const double* __restrict__ metrics64, const R* __restrict__ grad,
+                                               const R* __restrict__ fstar, const int* __restrict__ elem_face,
+                                               const double* __restrict__ mms, const double* __restrict__ tab, int E,
+                                               const Gas& g, const int* state = nullptr) {
   using S = Shape<N, EPB>;
   constexpr int n = S::n, P = S::P, NN = n * n, PER = 15 * P + 30 * NN;
   extern __shared__ __align__(16) unsigned char volume_lg_raw[];
@@ -554,7 +609,7 @@ k_volume_lg(StageArgs a, const R* __restrict__ metrics, const double* __restrict
       if (e >= E) return;   // the whole block, before any barrier
     }
   }
-  const bool active = e < E;
+  const bool active = e < E && (state == nullptr || state[le] == 2);
   R* sF = sm + le * PER;   // [3][5][P] contravariant fluxes
   R* sFs = sF + 15 * P;    // [6][5][NN] outward surface fluxes
   for (int t = threadIdx.x; t < n * n; t += blockDim.x) sDw[t] = to_op<R>(tab[GaussTab::Dw(n) + t]);
@@ -661,6 +716,26 @@ k_volume_lg(StageArgs a, const R* __restrict__ metrics, const double* __restrict
   }
 }
 
+template <int N, int EPB, bool LIST, typename R>
+__global__ void __launch_bounds__(Shape<N, EPB>::THREADS)
+k_volume_lg(StageArgs a, const R* __restrict__ metrics, const double* __restrict__ metrics64,
+            const R* __restrict__ grad, const R* __restrict__ fstar, const int* __restrict__ elem_face,
+            const double* __restrict__ mms, const double* __restrict__ tab, int E, Gas g) {
+  volume_lg_body<N, EPB, LIST, R>(a, metrics, metrics64, grad, fstar, elem_face, mms, tab, E, g);
+}
+template <int N, int EPB, bool LIST>
+__global__ void __launch_bounds__(Shape<N, EPB>::THREADS, volume_lg_fx_min_blocks<N>())
+k_volume_lg_fx(StageArgs a, const double* __restrict__ metrics, const i64* __restrict__ jx,
+               const float4* __restrict__ ejx, const double* __restrict__ grad, const double* __restrict__ fstar,
+               const int* __restrict__ elem_face, const double* __restrict__ mms, const double* __restrict__ tab, int E,
+               Gas g) {
+  __shared__ int s_state[EPB];
+  if (volume_lg_fx<N, EPB, LIST>(a, metrics, jx, ejx, grad, fstar, elem_face, mms, tab, E, g, s_state)) {
+    __syncthreads();
+    volume_lg_body<N, EPB, LIST, double>(a, metrics, metrics, grad, fstar, elem_face, mms, tab, E, g, s_state);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Launchers
 
@@ -685,8 +760,32 @@ static cudaError_t setup_lg_NR() {
 }
 
 template <int N>
+constexpr size_t lift_lg_f64_smem() {
+  constexpr int EPB = Shape<N>::EPB;
+  return lift_lg_fx_smem<N, EPB>() > lift_lg_smem<N, EPB>() ? lift_lg_fx_smem<N, EPB>() : lift_lg_smem<N, EPB>();
+}
+template <int N>
+constexpr size_t volume_lg_f64_smem() {
+  constexpr int EPB = Shape<N>::EPB;
+  return volume_lg_fx_smem<N, EPB>() > volume_lg_smem<N, EPB>() ? volume_lg_fx_smem<N, EPB>() : volume_lg_smem<N, EPB>();
+}
+
+template <int N>
+static cudaError_t setup_lg_fx_N() {
+  using S = Shape<N>;
+  const int ls = (int)lift_lg_f64_smem<N>(), vs = (int)volume_lg_f64_smem<N>();
+  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(k_lift_lg_fx<N, S::EPB, false>, at, ls);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lift_lg_fx<N, S::EPB, true>, at, ls);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_volume_lg_fx<N, S::EPB, false>, at, vs);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_volume_lg_fx<N, S::EPB, true>, at, vs);
+  return e;
+}
+
+template <int N>
 static cudaError_t setup_lg_N() {
   cudaError_t e = setup_lg_NR<N, double>();
+  if (e == cudaSuccess) e = setup_lg_fx_N<N>();
   if (e == cudaSuccess) e = setup_lg_NR<N, float>();
   constexpr int P = (N + 1) * (N + 1) * (N + 1);
   if (e == cudaSuccess)
@@ -731,6 +830,21 @@ static cudaError_t lift_lg_NR(const Ctx& c, const double* U, cudaStream_t s) {
   if (c.M > 0) {   // the mortar sides' neighbour face states first
     err = launch_mortar_lift(c, U, s);
     if (err != cudaSuccess) return err;
+  }
+  if constexpr (sizeof(R) == 8) {
+    if (c.d_jx) {   // absent in an FP32-operator context, whose diagnostics lift in FP64
+      if (c.M > 0)
+        k_lift_lg_fx<N, S::EPB, true><<<blocks, S::THREADS, lift_lg_f64_smem<N>(), s>>>(
+            U, Uf, c.d_metrics, c.d_jx, c.d_ejx, c.d_facegeo, c.d_elem_face, c.d_elem_nbr, c.d_lgb, (double*)c.d_grad,
+            gf, c.E, c.nfaces, c.gas, c.d_mortar_virt, c.M);
+      else
+        k_lift_lg_fx<N, S::EPB, false><<<blocks, S::THREADS, lift_lg_f64_smem<N>(), s>>>(
+            U, Uf, c.d_metrics, c.d_jx, c.d_ejx, c.d_facegeo, c.d_elem_face, c.d_elem_nbr, c.d_lgb, (double*)c.d_grad,
+            gf, c.E, c.nfaces, c.gas, nullptr, 0);
+      return cudaGetLastError();
+    }
+  }
+  if (c.M > 0) {
     k_lift_lg<N, S::EPB, true, R><<<blocks, S::THREADS, lift_lg_smem<N, S::EPB, R>(), s>>>(
         U, Uf, metrics_of<R>(c), facegeo_of<R>(c), c.d_elem_face, c.d_elem_nbr, c.d_lgb, (R*)c.d_grad, gf, c.E,
         c.nfaces, c.gas, c.d_mortar_virt, c.M);
@@ -777,6 +891,17 @@ static cudaError_t volume_lg_NR(const Ctx& c, const StageArgs& a0, cudaStream_t 
   StageArgs a = a0;
   a.nfaces = c.nfaces;
   const int blocks = (c.E + S::EPB - 1) / S::EPB;
+  if constexpr (sizeof(R) == 8) {
+    if (a.list != nullptr)
+      k_volume_lg_fx<N, S::EPB, true><<<blocks, S::THREADS, volume_lg_f64_smem<N>(), s>>>(
+          a, c.d_metrics, c.d_jx, c.d_ejx, (const double*)c.d_grad, (const double*)c.d_fstar, c.d_elem_face, c.d_mms,
+          c.d_lgb, c.E, c.gas);
+    else
+      k_volume_lg_fx<N, S::EPB, false><<<blocks, S::THREADS, volume_lg_f64_smem<N>(), s>>>(
+          a, c.d_metrics, c.d_jx, c.d_ejx, (const double*)c.d_grad, (const double*)c.d_fstar, c.d_elem_face, c.d_mms,
+          c.d_lgb, c.E, c.gas);
+    return cudaGetLastError();
+  }
   if (a.list != nullptr)
     k_volume_lg<N, S::EPB, true, R><<<blocks, S::THREADS, volume_lg_smem<N, S::EPB, R>(), s>>>(
         a, metrics_of<R>(c), c.d_metrics, (const R*)c.d_grad, (const R*)c.d_fstar, c.d_elem_face, c.d_mms, c.d_lgb,

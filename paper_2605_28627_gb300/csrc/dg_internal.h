@@ -124,7 +124,7 @@ struct Ctx {
   double* d_mms = nullptr;       // [E][2][P] sin, cos of pi (x + y + z); manufactured source only
   double* d_facegeo = nullptr;   // [F][4][NN]: unit normal (3), surface element
   float* d_metrics_f = nullptr;  // FP32 copies for the FP32-operator path
-  long long* d_jx = nullptr;     // [E][10][P] metric terms and 1/J in fixed point (FP64 operator on LGL nodes)
+  long long* d_jx = nullptr;     // [E][10][P] metric terms and 1/J in fixed point (FP64 operator)
   float4* d_ejx = nullptr;       // [E] their exponents (k_fx_metrics)
   float* d_facegeo_f = nullptr;
   FaceInfo* d_faces = nullptr;   // [F]: the conforming faces, then the mortars' small and big sides

@@ -93,8 +93,9 @@ cudaError_t setup_volume(int N) {
 }
 
 cudaError_t launch_fx_metrics(const Ctx& c, cudaStream_t s) {
+  const double* fg = c.prm.nodes == DG_NODES_LG ? c.d_facegeo : nullptr;
   switch (c.N) {
-#define DG_FXM(n) case n: k_fx_metrics<n><<<c.E, 256, 0, s>>>(c.d_metrics, c.d_jx, c.d_ejx); break;
+#define DG_FXM(n) case n: k_fx_metrics<n><<<c.E, 256, 0, s>>>(c.d_metrics, c.d_jx, c.d_ejx, fg, c.d_elem_face, c.nfaces); break;
     DG_FXM(1) DG_FXM(2) DG_FXM(3) DG_FXM(4) DG_FXM(5) DG_FXM(6) DG_FXM(7) DG_FXM(8) DG_FXM(9)
 #undef DG_FXM
     default: return cudaErrorInvalidValue;

@@ -93,3 +93,17 @@ def test_non_finite_state_stays_local():
         Rv = s.time_derivative(V)
         assert not bool(torch.isfinite(Rv[e]).all())
         assert torch.equal(Rv[far], R[far])
+
+
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 7, 8])
+@pytest.mark.parametrize("scale", [1.0, 1e30])
+def test_gauss_nodes(orc, N, scale):
+    """The weak form on Gauss nodes in range, and with density and pressure
+    scaled out of the fixed-point range (2^90), which all runs in FP64.  The
+    pressure's mean is 10 times its variation (see the bar above)."""
+    import paper_2605_28627_gb300 as dg
+    mesh = box_mesh(SIZE[N], min(N, 4), deform="sinprod", rotate_seed=450 + N)
+    o, s = orc.Oracle(mesh, N, mu=0.01 * scale, nodes=1), dg.Solver(mesh, N, mu=0.01 * scale, nodes=dg.NODES_LG)
+    U = random_state(mesh.n_elems, N, seed=550 + N, rho=(0.95, 1.05), vel=0.2, p=(0.95, 1.05)) * scale
+    err = _err(s.time_derivative(_cuda(U)).cpu().numpy(), o.time_derivative(U))
+    assert (err < 1e-11).all(), err
