@@ -17,7 +17,7 @@
 #include <algorithm>
 #include <vector>
 
-#include "dg_adjoint_fn.cuh"
+#include "dg_adjoint_fx.cuh"
 #include "dg_gauss.cuh"
 #include "dg_mortar.cuh"
 #include "dg_stage.cuh"
@@ -47,13 +47,20 @@ constexpr int kAdjVolWords = 27;
 template <int N>
 __global__ void __launch_bounds__(Shape<N>::THREADS, Shape<N>::THREADS <= 256 ? 2 : 1)
 k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const double* __restrict__ metrics,
-             const double* __restrict__ grad, const int* __restrict__ elem_face, const double* __restrict__ Dg,
-             int E, Gas g, double inv_w0, AdjBufs b) {
+             const i64* __restrict__ jx, const float4* __restrict__ ejx, const double* __restrict__ grad,
+             const int* __restrict__ elem_face, const double* __restrict__ Dg, int E, Gas g, double inv_w0, AdjBufs b) {
   using S = Shape<N>;
   constexpr int n = S::n, P = S::P, NN = S::NN, EPB = S::EPB;
   constexpr int FULL = (n - 1) / 2;       // shifts with a pair for every node
   constexpr bool HALF = (n % 2) == 0;     // the shift n/2, half as many pairs
-  extern __shared__ double adj_smem[];
+  extern __shared__ __align__(16) double adj_smem[];
+  // the two-point terms in fixed point; elements out of its range (state 2)
+  // are summed in FP64 below
+  __shared__ int s_state[EPB];
+  double pr[5] = {0, 0, 0, 0, 0};   // own primitive adjoint (rho, u, v, w, p)
+  const bool some64 = adj_pairs_fx<N>(U, lam, metrics, jx, ejx, Dg, E, g, reinterpret_cast<unsigned char*>(adj_smem),
+                                      s_state, pr);
+  __syncthreads();
   double* sD = adj_smem;                                   // [n*n]
   double* sD2 = sD + n * n;                                // [n*n] 2 D (exact)
   double* base = adj_smem + ((2 * n * n + 1) & ~1);
@@ -98,10 +105,10 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
   __syncthreads();
   const int i = id % n, j = (id / n) % n, k = id / NN;
   const int ijk[3] = {i, j, k};
-  double pr[5] = {0, 0, 0, 0, 0};   // own primitive adjoint (rho, u, v, w, p)
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int r = ijk[d];
+  const bool act64 = active && s_state[le] == 2;
+#pragma unroll 1
+  for (int d = 0; d < (some64 ? 3 : 0); ++d) {
+    const int r = d == 0 ? i : (d == 1 ? j : k);
     const int stride = d == 0 ? 1 : (d == 1 ? n : NN);
     const int line0 = id - r * stride;
 #pragma unroll 1
@@ -109,11 +116,11 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
       const int m = r + s < n ? r + s : r + s - n;
       const int mid = line0 + m * stride;
       double pm[5] = {0, 0, 0, 0, 0};
-      if (active) {
+      if (act64) {
         NodePrim<double> ot{sPr(0, mid), sPr(1, mid), sPr(2, mid), sPr(3, mid), sPr(4, mid), sPr(5, mid)};
-        const double nx = 0.5 * (Ja[d * 3] + sJa(d * 3, mid));
-        const double ny = 0.5 * (Ja[d * 3 + 1] + sJa(d * 3 + 1, mid));
-        const double nz = 0.5 * (Ja[d * 3 + 2] + sJa(d * 3 + 2, mid));
+        const double nx = 0.5 * (sJa(d * 3, id) + sJa(d * 3, mid));
+        const double ny = 0.5 * (sJa(d * 3 + 1, id) + sJa(d * 3 + 1, mid));
+        const double nz = 0.5 * (sJa(d * 3 + 2, id) + sJa(d * 3 + 2, mid));
         const double Drm2 = sD2[r * n + m], Dmr2 = sD2[m * n + r];
         double wb[5];
 #pragma unroll
@@ -124,7 +131,7 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
         for (int c = 0; c < 5; ++c) sX(c, mid) = pm[c];
       }
       __syncthreads();
-      if (active) {
+      if (act64) {
 #pragma unroll
         for (int c = 0; c < 5; ++c) pr[c] += sX(c, id);
       }
@@ -137,7 +144,7 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
       constexpr int H = n / 2;
       const int t = threadIdx.x;
       const int le2 = t / (P / 2), w2 = t - le2 * (P / 2);
-      if (t < EPB * (P / 2) && blockIdx.x * EPB + le2 < E) {
+      if (t < EPB * (P / 2) && s_state[le2] == 2) {
         const int hi = w2 / stride;
         const int ra = hi % H, rb = ra + H;
         const int ia = w2 - hi * stride + stride * (ra + n * (hi / H));   // node with r < n/2
@@ -164,7 +171,7 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
         }
       }
       __syncthreads();
-      if (active) {
+      if (act64) {
 #pragma unroll
         for (int c = 0; c < 5; ++c) pr[c] += sX(c, id);
       }
@@ -1083,7 +1090,7 @@ static cudaError_t vjp_N(const Ctx& c, const double* U, const double* lam, doubl
   const int blocks = (c.E + S::EPB - 1) / S::EPB;
   const double inv_w0 = 1.0 / c.w[0];
   const double* grad = (const double*)c.d_grad;
-  k_adj_volume<N><<<blocks, S::THREADS, adj_volume_smem<N>(), s>>>(U, lam, c.d_metrics, grad, c.d_elem_face, c.d_D,
+  k_adj_volume<N><<<blocks, S::THREADS, adj_volume_smem<N>(), s>>>(U, lam, c.d_metrics, c.d_jx, c.d_ejx, grad, c.d_elem_face, c.d_D,
                                                                    c.E, c.gas, inv_w0, b);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;

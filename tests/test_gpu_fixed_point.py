@@ -95,6 +95,30 @@ def test_non_finite_state_stays_local():
         assert torch.equal(Rv[far], R[far])
 
 
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 7])
+@pytest.mark.parametrize("kind,scale", [("means by long series", 1.0), ("means by logarithm", 1.0),
+                                        ("edge of the range", 1e3), ("FP64 elements", 1.0), ("at rest", 1.0),
+                                        ("Mach 17", 1e-3), ("low Mach", 1e4)])
+def test_vjp(orc, N, kind, scale):
+    """<(dR/dU)^T v, w> against <v, (dR/dU) w> of the oracle's tangent-linear,
+    as in the adjoint's dot-product tests (bar 1e-11 of the terms' sum), with
+    the components of v of different sizes (mass scale^2, momentum scale,
+    energy 1) and every fifth element's v zero."""
+    import paper_2605_28627_gb300 as dg
+    mesh = box_mesh(2, min(N, 4), deform="sinprod", rotate_seed=440 + N)
+    o, s = orc.Oracle(mesh, N, mu=0.02), dg.Solver(mesh, N, mu=0.02)
+    U = random_state(mesh.n_elems, N, seed=540 + N, **STATES[kind])
+    rng = np.random.default_rng(640 + N)
+    w, v = rng.normal(size=U.shape), rng.normal(size=U.shape)
+    v[:, 0] *= scale ** 2
+    v[:, 1:4] *= scale
+    v[::5] = 0.0
+    _, Jw = o.time_derivative_tl(U, w, 0.0)
+    JTv = s.time_derivative_vjp(_cuda(U), _cuda(v)).cpu().numpy()
+    lhs, rhs = float((JTv * w).sum()), float((v * Jw).sum())
+    assert abs(lhs - rhs) <= 1e-11 * float(np.abs(JTv * w).sum()), (lhs, rhs)
+
+
 @pytest.mark.parametrize("N", [1, 2, 3, 4, 7, 8])
 @pytest.mark.parametrize("scale", [1.0, 1e30])
 def test_gauss_nodes(orc, N, scale):
