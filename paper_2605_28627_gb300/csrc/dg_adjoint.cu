@@ -36,6 +36,26 @@ struct AdjBufs {
   int F;             // face slots (conforming faces, then the mortars' slots)
 };
 
+// Sum of x over the T threads of a block, in a fixed order: 16 threads sum every
+// 16th value, one sums theirs (the block need not be a whole number of warps).
+// One thread alone would be a chain of T additions at some 70 cycles each.
+// Returned to thread 0.
+template <int T>
+__device__ __forceinline__ double block_sum(double* buf, double x, int t) {
+  constexpr int L = T < 16 ? T : 16;
+  buf[t] = x;
+  __syncthreads();
+  double s = 0.0;
+  if (t < L) {
+    for (int m = t; m < T; m += L) s += buf[m];
+    buf[t] = s;
+  }
+  __syncthreads();
+  if (t == 0)
+    for (int m = 1; m < L; ++m) s += buf[m];
+  return s;
+}
+
 // ---------------------------------------------------------------------------
 // Words per node of the volume adjoint's element tile: rho, u, v, w, beta,
 // beta/p, 1/(2p) and |u|^2 (8), metric terms (9), lamV (5), the partner's
@@ -90,12 +110,12 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
     iJ = mt[9 * P];
 #pragma unroll
     for (int c = 0; c < 5; ++c) { lv[c] = -lam[((size_t)e * 5 + c) * P + id] * iJ; sL(c, id) = lv[c]; }
-    const double ir = 1.0 / q[0];
+    const double ir = adj_rcp(q[0]);
     me.rho = q[0]; me.u = q[1] * ir; me.v = q[2] * ir; me.w = q[3] * ir;
     me.p = g.gm1 * (q[4] - 0.5 * (q[1] * me.u + q[2] * me.v + q[3] * me.w));
-    me.beta = 0.5 * q[0] / me.p;
-    sPr(0, id) = me.rho; sPr(1, id) = me.u; sPr(2, id) = me.v; sPr(3, id) = me.w;
     const double ip = adj_rcp(me.p);
+    me.beta = 0.5 * q[0] * ip;
+    sPr(0, id) = me.rho; sPr(1, id) = me.u; sPr(2, id) = me.v; sPr(3, id) = me.w;
     hip_me = 0.5 * ip;
     bip_me = me.beta * ip;
     sPr(4, id) = bip_me; sPr(5, id) = me.beta;
@@ -185,11 +205,12 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
     const double* gg = grad + (size_t)e * 12 * P + id;
 #pragma unroll
     for (int r2 = 0; r2 < 12; ++r2) gr[r2] = gg[r2 * P];
-    double gb[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    double gb[12];
     double ub[3] = {0, 0, 0};
+    ViscVjp vis{};
     // viscosity law: mu = mu_ref s(T), T = p / (rho R)
-    const double Tn = me.p / me.rho * g.inv_R;
-    double sv, dsv, vr = 0.0;
+    const double ir = adj_rcp(me.rho), Tn = me.p * ir * g.inv_R;
+    double sv, dsv;
     visc_factor_d(g, Tn, sv, dsv);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -209,19 +230,19 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
 #pragma unroll
         for (int c = 0; c < 4; ++c) fb[c] += vs * lv[1 + c];
       }
-      vr += visc_flux_vjp(gr, me.u, me.v, me.w, g.mu * sv, g.kappa, Ja[d * 3], Ja[d * 3 + 1], Ja[d * 3 + 2], fb,
-                          gb, ub);
+      visc_vjp_add(vis, me.u, me.v, me.w, Ja[d * 3], Ja[d * 3 + 1], Ja[d * 3 + 2], fb);
     }
+    const double vr = visc_vjp_end(vis, gr, g.mu * sv, g.kappa, gb, ub);
     mub += sv * vr;
     pr[1] += ub[0]; pr[2] += ub[1]; pr[3] += ub[2];
     if (dsv != 0.0) {   // through T = p / (rho R)
       const double Tb = g.mu * dsv * vr;
-      pr[4] += Tb * g.inv_R / me.rho;
-      pr[0] -= Tb * Tn / me.rho;
+      pr[4] += Tb * g.inv_R * ir;
+      pr[0] -= Tb * Tn * ir;
     }
     double qb[5] = {0, 0, 0, 0, 0};
     const double uu[3] = {pr[1], pr[2], pr[3]};
-    prim_vjp(q, pr[0], uu, pr[4], g.gm1, qb);
+    prim_vjp(ir, me.u, me.v, me.w, pr[0], uu, pr[4], g.gm1, qb);
 #pragma unroll
     for (int c = 0; c < 5; ++c) b.qbar[((size_t)e * 5 + c) * P + id] = qb[c];
 #pragma unroll
@@ -248,22 +269,15 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
       }
     }
   }
-  // block partial of d/dmu (the block need not be a whole number of warps,
-  // so the partials go through shared memory, summed by one thread in order)
-  smu[threadIdx.x] = mub;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int t = 0; t < S::THREADS; ++t) s += smu[t];
-    b.mupart[blockIdx.x] = s;
-  }
+  const double mu = block_sum<S::THREADS>(smu, mub, threadIdx.x);   // block partial of d/dmu
+  if (threadIdx.x == 0) b.mupart[blockIdx.x] = mu;
 }
 
 // ---------------------------------------------------------------------------
 // Face VJP at one face point: from the adjoint Fb of F* (F* = (f* - f_v avg) sJ)
-// to the conserved (5) and gradient (12) adjoints of the two sides, added to
-// qbL, gbL (side L, whose outward normal (nx, ny, nz) is) and qbR, gbR; returns
-// the d/dmu contribution.
+// to the conserved (5) and gradient (12) adjoints of the two sides: added to
+// qbL (side L, whose outward normal (nx, ny, nz) is) and qbR, set in gbL and gbR;
+// returns the d/dmu contribution.
 __device__ __forceinline__ double face_vjp_point(const double qL[5], const double qR[5], const double gL[12],
                                                  const double gR[12], double nx, double ny, double nz, double sJ,
                                                  const double Fb[5], const Gas& g, double qbL[5], double qbR[5],
@@ -271,43 +285,47 @@ __device__ __forceinline__ double face_vjp_point(const double qL[5], const doubl
   double fa_b[5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) fa_b[c] = Fb[c] * sJ;
+  const double irL = adj_rcp(qL[0]), irR = adj_rcp(qR[0]);
+  const double uL[3] = {qL[1] * irL, qL[2] * irL, qL[3] * irL}, uR[3] = {qR[1] * irR, qR[2] * irR, qR[3] * irR};
+  const double pL = g.gm1 * (qL[4] - 0.5 * (qL[1] * uL[0] + qL[2] * uL[1] + qL[3] * uL[2]));
+  const double pR = g.gm1 * (qR[4] - 0.5 * (qR[1] * uR[0] + qR[2] * uR[1] + qR[3] * uR[2]));
+  // primitive adjoints of both sides, to the conserved ones once at the end
+  double rbL = 0, pbL = 0, ubL[3] = {0, 0, 0}, rbR = 0, pbR = 0, ubR[3] = {0, 0, 0};
   if (g.surf_flux == DG_FLUX_EC) {
-    const double irL = 1.0 / qL[0], irR = 1.0 / qR[0];
-    NodePrim<double> A{qL[0], qL[1] * irL, qL[2] * irL, qL[3] * irL, 0, 0};
-    A.p = g.gm1 * (qL[4] - 0.5 * (qL[1] * A.u + qL[2] * A.v + qL[3] * A.w));
-    A.beta = 0.5 * qL[0] / A.p;
-    NodePrim<double> B{qR[0], qR[1] * irR, qR[2] * irR, qR[3] * irR, 0, 0};
-    B.p = g.gm1 * (qR[4] - 0.5 * (qR[1] * B.u + qR[2] * B.v + qR[3] * B.w));
-    B.beta = 0.5 * qR[0] / B.p;
+    const NodePrim<double> A{qL[0], uL[0], uL[1], uL[2], pL, 0.5 * qL[0] * adj_rcp(pL)};
+    const NodePrim<double> B{qR[0], uR[0], uR[1], uR[2], pR, 0.5 * qR[0] * adj_rcp(pR)};
     double pa[5] = {0, 0, 0, 0, 0}, pb[5] = {0, 0, 0, 0, 0};
     ec_flux_vjp(A, B, nx, ny, nz, g.inv_gm1, fa_b, pa, pb);
-    const double ua[3] = {pa[1], pa[2], pa[3]}, ubv[3] = {pb[1], pb[2], pb[3]};
-    prim_vjp(qL, pa[0], ua, pa[4], g.gm1, qbL);
-    prim_vjp(qR, pb[0], ubv, pb[4], g.gm1, qbR);
+    rbL = pa[0]; pbL = pa[4];
+    rbR = pb[0]; pbR = pb[4];
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+      ubL[l] = pa[1 + l];
+      ubR[l] = pb[1 + l];
+    }
   } else if (g.surf_flux == DG_FLUX_ROE) {
     roe_vjp(qL, qR, nx, ny, nz, g.gamma, g.gm1, fa_b, qbL, qbR);
   } else {
-    llf_vjp(qL, qR, nx, ny, nz, g.gamma, g.gm1, fa_b, qbL, qbR);
+    llf_vjp(qL, qR, irL, uL, pL, irR, uR, pR, nx, ny, nz, g.gamma, fa_b, qbL, qbR, rbL, ubL, pbL, rbR, ubR, pbR);
   }
   // viscous part: F* includes -1/2 (f_v(L) + f_v(R)) . n sJ
   double fvb[4];
 #pragma unroll
-  for (int c = 0; c < 4; ++c) fvb[c] = -0.5 * Fb[1 + c] * sJ;
-  double ubL[3] = {0, 0, 0}, ubR[3] = {0, 0, 0};
-  const double irL = 1.0 / qL[0], irR = 1.0 / qR[0];
+  for (int c = 0; c < 4; ++c) fvb[c] = -0.5 * fa_b[1 + c];
   // viscosity law on each side: mu = mu_ref s(T), T = p / (rho R)
-  const double uL = qL[1] * irL, vL = qL[2] * irL, wL = qL[3] * irL;
-  const double uR = qR[1] * irR, vR = qR[2] * irR, wR = qR[3] * irR;
-  const double TL = g.gm1 * (qL[4] - 0.5 * (qL[1] * uL + qL[2] * vL + qL[3] * wL)) * irL * g.inv_R;
-  const double TR = g.gm1 * (qR[4] - 0.5 * (qR[1] * uR + qR[2] * vR + qR[3] * wR)) * irR * g.inv_R;
+  const double TL = pL * irL * g.inv_R, TR = pR * irR * g.inv_R;
   double sL, dsL, sR, dsR;
   visc_factor_d(g, TL, sL, dsL);
   visc_factor_d(g, TR, sR, dsR);
-  const double vrL = visc_flux_vjp(gL, uL, vL, wL, g.mu * sL, g.kappa, nx, ny, nz, fvb, gbL, ubL);
-  const double vrR = visc_flux_vjp(gR, uR, vR, wR, g.mu * sR, g.kappa, nx, ny, nz, fvb, gbR, ubR);
-  const double TbL = g.mu * dsL * vrL, TbR = g.mu * dsR * vrR;   // through T = p / (rho R)
-  prim_vjp(qL, -TbL * TL * irL, ubL, TbL * g.inv_R * irL, g.gm1, qbL);
-  prim_vjp(qR, -TbR * TR * irR, ubR, TbR * g.inv_R * irR, g.gm1, qbR);
+  ViscVjp vis{};
+  visc_vjp_add(vis, uL[0], uL[1], uL[2], nx, ny, nz, fvb);
+  const double vrL = visc_vjp_end(vis, gL, g.mu * sL, g.kappa, gbL, ubL);
+  vis = ViscVjp{};
+  visc_vjp_add(vis, uR[0], uR[1], uR[2], nx, ny, nz, fvb);
+  const double vrR = visc_vjp_end(vis, gR, g.mu * sR, g.kappa, gbR, ubR);
+  const double TbL = g.mu * dsL * vrL * irL, TbR = g.mu * dsR * vrR * irR;   // through T = p / (rho R)
+  prim_vjp(irL, uL[0], uL[1], uL[2], rbL - TbL * TL, ubL, fma(TbL, g.inv_R, pbL), g.gm1, qbL);
+  prim_vjp(irR, uR[0], uR[1], uR[2], rbR - TbR * TR, ubR, fma(TbR, g.inv_R, pbR), g.gm1, qbR);
   return sL * vrL + sR * vrR;
 }
 
@@ -350,8 +368,6 @@ k_adj_face(const double* __restrict__ U, const double* __restrict__ grad, const 
     for (int r = 0; r < 12; ++r) {
       gL[r] = gM[r * sg];
       gR[r] = gS[r * sg];
-      gbL[r] = 0.0;
-      gbR[r] = 0.0;
     }
     double qbL[5] = {0, 0, 0, 0, 0}, qbR[5] = {0, 0, 0, 0, 0};
     mub = face_vjp_point(qL, qR, gL, gR, fg[0], fg[NN], fg[2 * NN], fg[3 * NN], Fb, g, qbL, qbR, gbL, gbR);
@@ -450,8 +466,6 @@ k_adj_mortar_face(const double* __restrict__ U, const double* __restrict__ grad,
   for (int x = 0; x < 12; ++x) gL[x] = gs[x * sg];
   const double* fg = facegeo + (size_t)slot * 4 * NN + o;
   double qbL[5] = {0, 0, 0, 0, 0}, qbR[5] = {0, 0, 0, 0, 0}, gbL[12], gbR[12];
-#pragma unroll
-  for (int x = 0; x < 12; ++x) { gbL[x] = 0.0; gbR[x] = 0.0; }
   double mub = face_vjp_point(qL, qR, gL, qR + 5, fg[0], fg[NN], fg[2 * NN], fg[3 * NN], Fb, g, qbL, qbR, gbL, gbR);
   double* os = b.face + ((size_t)slot * 2 + 0) * 17 * NN + o;
 #pragma unroll
@@ -471,15 +485,9 @@ k_adj_mortar_face(const double* __restrict__ U, const double* __restrict__ grad,
     const int f = ox / NN, ij = ox - f * NN;
     b.face[((size_t)slotB * 2 + 0) * 17 * NN + (size_t)f * NN + ij] = mortar_proj2<n, 17>(sI, sS, f, ij % n, ij / n);
   }
-  // d/dmu: the block's partial, summed in a fixed order
-  __shared__ double smu[MortarShape<N>::THREADS];
-  smu[t] = mub;
-  __syncthreads();
-  if (t == 0) {
-    double acc = 0.0;
-    for (int x = 0; x < T; ++x) acc += smu[x];
-    b.mupart[mu_offset + m] = acc;
-  }
+  __shared__ double smu[T];
+  const double mu = block_sum<T>(smu, mub, t);   // block partial of d/dmu
+  if (t == 0) b.mupart[mu_offset + m] = mu;
 }
 
 // A3': the mortar sides' terms of the lifting transpose.  Forward: the face
@@ -691,7 +699,7 @@ k_adj_lift(const double* __restrict__ U, const double* __restrict__ metrics, con
   double q[5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) q[c] = U[((size_t)e * 5 + c) * P + id];
-  const double ir = 1.0 / q[0];
+  const double ir = adj_rcp(q[0]);
   const double u = q[1] * ir, v = q[2] * ir, w = q[3] * ir;
   const double p = g.gm1 * (q[4] - 0.5 * (q[1] * u + q[2] * v + q[3] * w));
   const double T = p * ir * g.inv_R;
@@ -699,7 +707,7 @@ k_adj_lift(const double* __restrict__ U, const double* __restrict__ metrics, con
   double qb[5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) qb[c] = b.qbar[((size_t)e * 5 + c) * P + id];
-  prim_vjp(q, -phib[3] * T * ir, ub, phib[3] * ir * g.inv_R, g.gm1, qb);
+  prim_vjp(ir, u, v, w, -phib[3] * T * ir, ub, phib[3] * ir * g.inv_R, g.gm1, qb);
 #pragma unroll
   for (int c = 0; c < 5; ++c) out[((size_t)e * 5 + c) * P + id] = qb[c];
 }
@@ -757,13 +765,14 @@ k_adjlg_volume(const double* __restrict__ U, const double* __restrict__ lam, con
     for (int r = 0; r < 12; ++r) gr[r] = grad[((size_t)e * 12 + r) * P + id];
 #pragma unroll
     for (int r = 0; r < 9; ++r) Ja[r] = metrics[((size_t)e * 10 + r) * P + id];
-    const double ir = 1.0 / q[0];
+    const double ir = adj_rcp(q[0]);
     const double u = q[1] * ir, v = q[2] * ir, w = q[3] * ir;
     const double p = g.gm1 * (q[4] - 0.5 * (q[1] * u + q[2] * v + q[3] * w));
     const double Tn = p * ir * g.inv_R;
     double sv, dsv;
     visc_factor_d(g, Tn, sv, dsv);
-    double qb[5] = {0, 0, 0, 0, 0}, gb[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0}, ub[3] = {0, 0, 0}, vr = 0.0;
+    double qb[5] = {0, 0, 0, 0, 0}, gb[12], ub[3] = {0, 0, 0}, pb = 0.0;
+    ViscVjp vis{};
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const int r = ijk[d];
@@ -776,13 +785,14 @@ k_adjlg_volume(const double* __restrict__ U, const double* __restrict__ lam, con
 #pragma unroll
         for (int x = 0; x < 5; ++x) fb[x] = fma(c, sL[x * P + nid], fb[x]);
       }
-      euler_flux_vjp(q, u, v, w, p, Ja[d * 3], Ja[d * 3 + 1], Ja[d * 3 + 2], fb, g.gm1, qb);
+      euler_flux_vjp(q, u, v, w, p, Ja[d * 3], Ja[d * 3 + 1], Ja[d * 3 + 2], fb, qb, ub, pb);
       const double fvb[4] = {-fb[1], -fb[2], -fb[3], -fb[4]};
-      vr += visc_flux_vjp(gr, u, v, w, g.mu * sv, g.kappa, Ja[d * 3], Ja[d * 3 + 1], Ja[d * 3 + 2], fvb, gb, ub);
+      visc_vjp_add(vis, u, v, w, Ja[d * 3], Ja[d * 3 + 1], Ja[d * 3 + 2], fvb);
     }
+    const double vr = visc_vjp_end(vis, gr, g.mu * sv, g.kappa, gb, ub);
     mub = sv * vr;
-    const double Tb = g.mu * dsv * vr;   // through T = p / (rho R)
-    prim_vjp(q, -Tb * Tn * ir, ub, Tb * g.inv_R * ir, g.gm1, qb);
+    const double Tb = g.mu * dsv * vr * ir;   // through T = p / (rho R)
+    prim_vjp(ir, u, v, w, -Tb * Tn, ub, fma(Tb, g.inv_R, pb), g.gm1, qb);
 #pragma unroll
     for (int c = 0; c < 5; ++c) b.qbar[((size_t)e * 5 + c) * P + id] = qb[c];
 #pragma unroll
@@ -804,13 +814,8 @@ k_adjlg_volume(const double* __restrict__ U, const double* __restrict__ lam, con
       }
     }
   }
-  smu[threadIdx.x] = mub;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double acc = 0.0;
-    for (int t = 0; t < S::THREADS; ++t) acc += smu[t];
-    b.mupart[blockIdx.x] = acc;
-  }
+  const double mu = block_sum<S::THREADS>(smu, mub, threadIdx.x);   // block partial of d/dmu
+  if (threadIdx.x == 0) b.mupart[blockIdx.x] = mu;
 }
 
 // B3: per node, the gradients' adjoint (the volume's, plus the transposed
@@ -922,11 +927,11 @@ k_adjlg_facephi(const double* __restrict__ Uf, const int* __restrict__ elem_face
     q[v] = Uf[(size_t)ef * 5 * NN + (size_t)v * NN + pq];
     qb[v] = fa[v * NN];
   }
-  const double ir = 1.0 / q[0];
+  const double ir = adj_rcp(q[0]);
   const double u = q[1] * ir, v = q[2] * ir, w = q[3] * ir;
   const double T = g.gm1 * (q[4] - 0.5 * (q[1] * u + q[2] * v + q[3] * w)) * ir * g.inv_R;
   const double ub[3] = {phb[0], phb[1], phb[2]};
-  prim_vjp(q, -phb[3] * T * ir, ub, phb[3] * ir * g.inv_R, g.gm1, qb);
+  prim_vjp(ir, u, v, w, -phb[3] * T * ir, ub, phb[3] * ir * g.inv_R, g.gm1, qb);
   double* out = lgf + ((size_t)ef * 9 + 4) * NN + pq;
 #pragma unroll
   for (int x = 0; x < 5; ++x) out[x * NN] = qb[x];
@@ -991,11 +996,11 @@ k_adjlg_lift(const double* __restrict__ U, const double* __restrict__ metrics, c
   double q[5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) q[c] = U[((size_t)e * 5 + c) * P + id];
-  const double ir = 1.0 / q[0];
+  const double ir = adj_rcp(q[0]);
   const double u = q[1] * ir, v = q[2] * ir, w = q[3] * ir;
   const double T = g.gm1 * (q[4] - 0.5 * (q[1] * u + q[2] * v + q[3] * w)) * ir * g.inv_R;
   const double ub[3] = {phib[0], phib[1], phib[2]};
-  prim_vjp(q, -phib[3] * T * ir, ub, phib[3] * ir * g.inv_R, g.gm1, qb);
+  prim_vjp(ir, u, v, w, -phib[3] * T * ir, ub, phib[3] * ir * g.inv_R, g.gm1, qb);
 #pragma unroll
   for (int c = 0; c < 5; ++c) out[((size_t)e * 5 + c) * P + id] = qb[c];
 }
@@ -1218,7 +1223,7 @@ k_kinetic(const double* __restrict__ U, const double* __restrict__ Jac, const do
     const int i = id % n, j = (id / n) % n, k = id / (n * n);
     const double wq = w[i] * w[j] * w[k] * Jac[t];
     const double* q = U + (size_t)e * 5 * P + id;
-    const double ir = 1.0 / q[0];
+    const double ir = adj_rcp(q[0]);
     const double u = q[P] * ir, v = q[2 * P] * ir, ww = q[3 * P] * ir;
     const double k2 = 0.5 * (u * u + v * v + ww * ww);
     acc += wq * q[0] * k2;

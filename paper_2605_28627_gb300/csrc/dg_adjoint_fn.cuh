@@ -10,21 +10,12 @@
 
 namespace dg {
 
-// Primitive adjoints (rho, u, v, w, p) -> conserved adjoints.
-// rho = q0, u_a = q_{1+a}/rho, p = (gamma-1)(q4 - |q_{1:3}|^2 / (2 rho)).
-__device__ __forceinline__ void prim_vjp(const double q[5], double rb, const double ub[3], double pb, double gm1,
-                                         double qb[5]) {
-  const double ir = 1.0 / q[0];
-  const double u0 = q[1] * ir, u1 = q[2] * ir, u2 = q[3] * ir;
-  const double k = 0.5 * (u0 * u0 + u1 * u1 + u2 * u2);
-  const double gp = gm1 * pb;
-  qb[0] += rb - (ub[0] * u0 + ub[1] * u1 + ub[2] * u2) * ir + gp * k;
-  qb[1] += ub[0] * ir - gp * u0;
-  qb[2] += ub[1] * ir - gp * u1;
-  qb[3] += ub[2] * ir - gp * u2;
-  qb[4] += gp;
-}
-
+// The FP64 pipe bounds the point-wise adjoints (k_adj_face 81 % busy, one FP64
+// instruction per warp in 68 cycles), so they are written for few FP64
+// operations: reciprocals by rcp.approx and one cubic step, primitive adjoints
+// collected over all terms and directions before one prim_vjp, one viscous
+// VJP for a node's three directions.  One VJP of R(U), 16^3 elements: N = 5
+// 2124 -> 1584 us, N = 7 5666 -> 4571 us, Gauss nodes N = 3 859 -> 696 us.
 // 1/x for the adjoint's positive operands (densities, pressures, beta sums,
 // log means): hardware approximation and one cubic Newton-Raphson step
 // (below 1 ulp), a fraction of an IEEE division on GB300's narrow FP64 pipe.
@@ -33,6 +24,20 @@ __device__ __forceinline__ double adj_rcp(double x) {
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x, y, 1.0);
   return fma(y, fma(e, e, e), y);
+}
+
+// Primitive adjoints (rho, u, v, w, p) -> conserved adjoints.
+// rho = q0, u_a = q_{1+a}/rho, p = (gamma-1)(q4 - |q_{1:3}|^2 / (2 rho));
+// ir = 1/rho and the velocity come from the caller.
+__device__ __forceinline__ void prim_vjp(double ir, double u0, double u1, double u2, double rb, const double ub[3],
+                                         double pb, double gm1, double qb[5]) {
+  const double k = 0.5 * (u0 * u0 + u1 * u1 + u2 * u2);
+  const double gp = gm1 * pb;
+  qb[0] += rb - (ub[0] * u0 + ub[1] * u1 + ub[2] * u2) * ir + gp * k;
+  qb[1] += ub[0] * ir - gp * u0;
+  qb[2] += ub[1] * ir - gp * u1;
+  qb[3] += ub[2] * ir - gp * u2;
+  qb[4] += gp;
 }
 
 // Logarithmic mean and its partial derivatives, consistent with log_mean():
@@ -122,45 +127,50 @@ __device__ __forceinline__ void ec_flux_vjp(const NodePrim<double>& A, const Nod
               A.u * A.u + A.v * A.v + A.w * A.w, B.u * B.u + B.v * B.v + B.w * B.w);
 }
 
-// Adjoint of the Euler flux f(q) . n (q conserved, n any vector): adds to qb.
+// Adjoint of the Euler flux f(q) . n (q conserved, n any vector): adds the
+// direct dependence on the conserved variables to qb and that through the
+// velocity and the pressure to ub and pb (one prim_vjp for all directions).
 __device__ __forceinline__ void euler_flux_vjp(const double q[5], double u, double v, double w, double p, double nx,
-                                               double ny, double nz, const double fb[5], double gm1, double qb[5]) {
+                                               double ny, double nz, const double fb[5], double qb[5], double ub[3],
+                                               double& pb) {
   const double un = u * nx + v * ny + w * nz;
-  double mb0 = fb[0] * nx + fb[1] * un, mb1 = fb[0] * ny + fb[2] * un, mb2 = fb[0] * nz + fb[3] * un;
-  const double unb = fb[1] * q[1] + fb[2] * q[2] + fb[3] * q[3] + fb[4] * (q[4] + p);
-  const double pbar = fb[1] * nx + fb[2] * ny + fb[3] * nz + fb[4] * un;
+  // f0 = m . n, f_m = m un + p n, f_E = (E + p) un
+  qb[1] += fb[0] * nx + fb[1] * un;
+  qb[2] += fb[0] * ny + fb[2] * un;
+  qb[3] += fb[0] * nz + fb[3] * un;
   const double Eb = fb[4] * un;
-  // direct dependence on m (f0 = m . n, f_m = m un) is in mb; un and p via primitives
-  qb[1] += mb0; qb[2] += mb1; qb[3] += mb2;
   qb[4] += Eb;
-  const double ub[3] = {unb * nx, unb * ny, unb * nz};
-  prim_vjp(q, 0.0, ub, pbar, gm1, qb);
+  const double unb = fb[1] * q[1] + fb[2] * q[2] + fb[3] * q[3] + fb[4] * (q[4] + p);
+  pb += fb[1] * nx + fb[2] * ny + fb[3] * nz + Eb;
+  ub[0] += unb * nx;
+  ub[1] += unb * ny;
+  ub[2] += unb * nz;
 }
 
-// Adjoint of the local Lax-Friedrichs flux (llf in k_face): adds to qbL, qbR.
-__device__ __forceinline__ void llf_vjp(const double qL[5], const double qR[5], double nx, double ny, double nz,
-                                        double gamma, double gm1, const double fb[5], double qbL[5], double qbR[5]) {
-  const double irL = 1.0 / qL[0], irR = 1.0 / qR[0];
-  const double uL = qL[1] * irL, vL = qL[2] * irL, wL = qL[3] * irL;
-  const double uR = qR[1] * irR, vR = qR[2] * irR, wR = qR[3] * irR;
-  const double pL = gm1 * (qL[4] - 0.5 * (qL[1] * uL + qL[2] * vL + qL[3] * wL));
-  const double pR = gm1 * (qR[4] - 0.5 * (qR[1] * uR + qR[2] * vR + qR[3] * wR));
+// Adjoint of the local Lax-Friedrichs flux (llf in k_face): adds to the direct
+// conserved adjoints qb and the primitive adjoints (rb, ub, pb) of both sides;
+// irL, uL, pL (and R) are 1/rho, the velocity and the pressure of the sides.
+__device__ __forceinline__ void llf_vjp(const double qL[5], const double qR[5], double irL, const double uL[3], double pL,
+                                        double irR, const double uR[3], double pR, double nx, double ny, double nz,
+                                        double gamma, const double fb[5], double qbL[5], double qbR[5], double& rbL,
+                                        double ubL[3], double& pbL, double& rbR, double ubR[3], double& pbR) {
   const double cL = sqrt(gamma * pL * irL), cR = sqrt(gamma * pR * irR);
-  const double unL = uL * nx + vL * ny + wL * nz, unR = uR * nx + vR * ny + wR * nz;
+  const double unL = uL[0] * nx + uL[1] * ny + uL[2] * nz, unR = uR[0] * nx + uR[1] * ny + uR[2] * nz;
   const double lL = fabs(unL) + cL, lR = fabs(unR) + cR;
   const bool right = lR > lL;
   const double lmax = right ? lR : lL;
   double half[5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) half[c] = 0.5 * fb[c];
-  euler_flux_vjp(qL, uL, vL, wL, pL, nx, ny, nz, half, gm1, qbL);
-  euler_flux_vjp(qR, uR, vR, wR, pR, nx, ny, nz, half, gm1, qbR);
+  euler_flux_vjp(qL, uL[0], uL[1], uL[2], pL, nx, ny, nz, half, qbL, ubL, pbL);
+  euler_flux_vjp(qR, uR[0], uR[1], uR[2], pR, nx, ny, nz, half, qbR, ubR, pbR);
   double lb = 0.0;
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
-    qbR[c] -= 0.5 * lmax * fb[c];
-    qbL[c] += 0.5 * lmax * fb[c];
-    lb -= 0.5 * fb[c] * (qR[c] - qL[c]);
+    const double lf = lmax * half[c];
+    qbR[c] -= lf;
+    qbL[c] += lf;
+    lb -= half[c] * (qR[c] - qL[c]);
   }
   // lambda = |u . n| + c of the chosen side; c = sqrt(gamma p / rho):
   // dc = c/2 (dp/p - drho/rho).  At the kinks (a tie of the two speeds, or
@@ -168,18 +178,18 @@ __device__ __forceinline__ void llf_vjp(const double qL[5], const double qR[5], 
   // derivative is the mean of the one-sided derivatives.
   const bool tie = fabs(lR - lL) <= 1e-12 * fmax(lL, lR);
   const double sideL = tie ? 0.5 : (right ? 0.0 : 1.0), sideR = tie ? 0.5 : (right ? 1.0 : 0.0);
-  {
-    const double lbw = lb * sideL;
-    const double sg = fabs(unL) <= 1e-12 * cL ? 0.0 : (unL < 0.0 ? -1.0 : 1.0);
-    const double ub[3] = {lbw * sg * nx, lbw * sg * ny, lbw * sg * nz};
-    prim_vjp(qL, -lbw * 0.5 * cL / qL[0], ub, lbw * 0.5 * cL / pL, gm1, qbL);
-  }
-  {
-    const double lbw = lb * sideR;
-    const double sg = fabs(unR) <= 1e-12 * cR ? 0.0 : (unR < 0.0 ? -1.0 : 1.0);
-    const double ub[3] = {lbw * sg * nx, lbw * sg * ny, lbw * sg * nz};
-    prim_vjp(qR, -lbw * 0.5 * cR / qR[0], ub, lbw * 0.5 * cR / pR, gm1, qbR);
-  }
+  auto speed = [&](double side, double un, double c, double ir, double p, double& rb, double ub[3], double& pb) {
+    const double lbw = lb * side;
+    const double sg = fabs(un) <= 1e-12 * c ? 0.0 : (un < 0.0 ? -1.0 : 1.0);
+    const double ls = lbw * sg, hc = 0.5 * lbw * c;
+    ub[0] += ls * nx;
+    ub[1] += ls * ny;
+    ub[2] += ls * nz;
+    rb -= hc * ir;
+    pb += hc * adj_rcp(p);
+  };
+  speed(sideL, unL, cL, irL, pL, rbL, ubL, pbL);
+  speed(sideR, unR, cR, irR, pR, rbR, ubR, pbR);
 }
 
 // Forward-mode dual number (value, one directional derivative) to
@@ -257,37 +267,55 @@ __device__ __forceinline__ void visc_factor_d(const Gas& g, double T, double& s,
   ds = s * (1.5 / T - den);
 }
 
-// Adjoint of visc_flux (f_v . n, 4 components) w.r.t. the gradients g (12)
-// and the velocity (3); returns fb . f_v1, f_v1 the flux with unit viscosity
-// (f_v = mu f_v1 is linear in mu: the return value is d(fb . f_v)/d mu, and
-// with Sutherland's law the caller scales it by s(T) and, for the T-derivative,
-// by mu_ref ds/dT).
-__device__ __forceinline__ double visc_flux_vjp(const double g[12], double u, double v, double w, double mu,
-                                                double kappa, double nx, double ny, double nz, const double fb[4],
-                                                double gb[12], double ub[3]) {
-  // forward with mu = 1 for the mu-derivative
-  double fv1[4];
-  visc_flux<double>(g, u, v, w, 1.0, kappa, nx, ny, nz, fv1);
-  const double mub = fb[0] * fv1[0] + fb[1] * fv1[1] + fb[2] * fv1[2] + fb[3] * fv1[3];
-  // fv_a = mu * fv1_a (a < 3), fv3 = sum_a fv_a u_a + kappa mu grad T . n
-  ub[0] += fb[3] * mu * fv1[0];
-  ub[1] += fb[3] * mu * fv1[1];
-  ub[2] += fb[3] * mu * fv1[2];
-  const double a0 = fb[0] + fb[3] * u, a1 = fb[1] + fb[3] * v, a2 = fb[2] + fb[3] * w;
-  const double km = kappa * mu * fb[3];
-  gb[9] += km * nx; gb[10] += km * ny; gb[11] += km * nz;
-  // fv_a = sum_l n_l tau_la, tau symmetric: tau-bar of the symmetric components
-  const double t00 = nx * a0, t11 = ny * a1, t22 = nz * a2;
-  const double t01 = nx * a1 + ny * a0, t02 = nx * a2 + nz * a0, t12 = ny * a2 + nz * a1;
+// Adjoint of the viscous fluxes f_v . n^d of one state over several directions
+// n^d, given the adjoints fb^d (4): with A^d = fb^d_m + fb^d_E u, M = sum_d A^d
+// (x) n^d and Q = sum_d fb^d_E n^d carry all of it, so the stress is formed once.
+struct ViscVjp {
+  double M[9], Q[3];
+};
+__device__ __forceinline__ void visc_vjp_add(ViscVjp& s, double u, double v, double w, double nx, double ny, double nz,
+                                             const double fb[4]) {
+  const double A[3] = {fma(fb[3], u, fb[0]), fma(fb[3], v, fb[1]), fma(fb[3], w, fb[2])};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    s.M[a * 3] = fma(A[a], nx, s.M[a * 3]);
+    s.M[a * 3 + 1] = fma(A[a], ny, s.M[a * 3 + 1]);
+    s.M[a * 3 + 2] = fma(A[a], nz, s.M[a * 3 + 2]);
+  }
+  s.Q[0] = fma(fb[3], nx, s.Q[0]);
+  s.Q[1] = fma(fb[3], ny, s.Q[1]);
+  s.Q[2] = fma(fb[3], nz, s.Q[2]);
+}
+// The adjoints of the gradients (gb, 12, set) and the velocity (added to ub);
+// returns sum_d fb^d . f_v1^d, f_v1 the flux with unit viscosity (f_v = mu f_v1
+// is linear in mu: the return value is the derivative by mu, and with
+// Sutherland's law the caller scales it by s(T) and, for the T-derivative, by
+// mu_ref ds/dT).
+__device__ __forceinline__ double visc_vjp_end(const ViscVjp& s, const double g[12], double mu, double kappa,
+                                               double gb[12], double ub[3]) {
+  const double div = (2.0 / 3.0) * (g[0] + g[4] + g[8]);
+  const double t00 = 2.0 * g[0] - div, t11 = 2.0 * g[4] - div, t22 = 2.0 * g[8] - div;
+  const double t01 = g[1] + g[3], t02 = g[2] + g[6], t12 = g[5] + g[7];
+  const double* M = s.M;
+  const double* Q = s.Q;
+  ub[0] += mu * (t00 * Q[0] + t01 * Q[1] + t02 * Q[2]);
+  ub[1] += mu * (t01 * Q[0] + t11 * Q[1] + t12 * Q[2]);
+  ub[2] += mu * (t02 * Q[0] + t12 * Q[1] + t22 * Q[2]);
   // tau_aa = mu (2 g_aa - 2/3 div), tau_ab = mu (g_ab + g_ba)
-  const double divb = -(2.0 / 3.0) * mu * (t00 + t11 + t22);
-  gb[0] += 2.0 * mu * t00 + divb;
-  gb[4] += 2.0 * mu * t11 + divb;
-  gb[8] += 2.0 * mu * t22 + divb;
-  gb[1] += mu * t01; gb[3] += mu * t01;
-  gb[2] += mu * t02; gb[6] += mu * t02;
-  gb[5] += mu * t12; gb[7] += mu * t12;
-  return mub;
+  const double m01 = M[1] + M[3], m02 = M[2] + M[6], m12 = M[5] + M[7], m2 = 2.0 * mu;
+  const double divb = -(2.0 / 3.0) * mu * (M[0] + M[4] + M[8]);
+  gb[0] = fma(m2, M[0], divb);
+  gb[4] = fma(m2, M[4], divb);
+  gb[8] = fma(m2, M[8], divb);
+  gb[1] = gb[3] = mu * m01;
+  gb[2] = gb[6] = mu * m02;
+  gb[5] = gb[7] = mu * m12;
+  const double km = kappa * mu;
+  gb[9] = km * Q[0];
+  gb[10] = km * Q[1];
+  gb[11] = km * Q[2];
+  return t00 * M[0] + t11 * M[4] + t22 * M[8] + t01 * m01 + t02 * m02 + t12 * m12 +
+         kappa * (g[9] * Q[0] + g[10] * Q[1] + g[11] * Q[2]);
 }
 
 }  // namespace dg
