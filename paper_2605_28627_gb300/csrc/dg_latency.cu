@@ -4,7 +4,7 @@
 //
 // With few elements (the 4^3 Taylor-Green case has 128 warps for the GPU's
 // 608 SM sub-partitions) every warp runs alone on its sub-partition, and the
-// FP64 pipe, which takes a warp instruction in about 76 cycles, makes a
+// FP64 pipe, which takes a warp instruction in about 68 cycles, makes a
 // kernel last as long as its longest warp's FP64 instruction stream.  These
 // kernels spread a node's work over three threads, one per reference
 // direction d: the d-thread evaluates the split-form pairs, the viscous flux,
@@ -12,10 +12,10 @@
 // the line derivatives of its direction and one component of every lifted
 // gradient (lifting); the three directions' partial sums are added in a
 // fixed order.  The face flux (LLF) takes two threads per face node, one per
-// side.  One element per block of 3 (N+1)^3 threads, N <= 3.  The
-// sums are grouped differently from the one-thread-per-node kernels, so
-// results agree with them to rounding, not bit for bit.
-#include "dg_stage.cuh"
+// side.  One element per block of 3 (N+1)^3 threads, N <= 3.  The sums of
+// the FP64 parts are grouped differently from the one-thread-per-node kernels,
+// so results agree with them to rounding, not bit for bit.
+#include "dg_volume_fx.cuh"
 
 namespace dg {
 
@@ -107,25 +107,310 @@ k_lift_lat(const double* __restrict__ U, const double* __restrict__ metrics, con
 
 // ---------------------------------------------------------------------------
 // Volume: thread (d, node) takes direction d's pairs, viscous line sum and
-// surface terms; the three partial sums meet in shared memory, and thread
+// surface terms; the three directions' sums meet in shared memory, and thread
 // (d, node) finishes the variables c = d and c = d + 3.
+//
+// Component c of the manufactured source (density wave, see volume_body).
+__device__ __forceinline__ double mms_source_lat(const Gas& g, double sa, double ca, const double* tc, int c) {
+  const double st = tc[0], ct = tc[1];
+  const double sphi = fma(sa, ct, -ca * st);
+  const double cphi = fma(ca, ct, sa * st);
+  const double A = g.mms_amp;
+  const double rp = M_PI * A * cphi;
+  if (c < 4) return 2.0 * rp;
+  const double rw = 2.0 + A * sphi;
+  const double irw = rcp_op(rw);
+  const double lapT = 3.0 * g.inv_R * fma(M_PI * M_PI * A, sphi, 2.0 * rp * rp * irw) * (irw * irw);
+  return fma(-(g.mu * g.kappa), lapT, 3.0 * rp);
+}
+
+// Fixed-point body (the terms and scales of volume_body_fx): the FP64 chain of
+// a warp is the node's primitives, the surface sums and the update, 30
+// instructions instead of 250; what is left is mostly the latency of the launch
+// and of the loads, so every operand is asked for at the start.  Taylor-Green,
+// CUDA events per launch with the FP64 body -> now: N = 2, 4^3 12.3 -> 10.3 us,
+// N = 3, 4^3 16.4 -> 12.3, N = 3, 6^3 24.6 -> 14.3.
+// Words of 8 bytes: the Fx table of D, node data (6 P), metric terms, viscous
+// fluxes (12 P), exchange buffers, primitives (6 P), the directions' sums (54 P).
 template <int N>
-constexpr size_t volume_lat_smem_bytes() {
+struct LatFx {
+  static constexpr int n = N + 1, P = n * n * n, PW = P + (P & 1), ROUNDS = n / 2, JW = 2 * P + PW, XW = 4 * P + PW;
+  static constexpr int tables = (n * n + 1) & ~1, words = tables + 6 * P + 3 * JW + 12 * P + 3 * ROUNDS * XW + 6 * P + 54 * P;
+};
+
+// False (the whole block): the element is out of the fixed-point range.
+template <int N>
+__device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* __restrict__ metrics,
+                                              const i64* __restrict__ jx, const float4* __restrict__ ejx,
+                                              const double* __restrict__ grad, const double* __restrict__ fstar,
+                                              const int* __restrict__ elem_face, const double* __restrict__ mms,
+                                              const double* __restrict__ Dg, int E, const Gas& g, double inv_w0,
+                                              unsigned char* raw, const double* s_tc) {
+  using S = LatShape<N>;
+  using B = LatFx<N>;
+  constexpr int n = S::n, P = S::P, NN = S::NN, JW = B::JW, XW = B::XW, eD = fx_eD(N);
+  Fx* sD = reinterpret_cast<Fx*>(raw);
+  i64* base = reinterpret_cast<i64*>(raw) + B::tables;
+  longlong2* sN = reinterpret_cast<longlong2*>(base);   // [3][P] (rho, b), (|u|^2, u), (v, w)
+  i64* sJ = base + 6 * P;                                // [3]: (J0, J1) [P], J2 [P]
+  i64* sFv = sJ + 3 * JW;                                // [3][4][P]
+  i64* sX = sFv + 12 * P;                                // [ROUNDS][3]: (F0, F1) [P], (F2, F3) [P], F4 [P]
+  double* sQ = reinterpret_cast<double*>(sX + 3 * B::ROUNDS * XW);   // [6][P] u, v, w, rho, b, |u|^2
+  longlong2* sS = reinterpret_cast<longlong2*>(sQ + 6 * P);          // [9][3][P] sums: flux (5), viscous (4)
+  __shared__ int s_mx[kMxCount];
+  __shared__ FxAlign s_al;
+  __shared__ Fx s_G;
+  const int d = threadIdx.x / P, id = threadIdx.x - d * P;
+  const int e = blockIdx.x;
+  const int ijk[3] = {id % n, (id / n) % n, id / NN};
+  // every operand is asked for here: one memory latency (two for the surface
+  // flux) instead of one per phase
+  if (threadIdx.x < kMxCount) s_mx[threadIdx.x] = 0;
+  double q[5] = {1, 0, 0, 0, 1};
+  if (d == 0) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) q[v] = a.U[((size_t)e * 5 + v) * P + id];
+  }
+  const i64* mt = jx + (size_t)e * 10 * P + id;
+  const i64 Ja[3] = {mt[(d * 3) * P], mt[(d * 3 + 1) * P], mt[(d * 3 + 2) * P]};
+  double gr[12];
+#pragma unroll
+  for (int r = 0; r < 12; ++r) gr[r] = grad[((size_t)e * 12 + r) * P + id];
+  const float4 ej = ejx[e];
+  const double* fsr[3] = {nullptr, nullptr, nullptr};
+  double fsg[3] = {0, 0, 0};
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    if (ijk[x] != 0 && ijk[x] != N) continue;
+    const int code = elem_face[e * 6 + 2 * x + (ijk[x] == N ? 1 : 0)];
+    const int fid = dg_idx(code >> 4, 3L * E, kSiteVolFace);   // F = 3 E
+    int p2 = x == 0 ? ijk[1] : ijk[0], q2 = x == 2 ? ijk[1] : ijk[2];
+    if (!(code & 8)) apply_flip<n>(code & 7, p2, q2, p2, q2);
+    fsr[x] = fstar + (size_t)fid * 5 * NN + p2 + n * q2;
+    fsg[x] = (code & 8) ? inv_w0 : -inv_w0;
+  }
+  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
+    const double dr = Dg[t];
+    sD[t] = fx_split(fx_round(t == 0 ? dr + inv_w0 : (t == n * n - 1 ? dr - inv_w0 : dr), kFxQD - eD));
+  }
+  double fs[2][3], Uc[2] = {0, 0}, Gc[2] = {0, 0}, sa = 0.0, ca = 0.0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int c = d + 3 * h;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) fs[h][x] = c < 5 && fsr[x] != nullptr ? fsr[x][c * NN] : 0.0;
+    if (c < 5 && a.mode != 0) {
+      Uc[h] = a.U[((size_t)e * 5 + c) * P + id];
+      Gc[h] = a.Gk[((size_t)e * 5 + c) * P + id];
+    }
+  }
+  const double iJ = metrics[((size_t)e * 10 + 9) * P + id];
+  if (g.source == DG_SOURCE_MMS) {
+    sa = mms[((size_t)e * 2) * P + id];
+    ca = mms[((size_t)e * 2 + 1) * P + id];
+  }
+  __syncthreads();
+  {
+    int mx[kMxCount] = {};
+    auto mag2 = [](double x, double y) { return max(fx_mag(x), fx_mag(y)); };
+    if (d == 0) {
+      const double rho = q[0], ir = rcp_op(rho);
+      const double u = q[1] * ir, v = q[2] * ir, w = q[3] * ir;
+      const double kk = u * u + v * v + w * w;
+      const double p = g.gm1 * fma(-0.5 * rho, kk, q[4]);
+      const double bt = 0.125 * rho * rcp_op(p);   // beta / 4
+      sQ[id] = u; sQ[P + id] = v; sQ[2 * P + id] = w;
+      sQ[3 * P + id] = rho; sQ[4 * P + id] = bt; sQ[5 * P + id] = kk;
+      const int hr = max(__double2hiint(rho), 0), hb = max(__double2hiint(bt), 0);
+      mx[kMxR] = hr;
+      mx[kMxRmin] = 0x7fffffff - hr;
+      mx[kMxB] = hb;
+      mx[kMxBmin] = 0x7fffffff - hb;
+      mx[kMxU] = max(mag2(u, v), fx_mag(w));
+    } else if (d == 1) {
+      mx[kMxG] = max(max(mag2(gr[0], gr[1]), mag2(gr[2], gr[3])),
+                     max(max(mag2(gr[4], gr[5]), mag2(gr[6], gr[7])), fx_mag(gr[8])));
+      mx[kMxT] = max(mag2(gr[9], gr[10]), fx_mag(gr[11]));
+    }
+    __syncwarp();
+    fx_maxima<kMxCount>(0, s_mx, mx);
+  }
+  __syncthreads();
+  FxElem ex = fx_element(s_mx, ej);
+  if (!ex.ok) return false;
+  const int eg = ((__double2hiint(g.inv_gm1) >> 20) & 0x7ff) - 1022;
+  const int ek = ((__double2hiint(g.kappa) >> 20) & 0x7ff) - 1022;
+  const int q1 = 56 - ex.g - ex.e.u, q2 = 59 - ex.t - ek;   // of the viscous energy flux's two terms, + (-e_j)
+  if (threadIdx.x == 3 * P - 1) {
+    FxElem el = ex;
+    fx_element_logs(el, s_mx, ej);
+    s_al = fx_align(el.e, eg, fx_log_mantissa(__double2hiint(g.inv_gm1), 1), eD);
+    s_G = fx_split(fx_from(g.inv_gm1, 62 - eg));
+  }
+  {
+    // node data, and the viscous flux of this direction (scales as in volume_body_fx)
+    const i64 xu = fx_from(sQ[id], kFxQ - ex.e.u), xv = fx_from(sQ[P + id], kFxQ - ex.e.u),
+              xw = fx_from(sQ[2 * P + id], kFxQ - ex.e.u);
+    if (d == 0) sN[id] = make_longlong2(fx_from(sQ[3 * P + id], kFxQ - ex.e.r), fx_from(sQ[4 * P + id], kFxQ - ex.e.b));
+    else if (d == 1) sN[P + id] = make_longlong2(fx_from(sQ[5 * P + id], kFxQ - 2 - 2 * ex.e.u), xu);
+    else sN[2 * P + id] = make_longlong2(xv, xw);
+    reinterpret_cast<longlong2*>(sJ + d * JW)[id] = make_longlong2(Ja[0], Ja[1]);
+    sJ[d * JW + 2 * P + id] = Ja[2];
+    i64 G[9];
+#pragma unroll
+    for (int r = 0; r < 9; ++r) G[r] = fx_from(gr[r], 59 - ex.g);
+    const Fx twothird{715827883, -1431655765};   // 2^62 2/3 / 2^32 and the low word of 2^62 2/3
+    const i64 div = fx_mul<2>(fx_split(G[0] + G[4] + G[8]), twothird);
+    const Fx t00 = fx_split(2 * G[0] - div), t11 = fx_split(2 * G[4] - div), t22 = fx_split(2 * G[8] - div);
+    const Fx t01 = fx_split(G[1] + G[3]), t02 = fx_split(G[2] + G[6]), t12 = fx_split(G[5] + G[7]);
+    const Fx kap = fx_split(fx_from(g.kappa, kFxQ - ek));
+    const Fx J[3] = {fx_split(Ja[0]), fx_split(Ja[1]), fx_split(Ja[2])};
+    FxSum f0 = fx_zero<3>(), f1 = fx_zero<3>(), f2 = fx_zero<3>(), h = fx_zero<3>(), en = fx_zero<2>();
+    fx_add(f0, t00, J[0]); fx_add(f0, t01, J[1]); fx_add(f0, t02, J[2]);
+    fx_add(f1, t01, J[0]); fx_add(f1, t11, J[1]); fx_add(f1, t12, J[2]);
+    fx_add(f2, t02, J[0]); fx_add(f2, t12, J[1]); fx_add(f2, t22, J[2]);
+#pragma unroll
+    for (int l = 0; l < 3; ++l) fx_add(h, fx_split(fx_mul<4>(fx_split(fx_from(gr[9 + l], kFxQ - ex.t)), kap)), J[l]);
+    const i64 v0 = fx_end<3>(f0), v1 = fx_end<3>(f1), v2 = fx_end<3>(f2);
+    fx_add(en, fx_split(v0), fx_split(xu)); fx_add(en, fx_split(v1), fx_split(xv)); fx_add(en, fx_split(v2), fx_split(xw));
+    i64* fv = sFv + d * 4 * P + id;
+    fv[0] = v0;
+    fv[P] = v1;
+    fv[2 * P] = v2;
+    fv[3 * P] = (fx_end<2>(en) >> fx_clamp(q1 - q2)) + (fx_end<3>(h) >> fx_clamp(q2 - q1));
+  }
+  __syncthreads();
+  const int r = d == 0 ? ijk[0] : (d == 1 ? ijk[1] : ijk[2]);
+  const int stride = d == 0 ? 1 : (d == 1 ? n : NN);
+  const int line0 = id - r * stride;
+  FxSum acc[5] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}};
+  constexpr int FULL = (n - 1) / 2;
+  constexpr bool HALF = (n % 2) == 0;
+  const i64* jd = sJ + d * JW;
+  const longlong2* jp = reinterpret_cast<const longlong2*>(jd);
+  auto pair = [&](int ia, int ib, i64 F[5]) {
+    const longlong2 r0 = sN[ia], r1 = sN[ib], k0 = sN[P + ia], k1 = sN[P + ib], v0 = sN[2 * P + ia], v1 = sN[2 * P + ib];
+    const longlong2 j0 = jp[ia], j1 = jp[ib];
+    fx_pair(r0.x, r1.x, r0.y, r1.y, k0.y + k1.y, v0.x + v1.x, v0.y + v1.y, k0.x + k1.x, j0.x + j1.x, j0.y + j1.y,
+            jd[2 * P + ia] + jd[2 * P + ib], s_G, s_al, F, FxLong());
+  };
+  auto put = [&](i64* xs, int at, const i64 F[5]) {
+    reinterpret_cast<longlong2*>(xs)[at] = make_longlong2(F[0], F[1]);
+    reinterpret_cast<longlong2*>(xs)[P + at] = make_longlong2(F[2], F[3]);
+    xs[4 * P + at] = F[4];
+  };
+#pragma unroll 1
+  for (int s = 1; s <= FULL; ++s) {
+    const int m = r + s < n ? r + s : r + s - n;
+    const int mid = line0 + m * stride;
+    i64 F[5];
+    pair(id, mid, F);
+    put(sX + ((s - 1) * 3 + d) * XW, mid, F);
+    const Fx D = sD[r * n + m];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) fx_add(acc[c], D, fx_split(F[c]));
+  }
+  if constexpr (HALF) {
+    // s = n/2: the pairs (r, r + n/2), r < n/2, on half of the direction's threads
+    // (the second half for d > 0, whose warps share no sub-partition with d = 0's)
+    constexpr int H = n / 2;
+    const int w2 = d == 0 ? id : id - P / 2;
+    if (w2 >= 0 && w2 < P / 2) {
+      const int hi = w2 / stride;
+      const int ia = w2 - hi * stride + stride * (hi % H + n * (hi / H));
+      const int ib = ia + H * stride;
+      i64 F[5];
+      pair(ia, ib, F);
+      i64* xh = sX + (FULL * 3 + d) * XW;
+      put(xh, ia, F);
+      put(xh, ib, F);
+    }
+  }
+  // viscous line sum of direction d, with the viscous surface part in the end diagonals
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const i64* line = sFv + (d * 4 + c) * P + line0;
+    FxSum s{0, 0};
+#pragma unroll
+    for (int m = 0; m < n; ++m) fx_add(s, sD[r * n + m], fx_split(line[m * stride]));
+    sS[((5 + c) * 3 + d) * P + id] = make_longlong2(s.p, s.c >> 2);
+  }
+  __syncthreads();
+  auto take_share = [&](const i64* xs, int src) {
+    const Fx D = sD[r * n + src];
+    const longlong2 a0 = reinterpret_cast<const longlong2*>(xs)[id], a1 = reinterpret_cast<const longlong2*>(xs)[P + id];
+    fx_add(acc[0], D, fx_split(a0.x));
+    fx_add(acc[1], D, fx_split(a0.y));
+    fx_add(acc[2], D, fx_split(a1.x));
+    fx_add(acc[3], D, fx_split(a1.y));
+    fx_add(acc[4], D, fx_split(xs[4 * P + id]));
+  };
+#pragma unroll
+  for (int s = 1; s <= FULL; ++s) take_share(sX + ((s - 1) * 3 + d) * XW, r - s >= 0 ? r - s : r - s + n);
+  if constexpr (HALF) take_share(sX + (FULL * 3 + d) * XW, r >= n / 2 ? r - n / 2 : r + n / 2);
+#pragma unroll
+  for (int c = 0; c < 5; ++c) {
+    fx_fold(acc[c]);
+    sS[(c * 3 + d) * P + id] = make_longlong2(acc[c].p, acc[c].c);
+  }
+  __syncthreads();
+  const FxAlign al = s_al;
+  const int qv = kFxQD - 6 - ex.g - ex.e.j - eD, qe = (q1 < q2 ? q1 : q2) - (64 - kFxQD) - ex.e.j - eD;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int c = d + 3 * h;
+    if (c >= 5) break;
+    auto sum = [&](int row, i64& p, i64& f) {
+      const longlong2 x = sS[row * 3 * P + id], y = sS[(row * 3 + 1) * P + id], z = sS[(row * 3 + 2) * P + id];
+      p = x.x + y.x + z.x;
+      f = x.y + y.y + z.y;
+    };
+    i64 p, f;
+    sum(c, p, f);
+    double R = fx_to2<32>(p, f, c == 0 ? al.q0 : (c < 4 ? al.qm : al.qe));
+    if (c > 0) {
+      sum(4 + c, p, f);
+      R = fma(-g.mu, fx_to2<30>(p, f, c < 4 ? qv : qe), R);
+    }
+#pragma unroll
+    for (int x = 0; x < 3; ++x)
+      if (fsr[x] != nullptr) R = fma(fsg[x], fs[h][x], R);
+    const double src = g.source == DG_SOURCE_MMS ? mms_source_lat(g, sa, ca, s_tc, c) : 0.0;
+    const size_t o = ((size_t)e * 5 + c) * P + id;
+    if (a.mode == 0) {
+      a.Ut[o] = fma(-R, iJ, src);
+    } else {
+      const double gk = fma(a.A, Gc[h], a.clock[1] * fma(-R, iJ, src));
+      a.Gk[o] = gk;
+      a.Uw[o] = fma(a.B, gk, Uc[h]);
+    }
+  }
+  return true;
+}
+
+// FP64 body: elements out of the fixed-point range, and Sutherland's law
+// (whose factor every thread of a node would have to apply to the gradients).
+template <int N>
+constexpr size_t volume_lat_f64_bytes() {
   constexpr int n = N + 1, P = n * n * n;
   // D and its three scalings, rho, u (3), beta/4, |u|^2, J a (9), f_v . J a (12),
   // the three directions' exchange buffers (15), which also hold the partial sums
   return sizeof(double) * ((size_t)4 * n * n + 6 * P + 9 * P + 12 * P + 15 * P);
 }
+template <int N>
+constexpr size_t volume_lat_smem_bytes() {
+  return 8 * LatFx<N>::words > volume_lat_f64_bytes<N>() ? 8 * LatFx<N>::words : volume_lat_f64_bytes<N>();
+}
 
 template <int N>
-__global__ void __launch_bounds__(LatShape<N>::THREADS)
-k_volume_lat(StageArgs a, const double* __restrict__ metrics, const double* __restrict__ grad,
-             const double* __restrict__ fstar, const int* __restrict__ elem_face, const double* __restrict__ mms,
-             const double* __restrict__ Dg, int E, Gas g, double inv_w0) {
+__device__ __forceinline__ void volume_lat_f64(const StageArgs& a, const double* __restrict__ metrics,
+                                               const double* __restrict__ grad, const double* __restrict__ fstar,
+                                               const int* __restrict__ elem_face, const double* __restrict__ mms,
+                                               const double* __restrict__ Dg, int E, const Gas& g, double inv_w0,
+                                               unsigned char* raw, const double* s_tc) {
   using S = LatShape<N>;
   constexpr int n = S::n, P = S::P, NN = S::NN;
-  extern __shared__ __align__(16) unsigned char lat_raw[];
-  double* sD = reinterpret_cast<double*>(lat_raw);   // D, viscous surface part in the end diagonals
+  double* sD = reinterpret_cast<double*>(raw);   // D, viscous surface part in the end diagonals
   double* sT0 = sD + n * n;                          // D/4, D/8, D/16 (scaled two-point fluxes)
   double* sT1 = sT0 + n * n;
   double* sT2 = sT1 + n * n;
@@ -136,11 +421,8 @@ k_volume_lat(StageArgs a, const double* __restrict__ metrics, const double* __re
   double* sJ = sK + P;                               // [9][P] J a^d_l, row 3 d + l
   double* sFv = sJ + 9 * P;                          // [3][4][P] (f_v . J a^d)
   double* sX = sFv + 12 * P;                         // [3][5][P] exchange per direction, then partial sums
-  __shared__ double s_tc[2];
   const int d = threadIdx.x / P, id = threadIdx.x - d * P;
   const int e = blockIdx.x;
-  if (threadIdx.x == 0 && g.source == DG_SOURCE_MMS)
-    sincospi(a.clock[0] + a.c_stage * a.clock[1], &s_tc[0], &s_tc[1]);
   for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
     const double dr = Dg[t];
     sD[t] = t == 0 ? dr + inv_w0 : (t == n * n - 1 ? dr - inv_w0 : dr);
@@ -290,23 +572,7 @@ k_volume_lat(StageArgs a, const double* __restrict__ metrics, const double* __re
     const int c = d + 3 * h;
     if (c >= 5) break;
     const double tot = (sX[c * P + id] + sX[(5 + c) * P + id]) + sX[(10 + c) * P + id];
-    // manufactured source (density wave, see volume_body)
-    double src = 0.0;
-    if (g.source == DG_SOURCE_MMS) {
-      const double st = s_tc[0], ct = s_tc[1];
-      const double sphi = fma(sa, ct, -ca * st);
-      const double cphi = fma(ca, ct, sa * st);
-      const double A = g.mms_amp;
-      const double rp = M_PI * A * cphi;
-      if (c < 4) {
-        src = 2.0 * rp;
-      } else {
-        const double rw = 2.0 + A * sphi;
-        const double irw = rcp_op(rw);
-        const double lapT = 3.0 * g.inv_R * fma(M_PI * M_PI * A, sphi, 2.0 * rp * rp * irw) * (irw * irw);
-        src = fma(-(g.mu * g.kappa), lapT, 3.0 * rp);
-      }
-    }
+    const double src = g.source == DG_SOURCE_MMS ? mms_source_lat(g, sa, ca, s_tc, c) : 0.0;
     const size_t o = ((size_t)e * 5 + c) * P + id;
     if (a.mode == 0) {
       a.Ut[o] = fma(-tot, iJ, src);
@@ -316,6 +582,23 @@ k_volume_lat(StageArgs a, const double* __restrict__ metrics, const double* __re
       a.Uw[o] = fma(a.B, gk, a.U[o]);
     }
   }
+}
+
+template <int N>
+__global__ void __launch_bounds__(LatShape<N>::THREADS, 2)
+k_volume_lat(StageArgs a, const double* __restrict__ metrics, const i64* __restrict__ jx,
+             const float4* __restrict__ ejx, const double* __restrict__ grad, const double* __restrict__ fstar,
+             const int* __restrict__ elem_face, const double* __restrict__ mms, const double* __restrict__ Dg, int E,
+             Gas g, double inv_w0) {
+  extern __shared__ __align__(16) unsigned char lat_raw[];
+  __shared__ double s_tc[2];
+  if (threadIdx.x == 2 * LatShape<N>::P && g.source == DG_SOURCE_MMS)
+    sincospi(a.clock[0] + a.c_stage * a.clock[1], &s_tc[0], &s_tc[1]);
+  if (g.visc_law != DG_VISC_SUTHERLAND &&
+      volume_lat_fx<N>(a, metrics, jx, ejx, grad, fstar, elem_face, mms, Dg, E, g, inv_w0, lat_raw, s_tc))
+    return;
+  __syncthreads();
+  volume_lat_f64<N>(a, metrics, grad, fstar, elem_face, mms, Dg, E, g, inv_w0, lat_raw, s_tc);
 }
 
 // ---------------------------------------------------------------------------
@@ -435,8 +718,8 @@ static cudaError_t lift_lat_N(const Ctx& c, const double* U, cudaStream_t s) {
 template <int N>
 static cudaError_t volume_lat_N(const Ctx& c, const StageArgs& a, cudaStream_t s) {
   k_volume_lat<N><<<c.E, LatShape<N>::THREADS, volume_lat_smem_bytes<N>(), s>>>(
-      a, c.d_metrics, (const double*)c.d_grad, (const double*)c.d_fstar, c.d_elem_face, c.d_mms, c.d_D, c.E, c.gas,
-      1.0 / c.w[0]);
+      a, c.d_metrics, c.d_jx, c.d_ejx, (const double*)c.d_grad, (const double*)c.d_fstar, c.d_elem_face, c.d_mms,
+      c.d_D, c.E, c.gas, 1.0 / c.w[0]);
   return cudaGetLastError();
 }
 

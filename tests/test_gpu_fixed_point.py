@@ -74,6 +74,29 @@ def test_blocks_of_both_kinds(orc, N):
     assert np.abs(Ud.cpu().numpy() - ref).max() / np.abs(ref).max() < 1e-10
 
 
+@pytest.mark.parametrize("N,K", [(1, 2), (1, 5), (2, 3), (3, 2), (3, 5)])
+@pytest.mark.parametrize("kind", list(STATES) + ["both"])
+def test_latency_kernels(orc, N, K, kind):
+    """The same on meshes of the latency kernels (three threads per node, one
+    element per block): R(U), and three RK steps in place."""
+    import paper_2605_28627_gb300 as dg
+    kw = STATES["FP64 elements"] if kind == "both" else STATES[kind]
+    mesh = box_mesh(K, min(N, 4), deform="sinprod", rotate_seed=460 + N)
+    mu = 0.02 * (kw.get("rho", (1, 1))[1] * kw.get("vel", 0.5) if kind == "far-off scales" else 1.0)
+    o, s = orc.Oracle(mesh, N, mu=mu), dg.Solver(mesh, N, mu=mu)
+    U = random_state(mesh.n_elems, N, seed=560 + N, **kw)
+    if kind == "both":
+        U[1::2] = random_state(mesh.n_elems, N, seed=570 + N)[1::2]
+    err = _err(s.time_derivative(_cuda(U)).cpu().numpy(), o.time_derivative(U))
+    p = kw.get("p", (0.8, 1.2))
+    assert (err < 1e-12 * max(1.0, 0.5 * (p[0] + p[1]) / (p[1] - p[0]))).all(), err
+    dt = 2e-5 / (1e3 if kind in ("low Mach",) else 1e9 if kind == "far-off scales" else 1.0)
+    Ud = _cuda(U)
+    s.rk_step(Ud, torch.empty_like(Ud), 0.0, dt, 3)
+    ref = o.rk_steps(U, 0.0, dt, 3)
+    assert (np.abs(Ud.cpu().numpy() - ref).max(axis=(0, 2, 3, 4)) <= 1e-11 * np.abs(ref).max(axis=(0, 2, 3, 4))).all()
+
+
 def test_non_finite_state_stays_local():
     """A NaN gives NaN in its element and leaves elements that do not touch it
     as they are, bit for bit; so does an infinity."""
