@@ -24,39 +24,40 @@ __device__ __forceinline__ double sqrt_op(double x) {
   return fma(c * e, fma(0.375, e, 0.5), c);
 }
 
-// Average of the two sides' viscous fluxes . n, over mu for the momentum
-// (w[0..2], sums of both sides) and over mu for the energy (w[3]).
+// Sum of the NS sides' viscous fluxes . n over mu, momentum (w[0..2]) and energy
+// (w[3]); with NS = 1 of the left side alone.
 // False: a non-finite value or an exponent out of range; w is not set.
+template <int NS = 2>
 __device__ __forceinline__ bool face_visc_fx(const double* __restrict__ gL, const double* __restrict__ gR, size_t stride,
                                              double sfL, double sfR, bool scaled, const double uL[3], const double uR[3],
                                              const double nv[3], double kappa, double w[4]) {
-  double g[2][9], t[2][3];
+  double g[NS][9], t[NS][3];
 #pragma unroll
   for (int r = 0; r < 9; ++r) {
     g[0][r] = gL[r * stride];
-    g[1][r] = gR[r * stride];
+    if constexpr (NS == 2) g[1][r] = gR[r * stride];
   }
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
     t[0][l] = gL[(9 + l) * stride];
-    t[1][l] = gR[(9 + l) * stride];
+    if constexpr (NS == 2) t[1][l] = gR[(9 + l) * stride];
   }
   if (scaled) {
 #pragma unroll
     for (int r = 0; r < 9; ++r) {
       g[0][r] *= sfL;
-      g[1][r] *= sfR;
+      if constexpr (NS == 2) g[1][r] *= sfR;
     }
 #pragma unroll
     for (int l = 0; l < 3; ++l) {
       t[0][l] *= sfL;
-      t[1][l] *= sfR;
+      if constexpr (NS == 2) t[1][l] *= sfR;
     }
   }
   auto mag = [](double x) { return __double2hiint(x) & 0x7fffffff; };
   int mg = 0, mt = 0, mu = 0;
 #pragma unroll
-  for (int s = 0; s < 2; ++s) {
+  for (int s = 0; s < NS; ++s) {
 #pragma unroll
     for (int r = 0; r < 9; ++r) mg = max(mg, mag(g[s][r]));
 #pragma unroll
@@ -73,7 +74,7 @@ __device__ __forceinline__ bool face_visc_fx(const double* __restrict__ gL, cons
   const Fx twothird{715827883, -1431655765};   // 2^62 2/3
   i64 v[3] = {0, 0, 0}, en = 0;
 #pragma unroll
-  for (int s = 0; s < 2; ++s) {
+  for (int s = 0; s < NS; ++s) {
     i64 G[9];
 #pragma unroll
     for (int r = 0; r < 9; ++r) G[r] = fx_from(g[s][r], 59 - eg);
@@ -94,7 +95,8 @@ __device__ __forceinline__ bool face_visc_fx(const double* __restrict__ gL, cons
   }
   FxSum h = fx_zero<2>();
 #pragma unroll
-  for (int l = 0; l < 3; ++l) fx_add(h, fx_split(fx_from(t[0][l], 59 - et) + fx_from(t[1][l], 59 - et)), n[l]);
+  for (int l = 0; l < 3; ++l)
+    fx_add(h, fx_split(fx_from(t[0][l], 59 - et) + (NS == 2 ? fx_from(t[NS - 1][l], 59 - et) : 0)), n[l]);
 #pragma unroll
   for (int c = 0; c < 3; ++c) w[c] = fx_to(v[c], 57 - eg);
   w[3] = fma(kappa, fx_to(fx_end<2>(h), 57 - et), fx_to(en, 55 - eg - eu));

@@ -15,6 +15,7 @@
 // side.  One element per block of 3 (N+1)^3 threads, N <= 3.  The sums of
 // the FP64 parts are grouped differently from the one-thread-per-node kernels,
 // so results agree with them to rounding, not bit for bit.
+#include "dg_face_fx.cuh"
 #include "dg_volume_fx.cuh"
 
 namespace dg {
@@ -28,6 +29,11 @@ struct LatShape {
 // Lifting: thread (d, node) forms D_d phi + jump_d for the four lifted
 // variables, then the d-th component of their gradients
 // g_{a,d} = (1/J) sum_d' Ja^{d'}_d (D_d' phi_a + jump_d').
+// The threads of direction 0 evaluate the node's phi while the others evaluate
+// the neighbours' at the face points; the jump (phi_nbr - phi) h, h = +-1/(2
+// w_0), goes into the line sum, its own part through D's corners (D_00 + 1/(2
+// w_0) = 0 there up to rounding).  Bound by the memory latency of its two
+// dependent loads and by some 50 FP64 instructions a warp.
 template <int N>
 constexpr size_t lift_lat_smem_bytes() {
   constexpr int P = LatShape<N>::P, NN = LatShape<N>::NN;
@@ -44,65 +50,61 @@ k_lift_lat(const double* __restrict__ U, const double* __restrict__ metrics, con
   __shared__ double sD[n * n];
   extern __shared__ __align__(16) unsigned char lat_raw[];
   double* sphi = reinterpret_cast<double*>(lat_raw);   // [4][P]
-  double* sjmp = sphi + 4 * P;                         // [6][4][NN]
-  double* sdd = sjmp + 24 * NN;                        // [4][3][P]: D_d phi_a + jump_d
+  double* snb = sphi + 4 * P;                          // [6][4][NN] h phi_nbr
+  double* sdd = snb + 24 * NN;                         // [4][3][P]: D_d phi_a + jump_d
   const int d = threadIdx.x / P, id = threadIdx.x - d * P;
   const int e = blockIdx.x;
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) sD[t] = Dg[t];
+  const double hw = 0.5 * inv_w0;
+  const double* mt = metrics + (size_t)e * 10 * P + id;
+  const double J0 = mt[(0 * 3 + d) * P], J1 = mt[(1 * 3 + d) * P], J2 = mt[(2 * 3 + d) * P];
+  const double iJ = mt[9 * P];
+  auto lifted = [&](const double* q, double scale, double* out, int pitch) {
+    const double rho = q[0], m0 = q[P], m1 = q[2 * P], m2 = q[3 * P], en = q[4 * P], ir = rcp_op(rho);
+    const double u = m0 * ir, v = m1 * ir, w = m2 * ir;
+    const double T = g.gm1 * (en - 0.5 * (m0 * u + m1 * v + m2 * w)) * ir * g.inv_R;
+    out[0] = scale * u;
+    out[pitch] = scale * v;
+    out[2 * pitch] = scale * w;
+    out[3 * pitch] = scale * T;
+  };
   if (d == 0) {
-    const double* q = U + (size_t)e * 5 * P + id;
-    const double rho = q[0], ir = rcp_op(rho);
-    const double m0 = q[P], m1 = q[2 * P], m2 = q[3 * P];
-    const double u = m0 * ir, v = m1 * ir, w = m2 * ir;
-    const double p = g.gm1 * (q[4 * P] - 0.5 * (m0 * u + m1 * v + m2 * w));
-    sphi[id] = u; sphi[P + id] = v; sphi[2 * P + id] = w; sphi[3 * P + id] = p * ir * g.inv_R;
-  }
-  __syncthreads();
-  // face jumps (phi_nbr - phi)/2 (+-1/w_0), threads over the 6 (N+1)^2 face points
-  for (int t = threadIdx.x; t < NF; t += blockDim.x) {
-    const int f = t / NN, pq = t - f * NN;
-    const int code = elem_face[e * 6 + f], nb = elem_nbr[e * 6 + f];
-    int p2, q2;
-    apply_flip<n>(code & 7, pq % n, pq / n, p2, q2);
-    const int enb = dg_idx(nb >> 3, E, kSiteLiftNbr);
-    const double* qn = U + (size_t)enb * 5 * P + face_node<n>(nb & 7, p2, q2);
-    const double rho = qn[0], ir = rcp_op(rho);
-    const double m0 = qn[P], m1 = qn[2 * P], m2 = qn[3 * P];
-    const double u = m0 * ir, v = m1 * ir, w = m2 * ir;
-    const double pr = g.gm1 * (qn[4 * P] - 0.5 * (m0 * u + m1 * v + m2 * w));
-    const double onb[4] = {u, v, w, pr * ir * g.inv_R};
-    const int node = face_node<n>(f, pq % n, pq / n);
-    const double hs = (f & 1) ? 0.5 * inv_w0 : -0.5 * inv_w0;
-#pragma unroll
-    for (int a = 0; a < 4; ++a) sjmp[(f * 4 + a) * NN + pq] = (onb[a] - sphi[a * P + node]) * hs;
+    lifted(U + (size_t)e * 5 * P + id, 1.0, sphi + id, P);
+  } else {
+    for (int t = threadIdx.x - P; t < NF; t += 2 * P) {
+      const int f = t / NN, pq = t - f * NN;
+      const int code = elem_face[e * 6 + f], nb = elem_nbr[e * 6 + f];
+      int p2, q2;
+      apply_flip<n>(code & 7, pq % n, pq / n, p2, q2);
+      const int enb = dg_idx(nb >> 3, E, kSiteLiftNbr);
+      lifted(U + (size_t)enb * 5 * P + face_node<n>(nb & 7, p2, q2), (f & 1) ? hw : -hw, snb + f * 4 * NN + pq, NN);
+    }
+    for (int t = threadIdx.x - P; t < n * n; t += 2 * P) {
+      const double dr = Dg[t];
+      sD[t] = t == 0 ? dr + hw : (t == n * n - 1 ? dr - hw : dr);
+    }
   }
   __syncthreads();
   const int i = id % n, j = (id / n) % n, k = id / NN;
-  const int ijk[3] = {i, j, k};
-  const int r = ijk[d];
+  const int r = d == 0 ? i : (d == 1 ? j : k);
   const int stride = d == 0 ? 1 : (d == 1 ? n : NN);
   const int line0 = id - r * stride;
   const double* jm = nullptr;
   if (r == 0 || r == N)
-    jm = sjmp + (2 * d + (r == N ? 1 : 0)) * 4 * NN + (d == 0 ? j : i) + n * (d == 2 ? j : k);
+    jm = snb + (2 * d + (r == N ? 1 : 0)) * 4 * NN + (d == 0 ? j : i) + n * (d == 2 ? j : k);
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
     double s = jm ? jm[a * NN] : 0.0;
 #pragma unroll
-    for (int m = 0; m < n; ++m) s += sD[r * n + m] * sphi[a * P + line0 + m * stride];
+    for (int m = 0; m < n; ++m) s = fma(sD[r * n + m], sphi[a * P + line0 + m * stride], s);
     sdd[(a * 3 + d) * P + id] = s;
   }
   __syncthreads();
   // component l = d of the four gradients
-  const double* mt = metrics + (size_t)e * 10 * P + id;
-  const double J0 = mt[(0 * 3 + d) * P], J1 = mt[(1 * 3 + d) * P], J2 = mt[(2 * 3 + d) * P];
-  const double iJ = mt[9 * P];
+  const double K0 = J0 * iJ, K1 = J1 * iJ, K2 = J2 * iJ;
   double* go = grad + (size_t)e * 12 * P + id;
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const double gr = J0 * sdd[(a * 3) * P + id] + J1 * sdd[(a * 3 + 1) * P + id] + J2 * sdd[(a * 3 + 2) * P + id];
-    go[(a * 3 + d) * P] = gr * iJ;
-  }
+  for (int a = 0; a < 4; ++a)
+    go[(a * 3 + d) * P] = K0 * sdd[(a * 3) * P + id] + K1 * sdd[(a * 3 + 1) * P + id] + K2 * sdd[(a * 3 + 2) * P + id];
 }
 
 // ---------------------------------------------------------------------------
@@ -630,49 +632,49 @@ k_face_lat(const double* __restrict__ U, const double* __restrict__ grad, const 
     apply_flip<n>(fi.flip, p, q, pp, qq);
   }
   const int node = face_node<n>(lf, pp, qq);
-  double qs[5], gs[12];
+  double qs[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) qs[v] = U[((size_t)e * 5 + v) * P + node];
-#pragma unroll
-  for (int r = 0; r < 12; ++r) gs[r] = grad[((size_t)e * 12 + r) * P + node];
+  const double* gs = grad + (size_t)e * 12 * P + node;
   const double* fg = facegeo + (size_t)f * 4 * NN + pq;
-  const double nx = fg[0], ny = fg[NN], nz = fg[2 * NN], sJ = fg[3 * NN];
+  const double nv[3] = {fg[0], fg[NN], fg[2 * NN]}, sJ = fg[3 * NN];
+  const double nx = nv[0], ny = nv[1], nz = nv[2];
   const double ir = rcp_op(qs[0]);
-  const double u = qs[1] * ir, v = qs[2] * ir, w = qs[3] * ir;
-  const double pr = g.gm1 * (qs[4] - 0.5 * (qs[1] * u + qs[2] * v + qs[3] * w));
-  double fa[5];
-  euler_flux_pm<double>(qs, u, v, w, pr, pr, nx, ny, nz, fa);
-  const double lam = fabs(u * nx + v * ny + w * nz) + sqrt(g.gamma * pr * ir);
-  double mu = g.mu, lk = g.mu * g.kappa;
-  if (g.visc_law == DG_VISC_SUTHERLAND) {
-    const double sf = visc_factor<double>(g, pr * ir * g.inv_R);
-    mu *= sf;
-    lk *= sf;
-  }
+  const double us[3] = {qs[1] * ir, qs[2] * ir, qs[3] * ir};
+  const double pr = g.gm1 * (qs[4] - 0.5 * (qs[1] * us[0] + qs[2] * us[1] + qs[3] * us[2]));
+  const bool suth = g.visc_law == DG_VISC_SUTHERLAND;
+  const double sf = suth ? visc_factor<double>(g, pr * ir * g.inv_R) : 1.0;
   double fv[4];
-  visc_flux<double>(gs, u, v, w, mu, lk, nx, ny, nz, fv);
+  if (!face_visc_fx<1>(gs, gs, P, sf, sf, suth, us, us, nv, g.kappa, fv)) {
+    double a[12];
+#pragma unroll
+    for (int r = 0; r < 12; ++r) a[r] = gs[r * P];
+    visc_flux<double>(a, us[0], us[1], us[2], sf, g.kappa * sf, nx, ny, nz, fv);
+  }
+  const double un = us[0] * nx + us[1] * ny + us[2] * nz;
+  const double lam = fabs(un) + sqrt_op(g.gamma * pr * ir);
+  // f . n - mu f_v . n: one value per component to exchange
+  const double fa[5] = {qs[0] * un, fma(-g.mu, fv[0], fma(qs[1], un, pr * nx)), fma(-g.mu, fv[1], fma(qs[2], un, pr * ny)),
+                        fma(-g.mu, fv[2], fma(qs[3], un, pr * nz)), fma(-g.mu, fv[3], (qs[4] + pr) * un)};
   // the partner side's values
-  double qo[5], fo[5], fvo[4];
+  double qo[5], fo[5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
     qo[c] = __shfl_xor_sync(0xffffffffu, qs[c], 1);
     fo[c] = __shfl_xor_sync(0xffffffffu, fa[c], 1);
   }
-#pragma unroll
-  for (int c = 0; c < 4; ++c) fvo[c] = __shfl_xor_sync(0xffffffffu, fv[c], 1);
   const double lamo = __shfl_xor_sync(0xffffffffu, lam, 1);
   if (!live) return;
   // left = master (even lane), right = slave (odd lane)
   const double lL = side ? lamo : lam, lR = side ? lam : lamo;
-  const double lmax = lR > lL ? lR : lL;
+  const double lmax = lR > lL ? lR : lL, half = 0.5 * sJ;
   double* out = fstar + (size_t)f * 5 * NN + pq;
-  if (side == 0) {
-    out[0] = (0.5 * (fa[0] + fo[0]) - 0.5 * lmax * (qo[0] - qs[0])) * sJ;
+  const int c0 = side ? 3 : 0, c1 = side ? 5 : 3;
 #pragma unroll
-    for (int c = 1; c < 4; ++c)
-      out[(size_t)c * NN] = (0.5 * (fa[c] + fo[c]) - 0.5 * lmax * (qo[c] - qs[c]) - 0.5 * (fv[c - 1] + fvo[c - 1])) * sJ;
-  } else {
-    out[(size_t)4 * NN] = (0.5 * (fo[4] + fa[4]) - 0.5 * lmax * (qs[4] - qo[4]) - 0.5 * (fvo[3] + fv[3])) * sJ;
+  for (int c = 0; c < 5; ++c) {
+    if (c < c0 || c >= c1) continue;
+    const double jump = side ? qs[c] - qo[c] : qo[c] - qs[c];
+    out[(size_t)c * NN] = half * fma(-lmax, jump, fa[c] + fo[c]);
   }
 }
 
