@@ -149,7 +149,7 @@ static cudaError_t enqueue_steps(Ctx& c, double* U, double* G, int nsteps, cudaS
     if ((err = cudaMemsetAsync(G, 0, bytes, s)) != cudaSuccess) return err;
     for (int k = 0; k < rk.stages; ++k) {
       if ((err = launch_fv_switch(c, U, s)) != cudaSuccess) return err;
-      if ((err = launch_lift(c, U, s)) != cudaSuccess) return err;
+      if ((err = launch_lift(c, U, s, true, k > 0 && !c.fv_on)) != cudaSuccess) return err;
       if ((err = launch_face(c, U, s)) != cudaSuccess) return err;
       StageArgs a{U, U, G, nullptr, c.d_clock, rk.C[k], rk.A[k], rk.B[k], 1};
       if ((err = launch_volume(c, a, s)) != cudaSuccess) return err;

@@ -190,8 +190,10 @@ struct Ctx {
 // Launchers implemented per polynomial degree (dg_operator.cu).  With
 // latency_ok the FP64 lifting and volume launchers take the latency kernels
 // (dg_latency.cu) for meshes too small to fill the GPU; the ensemble passes
-// false, so its results do not depend on its tuned plan.
-cudaError_t launch_lift(const Ctx& c, const double* U, cudaStream_t s, bool latency_ok = true);
+// false, so its results do not depend on its tuned plan.  early: the stream's
+// previous operation is a kernel of the same chain (the latency kernels may
+// then start before it ends).
+cudaError_t launch_lift(const Ctx& c, const double* U, cudaStream_t s, bool latency_ok = true, bool early = false);
 cudaError_t launch_lift_fp64(const Ctx& c, const double* U, cudaStream_t s);   // diagnostics: always FP64
 cudaError_t launch_face(const Ctx& c, const double* U, cudaStream_t s, bool latency_ok = true);
 cudaError_t launch_volume(const Ctx& c, const StageArgs& a, cudaStream_t s, bool latency_ok = true);
@@ -199,7 +201,7 @@ cudaError_t launch_volume(const Ctx& c, const StageArgs& a, cudaStream_t s, bool
 constexpr long kLatencyNodes = 16384;
 bool use_latency_kernels(const Ctx& c);
 cudaError_t setup_latency(int N);
-cudaError_t launch_lift_lat(const Ctx& c, const double* U, cudaStream_t s);
+cudaError_t launch_lift_lat(const Ctx& c, const double* U, cudaStream_t s, bool early = false);
 cudaError_t launch_volume_lat(const Ctx& c, const StageArgs& a, cudaStream_t s);
 cudaError_t launch_face_lat(const Ctx& c, const double* U, cudaStream_t s);   // LLF surface flux only
 cudaError_t setup_kernels(int N);

@@ -20,6 +20,22 @@
 
 namespace dg {
 
+// The three kernels of a stage are launched so that the next one may start while
+// the last ends (programmatic dependent launch): each lets it before its last
+// few operations, loads what no kernel writes (metric terms, face lists, D) and
+// then waits for the previous kernel's completion.  Let start by a kernel's
+// first instruction the next one took its place on the SMs (6^3, N = 3: 32.4 us
+// per stage against 23.2, and 23.6 without).  Pointers to data of previous kernels go through after_previous():
+// an opaque copy made after the wait, so that no load of theirs is moved before
+// it or takes the read-only path.
+__device__ __forceinline__ void start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename T>
+__device__ __forceinline__ T* after_previous(T* p) {
+  asm volatile("" : "+l"(p)::"memory");
+  return p;
+}
+
 template <int N>
 struct LatShape {
   static constexpr int n = N + 1, P = n * n * n, NN = n * n, THREADS = 3 * P;
@@ -42,7 +58,7 @@ constexpr size_t lift_lat_smem_bytes() {
 
 template <int N>
 __global__ void __launch_bounds__(LatShape<N>::THREADS)
-k_lift_lat(const double* __restrict__ U, const double* __restrict__ metrics, const int* __restrict__ elem_nbr,
+k_lift_lat(const double* __restrict__ U_, const double* __restrict__ metrics, const int* __restrict__ elem_nbr,
            const int* __restrict__ elem_face, const double* __restrict__ Dg, double* __restrict__ grad, int E,
            Gas g, double inv_w0) {
   using S = LatShape<N>;
@@ -67,20 +83,35 @@ k_lift_lat(const double* __restrict__ U, const double* __restrict__ metrics, con
     out[2 * pitch] = scale * w;
     out[3 * pitch] = scale * T;
   };
-  if (d == 0) {
-    lifted(U + (size_t)e * 5 * P + id, 1.0, sphi + id, P);
-  } else {
-    for (int t = threadIdx.x - P; t < NF; t += 2 * P) {
+  constexpr int NI = (NF + 2 * P - 1) / (2 * P);   // face points of a thread of directions 1 and 2
+  int nbr[NI] = {};
+  if (d != 0) {
+#pragma unroll
+    for (int x = 0; x < NI; ++x) {
+      const int t = threadIdx.x - P + x * 2 * P;
+      if (t >= NF) break;
       const int f = t / NN, pq = t - f * NN;
       const int code = elem_face[e * 6 + f], nb = elem_nbr[e * 6 + f];
       int p2, q2;
       apply_flip<n>(code & 7, pq % n, pq / n, p2, q2);
-      const int enb = dg_idx(nb >> 3, E, kSiteLiftNbr);
-      lifted(U + (size_t)enb * 5 * P + face_node<n>(nb & 7, p2, q2), (f & 1) ? hw : -hw, snb + f * 4 * NN + pq, NN);
+      nbr[x] = dg_idx(nb >> 3, E, kSiteLiftNbr) * 5 * P + face_node<n>(nb & 7, p2, q2);
     }
     for (int t = threadIdx.x - P; t < n * n; t += 2 * P) {
       const double dr = Dg[t];
       sD[t] = t == 0 ? dr + hw : (t == n * n - 1 ? dr - hw : dr);
+    }
+  }
+  wait_previous();
+  const double* U = after_previous(U_);
+  if (d == 0) {
+    lifted(U + (size_t)e * 5 * P + id, 1.0, sphi + id, P);
+  } else {
+#pragma unroll
+    for (int x = 0; x < NI; ++x) {
+      const int t = threadIdx.x - P + x * 2 * P;
+      if (t >= NF) break;
+      const int f = t / NN, pq = t - f * NN;
+      lifted(U + nbr[x], (f & 1) ? hw : -hw, snb + f * 4 * NN + pq, NN);
     }
   }
   __syncthreads();
@@ -99,7 +130,7 @@ k_lift_lat(const double* __restrict__ U, const double* __restrict__ metrics, con
     sdd[(a * 3 + d) * P + id] = s;
   }
   __syncthreads();
-  // component l = d of the four gradients
+  start_next();
   const double K0 = J0 * iJ, K1 = J1 * iJ, K2 = J2 * iJ;
   double* go = grad + (size_t)e * 12 * P + id;
 #pragma unroll
@@ -144,10 +175,10 @@ struct LatFx {
 template <int N>
 __device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* __restrict__ metrics,
                                               const i64* __restrict__ jx, const float4* __restrict__ ejx,
-                                              const double* __restrict__ grad, const double* __restrict__ fstar,
+                                              const double* grad_, const double* fstar_,
                                               const int* __restrict__ elem_face, const double* __restrict__ mms,
                                               const double* __restrict__ Dg, int E, const Gas& g, double inv_w0,
-                                              unsigned char* raw, const double* s_tc) {
+                                              unsigned char* raw, double* s_tc) {
   using S = LatShape<N>;
   using B = LatFx<N>;
   constexpr int n = S::n, P = S::P, NN = S::NN, JW = B::JW, XW = B::XW, eD = fx_eD(N);
@@ -165,21 +196,12 @@ __device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* 
   const int d = threadIdx.x / P, id = threadIdx.x - d * P;
   const int e = blockIdx.x;
   const int ijk[3] = {id % n, (id / n) % n, id / NN};
-  // every operand is asked for here: one memory latency (two for the surface
-  // flux) instead of one per phase
+  // every operand is asked for here, what no kernel writes before the wait
   if (threadIdx.x < kMxCount) s_mx[threadIdx.x] = 0;
-  double q[5] = {1, 0, 0, 0, 1};
-  if (d == 0) {
-#pragma unroll
-    for (int v = 0; v < 5; ++v) q[v] = a.U[((size_t)e * 5 + v) * P + id];
-  }
   const i64* mt = jx + (size_t)e * 10 * P + id;
   const i64 Ja[3] = {mt[(d * 3) * P], mt[(d * 3 + 1) * P], mt[(d * 3 + 2) * P]};
-  double gr[12];
-#pragma unroll
-  for (int r = 0; r < 12; ++r) gr[r] = grad[((size_t)e * 12 + r) * P + id];
   const float4 ej = ejx[e];
-  const double* fsr[3] = {nullptr, nullptr, nullptr};
+  int fso[3] = {-1, -1, -1};   // surface flux of the node, per direction
   double fsg[3] = {0, 0, 0};
 #pragma unroll
   for (int x = 0; x < 3; ++x) {
@@ -188,28 +210,42 @@ __device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* 
     const int fid = dg_idx(code >> 4, 3L * E, kSiteVolFace);   // F = 3 E
     int p2 = x == 0 ? ijk[1] : ijk[0], q2 = x == 2 ? ijk[1] : ijk[2];
     if (!(code & 8)) apply_flip<n>(code & 7, p2, q2, p2, q2);
-    fsr[x] = fstar + (size_t)fid * 5 * NN + p2 + n * q2;
+    fso[x] = fid * 5 * NN + p2 + n * q2;
     fsg[x] = (code & 8) ? inv_w0 : -inv_w0;
   }
   for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
     const double dr = Dg[t];
     sD[t] = fx_split(fx_round(t == 0 ? dr + inv_w0 : (t == n * n - 1 ? dr - inv_w0 : dr), kFxQD - eD));
   }
-  double fs[2][3], Uc[2] = {0, 0}, Gc[2] = {0, 0}, sa = 0.0, ca = 0.0;
+  const double iJ = metrics[((size_t)e * 10 + 9) * P + id];
+  double sa = 0.0, ca = 0.0;
+  if (g.source == DG_SOURCE_MMS) {
+    sa = mms[((size_t)e * 2) * P + id];
+    ca = mms[((size_t)e * 2 + 1) * P + id];
+  }
+  wait_previous();
+  const double* grad = after_previous(grad_);
+  const double* fstar = after_previous(fstar_);
+  if (threadIdx.x == 2 * P && g.source == DG_SOURCE_MMS)
+    sincospi(a.clock[0] + a.c_stage * a.clock[1], &s_tc[0], &s_tc[1]);
+  double q[5] = {1, 0, 0, 0, 1};
+  if (d == 0) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) q[v] = a.U[((size_t)e * 5 + v) * P + id];
+  }
+  double gr[12];
+#pragma unroll
+  for (int r = 0; r < 12; ++r) gr[r] = grad[((size_t)e * 12 + r) * P + id];
+  double fs[2][3], Uc[2] = {0, 0}, Gc[2] = {0, 0};
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int c = d + 3 * h;
 #pragma unroll
-    for (int x = 0; x < 3; ++x) fs[h][x] = c < 5 && fsr[x] != nullptr ? fsr[x][c * NN] : 0.0;
+    for (int x = 0; x < 3; ++x) fs[h][x] = c < 5 && fso[x] >= 0 ? fstar[fso[x] + c * NN] : 0.0;
     if (c < 5 && a.mode != 0) {
       Uc[h] = a.U[((size_t)e * 5 + c) * P + id];
       Gc[h] = a.Gk[((size_t)e * 5 + c) * P + id];
     }
-  }
-  const double iJ = metrics[((size_t)e * 10 + 9) * P + id];
-  if (g.source == DG_SOURCE_MMS) {
-    sa = mms[((size_t)e * 2) * P + id];
-    ca = mms[((size_t)e * 2 + 1) * P + id];
   }
   __syncthreads();
   {
@@ -356,6 +392,7 @@ __device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* 
     sS[(c * 3 + d) * P + id] = make_longlong2(acc[c].p, acc[c].c);
   }
   __syncthreads();
+  start_next();
   const FxAlign al = s_al;
   const int qv = kFxQD - 6 - ex.g - ex.e.j - eD, qe = (q1 < q2 ? q1 : q2) - (64 - kFxQD) - ex.e.j - eD;
 #pragma unroll
@@ -376,7 +413,7 @@ __device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* 
     }
 #pragma unroll
     for (int x = 0; x < 3; ++x)
-      if (fsr[x] != nullptr) R = fma(fsg[x], fs[h][x], R);
+      if (fso[x] >= 0) R = fma(fsg[x], fs[h][x], R);
     const double src = g.source == DG_SOURCE_MMS ? mms_source_lat(g, sa, ca, s_tc, c) : 0.0;
     const size_t o = ((size_t)e * 5 + c) * P + id;
     if (a.mode == 0) {
@@ -406,7 +443,7 @@ constexpr size_t volume_lat_smem_bytes() {
 
 template <int N>
 __device__ __forceinline__ void volume_lat_f64(const StageArgs& a, const double* __restrict__ metrics,
-                                               const double* __restrict__ grad, const double* __restrict__ fstar,
+                                               const double* grad, const double* fstar,
                                                const int* __restrict__ elem_face, const double* __restrict__ mms,
                                                const double* __restrict__ Dg, int E, const Gas& g, double inv_w0,
                                                unsigned char* raw, const double* s_tc) {
@@ -594,13 +631,16 @@ k_volume_lat(StageArgs a, const double* __restrict__ metrics, const i64* __restr
              Gas g, double inv_w0) {
   extern __shared__ __align__(16) unsigned char lat_raw[];
   __shared__ double s_tc[2];
-  if (threadIdx.x == 2 * LatShape<N>::P && g.source == DG_SOURCE_MMS)
-    sincospi(a.clock[0] + a.c_stage * a.clock[1], &s_tc[0], &s_tc[1]);
-  if (g.visc_law != DG_VISC_SUTHERLAND &&
-      volume_lat_fx<N>(a, metrics, jx, ejx, grad, fstar, elem_face, mms, Dg, E, g, inv_w0, lat_raw, s_tc))
-    return;
-  __syncthreads();
-  volume_lat_f64<N>(a, metrics, grad, fstar, elem_face, mms, Dg, E, g, inv_w0, lat_raw, s_tc);
+  if (g.visc_law != DG_VISC_SUTHERLAND) {
+    if (volume_lat_fx<N>(a, metrics, jx, ejx, grad, fstar, elem_face, mms, Dg, E, g, inv_w0, lat_raw, s_tc)) return;
+    __syncthreads();
+  } else {
+    wait_previous();
+    if (threadIdx.x == 0 && g.source == DG_SOURCE_MMS)
+      sincospi(a.clock[0] + a.c_stage * a.clock[1], &s_tc[0], &s_tc[1]);
+  }
+  volume_lat_f64<N>(a, metrics, after_previous(grad), after_previous(fstar), elem_face, mms, Dg, E, g, inv_w0, lat_raw,
+                    s_tc);
 }
 
 // ---------------------------------------------------------------------------
@@ -612,7 +652,7 @@ k_volume_lat(StageArgs a, const double* __restrict__ metrics, const i64* __restr
 //   F* = (1/2 (f_L + f_R) . n - 1/2 lambda_max (q_R - q_L) - 1/2 (f_v,L + f_v,R) . n) sJ.
 template <int N>
 __global__ void __launch_bounds__(64)
-k_face_lat(const double* __restrict__ U, const double* __restrict__ grad, const FaceInfo* __restrict__ faces,
+k_face_lat(const double* __restrict__ U_, const double* __restrict__ grad_, const FaceInfo* __restrict__ faces,
            const double* __restrict__ facegeo, double* __restrict__ fstar, int F, Gas g) {
   constexpr int n = N + 1, P = n * n * n, NN = n * n;
   const long gid = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 1;
@@ -632,12 +672,14 @@ k_face_lat(const double* __restrict__ U, const double* __restrict__ grad, const 
     apply_flip<n>(fi.flip, p, q, pp, qq);
   }
   const int node = face_node<n>(lf, pp, qq);
-  double qs[5];
-#pragma unroll
-  for (int v = 0; v < 5; ++v) qs[v] = U[((size_t)e * 5 + v) * P + node];
-  const double* gs = grad + (size_t)e * 12 * P + node;
   const double* fg = facegeo + (size_t)f * 4 * NN + pq;
   const double nv[3] = {fg[0], fg[NN], fg[2 * NN]}, sJ = fg[3 * NN];
+  wait_previous();
+  const double* qp = after_previous(U_) + (size_t)e * 5 * P + node;
+  const double* gs = after_previous(grad_) + (size_t)e * 12 * P + node;
+  double qs[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) qs[v] = qp[v * P];
   const double nx = nv[0], ny = nv[1], nz = nv[2];
   const double ir = rcp_op(qs[0]);
   const double us[3] = {qs[1] * ir, qs[2] * ir, qs[3] * ir};
@@ -656,7 +698,7 @@ k_face_lat(const double* __restrict__ U, const double* __restrict__ grad, const 
   // f . n - mu f_v . n: one value per component to exchange
   const double fa[5] = {qs[0] * un, fma(-g.mu, fv[0], fma(qs[1], un, pr * nx)), fma(-g.mu, fv[1], fma(qs[2], un, pr * ny)),
                         fma(-g.mu, fv[2], fma(qs[3], un, pr * nz)), fma(-g.mu, fv[3], (qs[4] + pr) * un)};
-  // the partner side's values
+  start_next();
   double qo[5], fo[5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
@@ -686,6 +728,10 @@ static cudaError_t lat_setup() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_volume_lat<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)volume_lat_smem_bytes<N>());
+  // one split of L1 for the three, so that blocks of two of them fit on an SM at a time
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lift_lat<N>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_face_lat<N>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_volume_lat<N>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   return e;
 }
 
@@ -710,26 +756,49 @@ bool use_latency_kernels(const Ctx& c) {
          (long)c.E * c.P <= kLatencyNodes;
 }
 
+// Launch that may start before the stream's previous kernel has ended.  Only for
+// meshes of up to 8 warps per SM: there a stage takes 2 to 3 us less (4^3: N = 1
+// 17.4 -> 15.1, 2 17.3 -> 15.1, 3 18.8 -> 16.3; 5^3 N = 3 19.0 -> 18.6), with more
+// the waiting blocks keep the running kernel's out (8^3 N = 2 23.8 -> 27.1).
+constexpr int kEarlyWarpsPerSM = 8, kSMs = 152;
 template <int N>
-static cudaError_t lift_lat_N(const Ctx& c, const double* U, cudaStream_t s) {
-  k_lift_lat<N><<<c.E, LatShape<N>::THREADS, lift_lat_smem_bytes<N>(), s>>>(
-      U, c.d_metrics, c.d_elem_nbr, c.d_elem_face, c.d_D, (double*)c.d_grad, c.E, c.gas, 1.0 / c.w[0]);
-  return cudaGetLastError();
+static bool early_launch(const Ctx& c) {
+  return (long)c.E * ((LatShape<N>::THREADS + 31) / 32) <= (long)kEarlyWarpsPerSM * kSMs;
+}
+template <int N, typename... P, typename... A>
+static cudaError_t launch_lat(const Ctx& c, void (*kernel)(P...), bool early, int grid, int block, size_t smem,
+                              cudaStream_t s, A... args) {
+  cudaLaunchAttribute at[1] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = early && early_launch<N>(c) ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+template <int N>
+static cudaError_t lift_lat_N(const Ctx& c, const double* U, cudaStream_t s, bool early) {
+  return launch_lat<N>(c, k_lift_lat<N>, early, c.E, LatShape<N>::THREADS, lift_lat_smem_bytes<N>(), s, U, c.d_metrics,
+                       c.d_elem_nbr, c.d_elem_face, c.d_D, (double*)c.d_grad, c.E, c.gas, 1.0 / c.w[0]);
 }
 
 template <int N>
 static cudaError_t volume_lat_N(const Ctx& c, const StageArgs& a, cudaStream_t s) {
-  k_volume_lat<N><<<c.E, LatShape<N>::THREADS, volume_lat_smem_bytes<N>(), s>>>(
-      a, c.d_metrics, c.d_jx, c.d_ejx, (const double*)c.d_grad, (const double*)c.d_fstar, c.d_elem_face, c.d_mms,
-      c.d_D, c.E, c.gas, 1.0 / c.w[0]);
-  return cudaGetLastError();
+  return launch_lat<N>(c, k_volume_lat<N>, true, c.E, LatShape<N>::THREADS, volume_lat_smem_bytes<N>(), s, a, c.d_metrics,
+                       c.d_jx, c.d_ejx, (const double*)c.d_grad, (const double*)c.d_fstar, c.d_elem_face, c.d_mms, c.d_D,
+                       c.E, c.gas, 1.0 / c.w[0]);
 }
 
-cudaError_t launch_lift_lat(const Ctx& c, const double* U, cudaStream_t s) {
+cudaError_t launch_lift_lat(const Ctx& c, const double* U, cudaStream_t s, bool early) {
   switch (c.N) {
-    case 1: return lift_lat_N<1>(c, U, s);
-    case 2: return lift_lat_N<2>(c, U, s);
-    case 3: return lift_lat_N<3>(c, U, s);
+    case 1: return lift_lat_N<1>(c, U, s, early);
+    case 2: return lift_lat_N<2>(c, U, s, early);
+    case 3: return lift_lat_N<3>(c, U, s, early);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -737,9 +806,8 @@ cudaError_t launch_lift_lat(const Ctx& c, const double* U, cudaStream_t s) {
 template <int N>
 static cudaError_t face_lat_N(const Ctx& c, const double* U, cudaStream_t s) {
   const long threads = 2L * c.nfaces * (N + 1) * (N + 1);
-  k_face_lat<N><<<(int)((threads + 63) / 64), 64, 0, s>>>(U, (const double*)c.d_grad, c.d_faces, c.d_facegeo,
-                                                         (double*)c.d_fstar, c.nfaces, c.gas);
-  return cudaGetLastError();
+  return launch_lat<N>(c, k_face_lat<N>, true, (int)((threads + 63) / 64), 64, 0, s, U, (const double*)c.d_grad, c.d_faces,
+                       c.d_facegeo, (double*)c.d_fstar, c.nfaces, c.gas);
 }
 
 cudaError_t launch_face_lat(const Ctx& c, const double* U, cudaStream_t s) {

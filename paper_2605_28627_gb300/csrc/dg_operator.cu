@@ -121,9 +121,9 @@ static cudaError_t face_N(const Ctx& c, const double* U, cudaStream_t s) {
 
 // On Gauss nodes the lifting launcher also computes the face values of U
 // first (k_prolong_lg), and the face kernel works on face values.
-cudaError_t launch_lift(const Ctx& c, const double* U, cudaStream_t s, bool latency_ok) {
+cudaError_t launch_lift(const Ctx& c, const double* U, cudaStream_t s, bool latency_ok, bool early) {
   if (c.prm.nodes == DG_NODES_LG) return launch_lift_lg(c, U, s);
-  if (latency_ok && use_latency_kernels(c)) return launch_lift_lat(c, U, s);
+  if (latency_ok && use_latency_kernels(c)) return launch_lift_lat(c, U, s, early);
   DG_DISPATCH(lift_N, c, U, c.prm.precision != DG_FP32OP, s)
 }
 cudaError_t launch_lift_fp64(const Ctx& c, const double* U, cudaStream_t s) {
