@@ -68,7 +68,6 @@ static dg_status step_adjoint(Ctx* c, const double* Un, double* lam, double* dJd
   double* tmp = Gb + st;                // dt * Gb, then VJP output
   // forward recomputation of the stage states
   ADJ_CUDA(cudaMemcpyAsync(Ws, Un, bytes, cudaMemcpyDeviceToDevice, s), c, "stage copy");
-  ADJ_CUDA(cudaMemsetAsync(G, 0, bytes, s), c, "memset");
   ADJ_CUDA(launch_set_clock(c->d_clock, t, dt, s), c, "clock");
   for (int k = 0; k < rk.stages; ++k) {
     ADJ_CUDA(cudaMemcpyAsync(c->d_adj_stage + (size_t)k * st, Ws, bytes, cudaMemcpyDeviceToDevice, s), c, "stage copy");
@@ -89,14 +88,12 @@ static dg_status step_adjoint(Ctx* c, const double* Un, double* lam, double* dJd
   return DG_OK;
 }
 
-// forward steps from `from` (in place on U), each step zeroing the register
+// forward steps from `from` (in place on U)
 static dg_status advance(Ctx* c, double* U, double* G, double t, double dt, int nsteps, cudaStream_t s) {
   if (nsteps <= 0) return DG_OK;
   ADJ_CUDA(launch_set_clock(c->d_clock, t, dt, s), c, "clock");
-  const size_t bytes = sizeof(double) * (size_t)c->E * 5 * c->P;
   const RkScheme rk = rk_scheme(c->prm.rk_scheme);
   for (int st = 0; st < nsteps; ++st) {
-    ADJ_CUDA(cudaMemsetAsync(G, 0, bytes, s), c, "memset");
     for (int k = 0; k < rk.stages; ++k) {
       ADJ_CUDA(launch_lift(*c, U, s), c, "lift");
       ADJ_CUDA(launch_face(*c, U, s), c, "face");

@@ -139,17 +139,15 @@ static void release(Ctx* c) {
   if (c->h_clock) cudaFreeHost(c->h_clock);
 }
 
-// The RK step sequence for one call: per step, zero the register, five stages
-// of (lift, face, volume+update), advance the clock.
+// The RK step sequence for one call: per step, the stages of (lift, face,
+// volume+update), then advance the clock.  The first stage sets the register.
 static cudaError_t enqueue_steps(Ctx& c, double* U, double* G, int nsteps, cudaStream_t s) {
   cudaError_t err = cudaSuccess;
-  const size_t bytes = sizeof(double) * (size_t)c.E * 5 * c.P;
   const RkScheme rk = rk_scheme(c.prm.rk_scheme);
   for (int st = 0; st < nsteps; ++st) {
-    if ((err = cudaMemsetAsync(G, 0, bytes, s)) != cudaSuccess) return err;
     for (int k = 0; k < rk.stages; ++k) {
       if ((err = launch_fv_switch(c, U, s)) != cudaSuccess) return err;
-      if ((err = launch_lift(c, U, s, true, k > 0 && !c.fv_on)) != cudaSuccess) return err;
+      if ((err = launch_lift(c, U, s, true, st + k > 0 && !c.fv_on)) != cudaSuccess) return err;
       if ((err = launch_face(c, U, s)) != cudaSuccess) return err;
       StageArgs a{U, U, G, nullptr, c.d_clock, rk.C[k], rk.A[k], rk.B[k], 1};
       if ((err = launch_volume(c, a, s)) != cudaSuccess) return err;

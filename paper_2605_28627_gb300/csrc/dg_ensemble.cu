@@ -731,10 +731,6 @@ dg_status dg_ensemble_step(dg_ensemble* e, double* const* dU, double* const* dG,
         err = cudaStreamWaitEvent(bs, fork, 0);
         for (const Unit& u : lanes[b]) {
           const Group& g = e->groups[u.g];
-          for (int r : g.members) {
-            if (err != cudaSuccess || (u.r >= 0 && r != u.r)) continue;
-            err = cudaMemsetAsync(e->cur_G[r], 0, sizeof(double) * (size_t)e->members[r]->E * e->members[r]->P * 5, bs);
-          }
           for (int k = 0; k < e->rk.stages && err == cudaSuccess; ++k)
             err = u.r >= 0 ? one_member_stage(e, u.r, k, e->rk.A, e->rk.B, bs) : enqueue_stage(e, g, k, bs);
         }

@@ -582,7 +582,7 @@ k_fv_volume(StageArgs a, const int* __restrict__ lists, const int* __restrict__ 
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
       const size_t o = o0 + (size_t)c * P;
-      const double gk = fma(a.A, a.Gk[o], dt * fma(jr[c], iJ, src[c]));
+      const double gk = fma(a.A, rk_register(a, o), dt * fma(jr[c], iJ, src[c]));
       a.Gk[o] = gk;
       a.Uw[o] = fma(a.B, gk, a.U[o]);
     }

@@ -709,7 +709,7 @@ __device__ __forceinline__ void volume_lg_body(const StageArgs& a, const R* __re
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
       const size_t o = o0 + (size_t)c * P;
-      const double gk = fma(a.A, a.Gk[o], dt * fma(-accd[c], iJ, src[c]));
+      const double gk = fma(a.A, rk_register(a, o), dt * fma(-accd[c], iJ, src[c]));
       a.Gk[o] = gk;
       a.Uw[o] = fma(a.B, gk, q[c]);
     }

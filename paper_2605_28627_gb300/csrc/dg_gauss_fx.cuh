@@ -381,7 +381,7 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
     if (a.mode == 0) {
       a.Ut[o] = R;
     } else {
-      const double gk = fma(a.A, a.Gk[o], a.clock[1] * R);
+      const double gk = fma(a.A, rk_register(a, o), a.clock[1] * R);
       a.Gk[o] = gk;
       a.Uw[o] = fma(a.B, gk, q[c]);
     }

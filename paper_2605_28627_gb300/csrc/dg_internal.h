@@ -98,7 +98,7 @@ struct StageArgs {
   double* Gk;            // LSERK register or NULL
   double* Ut;            // time-derivative output (mode 0) or NULL
   const double* clock;   // device {t, dt}
-  double c_stage, A, B;  // stage time fraction and LSERK coefficients
+  double c_stage, A, B;  // stage time fraction and LSERK coefficients (A = 0, a step's first stage: Gk is not read)
   int mode;              // 0: write Ut; 1: LSERK update
   // Element slots of the DG volume kernel: NULL, every element; else slot s <
   // *list_len is element list[s] (the DG elements when FV sub-cell elements

@@ -244,7 +244,7 @@ __device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* 
     for (int x = 0; x < 3; ++x) fs[h][x] = c < 5 && fso[x] >= 0 ? fstar[fso[x] + c * NN] : 0.0;
     if (c < 5 && a.mode != 0) {
       Uc[h] = a.U[((size_t)e * 5 + c) * P + id];
-      Gc[h] = a.Gk[((size_t)e * 5 + c) * P + id];
+      Gc[h] = rk_register(a, ((size_t)e * 5 + c) * P + id);
     }
   }
   __syncthreads();
@@ -616,7 +616,7 @@ __device__ __forceinline__ void volume_lat_f64(const StageArgs& a, const double*
     if (a.mode == 0) {
       a.Ut[o] = fma(-tot, iJ, src);
     } else {
-      const double gk = fma(a.A, a.Gk[o], a.clock[1] * fma(-tot, iJ, src));
+      const double gk = fma(a.A, rk_register(a, o), a.clock[1] * fma(-tot, iJ, src));
       a.Gk[o] = gk;
       a.Uw[o] = fma(a.B, gk, a.U[o]);
     }

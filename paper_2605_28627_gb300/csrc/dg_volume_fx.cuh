@@ -151,7 +151,7 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
   }
   // operands read after the sweeps, asked for in L2 now (as in volume_body)
   if (active && id < 9) {
-    if (id == 0 && a.mode == 1) l2_prefetch(a.Gk + (size_t)e * 5 * P, 5 * P * sizeof(double));
+    if (id == 0 && a.mode == 1 && a.A != 0.0) l2_prefetch(a.Gk + (size_t)e * 5 * P, 5 * P * sizeof(double));
     else if (id == 1) l2_prefetch(metrics + (size_t)e * 10 * P + 9 * P, P * sizeof(double));
     else if (id == 2 && g.source == DG_SOURCE_MMS) l2_prefetch(mms + (size_t)e * 2 * P, 2 * P * sizeof(double));
     else if (id >= 3)
@@ -457,7 +457,7 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
       const size_t o = o0 + (size_t)c * P;
-      const double gk = fma(a.A, a.Gk[o], dt * fma(-R[c], iJ, src[c]));
+      const double gk = fma(a.A, rk_register(a, o), dt * fma(-R[c], iJ, src[c]));
       a.Gk[o] = gk;
       a.Uw[o] = fma(a.B, gk, q[c]);
     }
