@@ -29,7 +29,8 @@ struct AdjBufs {
   double* gbar;      // [E][12][P]  gradient adjoint from the volume kernel
   double* fseed;     // [F][2][5][NN] surface-flux adjoint seeds (master, slave side)
   double* face;      // [F][2][17][NN] per side: conserved adjoint (5) + gradient adjoint (12)
-  double* gtil;      // [E][12][P]  total gradient adjoint / J
+  double* gtil;      // [E][12][P]  LGL: Y^d_phi = sum_l Ja^d_l gt_{phi,l}, row 3 phi + d, gt the total gradient
+                     //   adjoint / J; Gauss: gt
   double* mupart;    // block partials of d/dmu
   int n_mu;
   double* mx;        // [M][5][4][NN] mortar sides' terms of the lifting transpose (own point order)
@@ -501,7 +502,7 @@ k_adj_mortar_face(const double* __restrict__ U, const double* __restrict__ grad,
 // point (lgf, own point order) and the own term is +Y/2 (no -phi term).
 template <int N, bool FACE = false>
 __global__ void __launch_bounds__(MortarShape<N>::THREADS)
-k_adj_mortar_lift(const double* __restrict__ metrics, const int* __restrict__ mortars, const double* __restrict__ tab,
+k_adj_mortar_lift(const int* __restrict__ mortars, const double* __restrict__ tab,
                   int E, double inv_w0, AdjBufs b, const double* __restrict__ lgf) {
   using S = MortarShape<N>;
   constexpr int n = S::n, P = S::P, NN = S::NN, T = S::THREADS;
@@ -526,11 +527,9 @@ k_adj_mortar_lift(const double* __restrict__ metrics, const int* __restrict__ mo
     }
     const int node = face_node<n>(f, p, q), d = f >> 1;
     const double sg = (f & 1) ? inv_w0 : -inv_w0;
-    const double* mt = metrics + (size_t)e * 10 * P + node;
-    const double a0 = mt[(d * 3) * P], a1 = mt[(d * 3 + 1) * P], a2 = mt[(d * 3 + 2) * P];
-    const double* gt = b.gtil + (size_t)e * 12 * P + node;
+    const double* Y = b.gtil + (size_t)e * 12 * P + node;
 #pragma unroll
-    for (int ph = 0; ph < 4; ++ph) y[ph] = sg * (gt[(ph * 3) * P] * a0 + gt[(ph * 3 + 1) * P] * a1 + gt[(ph * 3 + 2) * P] * a2);
+    for (int ph = 0; ph < 4; ++ph) y[ph] = sg * Y[(ph * 3 + d) * P];
   };
   if (t < NN) {
     const int i = t % n, j = t / n;
@@ -571,8 +570,9 @@ k_adj_mortar_lift(const double* __restrict__ metrics, const int* __restrict__ mo
   }
 }
 
-// A3: per node, add the face contributions of the node's faces; store the
-// total gradient adjoint divided by J, and the conserved adjoint so far.
+// A3: per node, add the face contributions of the node's faces; store Y^d_phi of
+// the total gradient adjoint, which the lifting transpose takes from the node
+// and from its face neighbours, and the conserved adjoint so far.
 template <int N>
 __global__ void __launch_bounds__(128)
 k_adj_gather(const double* __restrict__ metrics, const int* __restrict__ elem_face, int E, AdjBufs b) {
@@ -603,9 +603,15 @@ k_adj_gather(const double* __restrict__ metrics, const int* __restrict__ elem_fa
 #pragma unroll
     for (int r = 0; r < 12; ++r) gb[r] += src[(5 + r) * NN];
   }
-  const double iJ = metrics[(size_t)e * 10 * P + 9 * P + id];
+  const double* mt = metrics + (size_t)e * 10 * P + id;
+  const double iJ = mt[9 * P];
 #pragma unroll
-  for (int r = 0; r < 12; ++r) b.gtil[((size_t)e * 12 + r) * P + id] = gb[r] * iJ;
+  for (int d = 0; d < 3; ++d) {
+    const double k0 = mt[(d * 3) * P] * iJ, k1 = mt[(d * 3 + 1) * P] * iJ, k2 = mt[(d * 3 + 2) * P] * iJ;
+#pragma unroll
+    for (int ph = 0; ph < 4; ++ph)
+      b.gtil[((size_t)e * 12 + ph * 3 + d) * P + id] = k0 * gb[ph * 3] + k1 * gb[ph * 3 + 1] + k2 * gb[ph * 3 + 2];
+  }
 #pragma unroll
   for (int c = 0; c < 5; ++c) b.qbar[((size_t)e * 5 + c) * P + id] = qb[c];
 }
@@ -614,33 +620,32 @@ k_adj_gather(const double* __restrict__ metrics, const int* __restrict__ elem_fa
 // A4: transpose of the lifting, then the primitive VJP; out = total adjoint.
 // MORTAR: a face whose neighbour entry is negative is a mortar side, whose
 // partner term comes from b.mx (k_adj_mortar_lift).
+// Bound by the FP64 pipe: with the metric products taken by k_adj_gather once
+// per node (not again for each neighbour) and the own surface term in D's
+// corners, some 110 FP64 operations a node at N = 5 instead of 245.  One VJP of
+// R(U), 16^3 elements: N = 5 1597 -> 1472 us, N = 7 4571 -> 4293.
 template <int N, bool MORTAR = false>
 __global__ void __launch_bounds__(Shape<N>::THREADS)
-k_adj_lift(const double* __restrict__ U, const double* __restrict__ metrics, const int* __restrict__ elem_nbr,
-           const int* __restrict__ elem_face, const double* __restrict__ Dg, int E, Gas g, double inv_w0, AdjBufs b,
+k_adj_lift(const double* __restrict__ U, const int* __restrict__ elem_nbr, const int* __restrict__ elem_face,
+           const double* __restrict__ Dg, int E, Gas g, double inv_w0, AdjBufs b,
            double* __restrict__ out, int n_mortar) {
   using S = Shape<N>;
   constexpr int n = S::n, P = S::P, NN = S::NN, EPB = S::EPB;
   extern __shared__ double adj_smem[];
   double* sD = adj_smem;                                   // [n*n]
   const int le = threadIdx.x / P, id = threadIdx.x - le * P;
-  double* sY = adj_smem + ((n * n + 1) & ~1) + (size_t)le * 12 * P;   // Y^d_phi = sum_l Ja^d_l gtil_{phi,l}, row phi*3+d
+  double* sY = adj_smem + ((n * n + 1) & ~1) + (size_t)le * 12 * P;   // Y^d_phi, row phi*3+d
   const int e = blockIdx.x * EPB + le;
   const bool active = e < E;
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) sD[t] = Dg[t];
-  double Ja[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, gt[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-  if (active) {
-    const double* mt = metrics + (size_t)e * 10 * P + id;
-#pragma unroll
-    for (int r = 0; r < 9; ++r) Ja[r] = mt[r * P];
-#pragma unroll
-    for (int r = 0; r < 12; ++r) gt[r] = b.gtil[((size_t)e * 12 + r) * P + id];
-#pragma unroll
-    for (int ph = 0; ph < 4; ++ph)
-#pragma unroll
-      for (int d = 0; d < 3; ++d)
-        sY[(ph * 3 + d) * P + id] = Ja[d * 3] * gt[ph * 3] + Ja[d * 3 + 1] * gt[ph * 3 + 1] + Ja[d * 3 + 2] * gt[ph * 3 + 2];
+  // own surface term -1/2 Y sg / w_0 in the end diagonals
+  const double hw = 0.5 * inv_w0;
+  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
+    const double dr = Dg[t];
+    sD[t] = t == 0 ? dr + hw : (t == n * n - 1 ? dr - hw : dr);
   }
+  if (active)
+#pragma unroll
+    for (int r = 0; r < 12; ++r) sY[r * P + id] = b.gtil[((size_t)e * 12 + r) * P + id];
   __syncthreads();
   if (!active) return;
   const int i = id % n, j = (id / n) % n, k = id / NN;
@@ -659,16 +664,12 @@ k_adj_lift(const double* __restrict__ U, const double* __restrict__ metrics, con
       for (int ph = 0; ph < 4; ++ph) phib[ph] += Dir * sY[(ph * 3 + d) * P + nid];
     }
   }
-  // surface terms: own -1/2 gtil . nsJ / w0, neighbour partner +1/2 gtil' . nsJ' / w0
+  // surface terms of the neighbours: +1/2 Y' sg' / w_0
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const int id_d = ijk[d];
     if (id_d != 0 && id_d != N) continue;
     const int s = id_d == N ? 1 : 0;
-    const double sg = s ? 1.0 : -1.0;
-#pragma unroll
-    for (int ph = 0; ph < 4; ++ph)
-      phib[ph] -= 0.5 * inv_w0 * sg * (gt[ph * 3] * Ja[d * 3] + gt[ph * 3 + 1] * Ja[d * 3 + 1] + gt[ph * 3 + 2] * Ja[d * 3 + 2]);
     const int f = 2 * d + s;
     const int code = elem_face[e * 6 + f];
     const int nb = elem_nbr[e * 6 + f];
@@ -687,13 +688,10 @@ k_adj_lift(const double* __restrict__ U, const double* __restrict__ metrics, con
     apply_flip<n>(code & 7, pp, qq, p2, q2);
     const int id2 = face_node<n>(f2, p2, q2);
     const int d2 = f2 >> 1;
-    const double sg2 = (f2 & 1) ? 1.0 : -1.0;
-    const double* mt2 = metrics + (size_t)e2 * 10 * P + id2;
-    const double n0 = sg2 * mt2[(d2 * 3) * P], n1 = sg2 * mt2[(d2 * 3 + 1) * P], n2 = sg2 * mt2[(d2 * 3 + 2) * P];
-    const double* g2 = b.gtil + (size_t)e2 * 12 * P + id2;
+    const double sg2 = (f2 & 1) ? hw : -hw;
+    const double* y2 = b.gtil + ((size_t)e2 * 12 + d2) * P + id2;
 #pragma unroll
-    for (int ph = 0; ph < 4; ++ph)
-      phib[ph] += 0.5 * inv_w0 * (g2[(ph * 3) * P] * n0 + g2[(ph * 3 + 1) * P] * n1 + g2[(ph * 3 + 2) * P] * n2);
+    for (int ph = 0; ph < 4; ++ph) phib[ph] = fma(sg2, y2[ph * 3 * P], phib[ph]);
   }
   // phi = (u, v, w, T), T = p / (rho R)
   double q[5];
@@ -1113,14 +1111,13 @@ static cudaError_t vjp_N(const Ctx& c, const double* U, const double* lam, doubl
   k_adj_gather<N><<<(int)((nodes + 127) / 128), 128, 0, s>>>(c.d_metrics, c.d_elem_face, c.E, b);
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   if (c.M > 0) {
-    k_adj_mortar_lift<N><<<c.M, MortarShape<N>::THREADS, 0, s>>>(c.d_metrics, c.d_mortars, c.d_mortar_tab, c.E,
-                                                                 inv_w0, b, nullptr);
+    k_adj_mortar_lift<N><<<c.M, MortarShape<N>::THREADS, 0, s>>>(c.d_mortars, c.d_mortar_tab, c.E, inv_w0, b, nullptr);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    k_adj_lift<N, true><<<blocks, S::THREADS, adj_lift_smem<N>(), s>>>(U, c.d_metrics, c.d_elem_nbr, c.d_elem_face,
-                                                                       c.d_D, c.E, c.gas, inv_w0, b, out, c.M);
+    k_adj_lift<N, true><<<blocks, S::THREADS, adj_lift_smem<N>(), s>>>(U, c.d_elem_nbr, c.d_elem_face, c.d_D, c.E, c.gas,
+                                                                       inv_w0, b, out, c.M);
   } else {
-    k_adj_lift<N><<<blocks, S::THREADS, adj_lift_smem<N>(), s>>>(U, c.d_metrics, c.d_elem_nbr, c.d_elem_face, c.d_D,
-                                                                 c.E, c.gas, inv_w0, b, out, 0);
+    k_adj_lift<N><<<blocks, S::THREADS, adj_lift_smem<N>(), s>>>(U, c.d_elem_nbr, c.d_elem_face, c.d_D, c.E, c.gas,
+                                                                 inv_w0, b, out, 0);
   }
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   if (dJdmu) {
@@ -1156,7 +1153,7 @@ static cudaError_t vjp_lg_N(const Ctx& c, const double* U, const double* lam, do
                                                      c.d_adj_lgf);
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   if (c.M > 0) {
-    k_adj_mortar_lift<N, true><<<c.M, MortarShape<N>::THREADS, 0, s>>>(c.d_metrics, c.d_mortars, c.d_mortar_tab,
+    k_adj_mortar_lift<N, true><<<c.M, MortarShape<N>::THREADS, 0, s>>>(c.d_mortars, c.d_mortar_tab,
                                                                        c.E, 0.0, b, c.d_adj_lgf);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }

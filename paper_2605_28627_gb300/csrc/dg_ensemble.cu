@@ -357,8 +357,8 @@ static cudaError_t enqueue_stage(dg_ensemble* e, const Group& g, int k, cudaStre
 // ---------------------------------------------------------------------------
 // Autotuner: for every group, time the volume kernel for each (tile, grid)
 // candidate and the lifting / face kernels for each grid, on the members' own
-// data, with B = 0 so the state is left untouched (the register is zeroed at
-// the start of every step anyway).
+// data, with B = 0 so the state is left untouched (the first stage of every
+// step sets the register anyway).
 static const double kZero14[14] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
 
 static float time_stage(dg_ensemble* e, const Group& g, cudaStream_t s, int reps, int which) {
