@@ -103,12 +103,20 @@ def step_flops_per_dof(N):
 
 # ---------------------------------------------------------------------------
 # Algorithmic DRAM bytes per node and stage of the FP32-operator volume kernel
-# (HBM-bound): FP64 state U and register G read and written (160 B), FP32
+# (HBM-bound): FP64 state U and register G read and written (160 B; a step's
+# first stage does not read G), FP32
 # metric terms J a^d and 1/J (40 B), FP32 lifted gradients (48 B), the
 # manufactured source's phases (16 B, FP64) and the six faces' FP32 fluxes
 # F* (6 (N+1)^2 points x 20 B per element = 120/(N+1) B per node).
 def fp32_volume_bytes_per_dof(N, mms=True):
     return 160.0 + 40.0 + 48.0 + (16.0 if mms else 0.0) + 120.0 / (N + 1)
+
+
+# The same for the FP64 volume kernel: state and register (160 B), fixed-point
+# metric terms and FP64 1/J (80 B), FP64 gradients (96 B), phases (16 B), face
+# fluxes (240/(N+1) B).
+def fp64_volume_bytes_per_dof(N, mms=True):
+    return 160.0 + 80.0 + 96.0 + (16.0 if mms else 0.0) + 240.0 / (N + 1)
 
 
 def hbm_peak_gbs():
@@ -978,9 +986,9 @@ def run_adjoint(args, local):
     fp64_peak, _ = dg.probe_peaks(local)
     dof = s.E * (N + 1) ** 3
     adj_flops = adjoint_volume_flops_per_dof(N) * dof
-    adj_roof = {"bound": "alu", "unit": "TFLOP/s", "peak": fp64_peak,
+    adj_roof = {"bound": "alu (FP64 pipe and, for the two-point terms, integer multiplier)", "unit": "TFLOP/s", "peak": fp64_peak,
                 "achieved_lower_bound": adj_flops / (ms_vjp * 1e-3) / 1e12,
-                "frac_lower_bound": adj_flops / (ms_vjp * 1e-3) / 1e12 / fp64_peak,
+                "ratio_lower_bound": adj_flops / (ms_vjp * 1e-3) / 1e12 / fp64_peak,
                 "algorithmic_flops_per_dof": adjoint_volume_flops_per_dof(N),
                 "note": "the adjoint volume kernel's algorithmic FP64 count over the time of the whole VJP call "
                         "(volume, face, gather and lifting adjoint kernels): a lower bound of the volume "
@@ -1163,20 +1171,29 @@ def main():
     fp64_peak, fp32_peak = dg.probe_peaks(local)
     vol_flops = volume_flops_per_dof(N) * dof
     achieved = vol_flops / (ms3[2] * 1e-3) / 1e12
-    roofline = {"bound": "alu", "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
-                "frac": achieved / fp64_peak, "traffic": MEASURED_TRAFFIC.get((N, "fp64")),
+    # the arithmetic runs as 64-bit integer products beside the FP64 pipe, so the
+    # roof is the memory's, and the rate by the FP64 statement's flops is given
+    # against the FP64 pipe as a figure that may exceed 1
+    hbm_peak, hbm_src = hbm_peak_gbs()
+    vol_gbs = fp64_volume_bytes_per_dof(N) * dof / (ms3[2] * 1e-3) / 1e9
+    roofline = {"bound": "hbm", "achieved": vol_gbs, "peak": hbm_peak, "unit": "GB/s", "frac": vol_gbs / hbm_peak,
+                "traffic": MEASURED_TRAFFIC.get((N, "fp64")),
                 "kernel": "k_volume2<%d> (split-form volume + surface + Jacobian + LSERK update)" % N,
-                "peak_source": "measured FP64 DFMA chain throughput on this GPU (dg_probe_peaks)",
+                "peak_source": hbm_src,
+                "limited_by": "integer multiplier and issue slots (block fixed point), not HBM",
+                "fp64_equivalent": {"tflops": achieved, "fp64_pipe_tflops": fp64_peak, "ratio": achieved / fp64_peak,
+                                    "peak_source": "measured FP64 DFMA chain throughput on this GPU (dg_probe_peaks)"},
                 "stage_ms": {"lift": ms3[0], "face": ms3[1], "volume": ms3[2]}}
     # the whole stage (lifting, face fluxes, volume) by the same count
     stage_tf = step_flops_per_dof(N) * dof / (sum(ms3) * 1e-3) / 1e12
     roofline["stage"] = {
-        "achieved": stage_tf, "frac": stage_tf / fp64_peak,
+        "fp64_equivalent_tflops": stage_tf, "ratio_to_fp64_pipe": stage_tf / fp64_peak,
         "algorithmic_flops_per_dof": {"lift": lift_flops_per_dof(N), "face": face_flops_per_dof(N),
                                       "volume": volume_flops_per_dof(N)},
-        "kernel_frac": {"lift": lift_flops_per_dof(N) * dof / (ms3[0] * 1e-3) / 1e12 / fp64_peak,
-                        "face": face_flops_per_dof(N) * dof / (ms3[1] * 1e-3) / 1e12 / fp64_peak,
-                        "volume": achieved / fp64_peak}}
+        "kernel_ratio_to_fp64_pipe": {
+            "lift": lift_flops_per_dof(N) * dof / (ms3[0] * 1e-3) / 1e12 / fp64_peak,
+            "face": face_flops_per_dof(N) * dof / (ms3[1] * 1e-3) / 1e12 / fp64_peak,
+            "volume": achieved / fp64_peak}}
 
     # end to end through the C ABI with host buffers (pinned)
     host = U0.cpu().pin_memory()
@@ -1191,7 +1208,6 @@ def main():
     e2e = {"value": world * dof * 5 * args.steps / el, "unit": UNIT, "h2d_bytes_per_step": nb,
            "d2h_bytes_per_step": nb}
 
-    hbm_peak, hbm_src = hbm_peak_gbs()
     fp32 = fp32_operator_rate(dg, N, local, prm, U0, args.steps, value / world, hbm_peak, hbm_src) \
         if rank == 0 else None
     tgv_small = small_tgv_rate(dg, local) if rank == 0 else None
@@ -1205,13 +1221,13 @@ def main():
             dofs = K_ELEMS ** 3 * (Ns + 1) ** 3
             if Ns == N:
                 sweep[str(Ns)] = {"dof_stage_per_s": value / world, "pid_ns": 1e9 * world / value,
-                                  "volume_ms": ms3[2], "volume_roofline_frac": roofline["frac"]}
+                                  "volume_ms": ms3[2], "volume_ratio_to_fp64_pipe": achieved / fp64_peak}
             else:
                 ms, ms3n = sweep_rate(dg, Ns, local, prm)
-                # roofline of the volume kernel at this N: algorithmic FP64 flops / its event time
+                # the volume kernel at this N: algorithmic FP64 flops / its event time
                 ach = volume_flops_per_dof(Ns) * dofs / (ms3n[2] * 1e-3) / 1e12
                 sweep[str(Ns)] = {"dof_stage_per_s": dofs * 5 / (ms * 1e-3), "pid_ns": ms * 1e6 / (dofs * 5),
-                                  "volume_ms": ms3n[2], "volume_roofline_frac": ach / fp64_peak}
+                                  "volume_ms": ms3n[2], "volume_ratio_to_fp64_pipe": ach / fp64_peak}
             sweep[str(Ns)]["volume_traffic"] = MEASURED_TRAFFIC.get((Ns, "fp64"))
             sweep[str(Ns)]["fp32op_volume_traffic"] = MEASURED_TRAFFIC.get((Ns, "fp32op"))
             # the FP32-operator path on the same mesh and state, and its
