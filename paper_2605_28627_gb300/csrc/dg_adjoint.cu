@@ -1024,6 +1024,26 @@ __global__ void k_axpby(double* y, const double* x, double a, double b, size_t l
     y[t] = (a == 0.0 ? 0.0 : a * y[t]) + b * x[t];
 }
 
+// Between two VJPs of the step's reverse sweep, one pass over the state: the
+// finished stage's VJP into lam, the register's adjoint to the next stage, and
+// the next VJP's cotangent dt Gb.  With this for four launches and a memset, and
+// without the last stage's forward evaluation, a step on Gauss nodes (12^3, N = 3)
+// went from 2405 to 2181 us.
+__global__ void k_adj_stage(double* __restrict__ Gb, double* __restrict__ lam, double* __restrict__ tmp, double A,
+                            double B, double dt, bool first, size_t len) {
+  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < len; t += (size_t)gridDim.x * blockDim.x) {
+    double l = lam[t], g = 0.0;
+    if (!first) {
+      l += tmp[t];
+      lam[t] = l;
+      g = A * Gb[t];
+    }
+    g = fma(B, l, g);
+    Gb[t] = g;
+    tmp[t] = dt * g;
+  }
+}
+
 template <int N>
 static size_t adj_volume_smem() {
   using S = Shape<N>;
@@ -1268,6 +1288,13 @@ cudaError_t launch_kinetic(const Ctx& c, const double* U, double* grad, double* 
 cudaError_t launch_axpby(double* y, const double* x, double a, double b, size_t len, cudaStream_t s) {
   const size_t blocks = std::min<size_t>((len + 255) / 256, 152 * 16);
   k_axpby<<<(unsigned)blocks, 256, 0, s>>>(y, x, a, b, len);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_adj_stage(double* Gb, double* lam, double* tmp, double A, double B, double dt, bool first, size_t len,
+                             cudaStream_t s) {
+  const size_t blocks = std::min<size_t>((len + 255) / 256, 152 * 16);
+  k_adj_stage<<<(unsigned)blocks, 256, 0, s>>>(Gb, lam, tmp, A, B, dt, first, len);
   return cudaGetLastError();
 }
 

@@ -45,7 +45,7 @@ static dg_status ensure_adjoint(Ctx* c) {
   ADJ_CUDA(cudaMalloc(&c->d_adj_fseed, sizeof(double) * nn * 2 * 5), c, "adjoint buffers");
   ADJ_CUDA(cudaMalloc(&c->d_adj_face, sizeof(double) * nn * 2 * 17), c, "adjoint buffers");
   ADJ_CUDA(cudaMalloc(&c->d_adj_mu, sizeof(double) * (adjoint_mu_partials(*c) + 2)), c, "adjoint buffers");
-  ADJ_CUDA(cudaMalloc(&c->d_adj_stage, sizeof(double) * st * rk_scheme(c->prm.rk_scheme).stages), c,
+  ADJ_CUDA(cudaMalloc(&c->d_adj_stage, sizeof(double) * st * (rk_scheme(c->prm.rk_scheme).stages - 1)), c,
            "adjoint stage states");
   ADJ_CUDA(cudaMalloc(&c->d_adj_work, sizeof(double) * st * 4), c, "adjoint work");
   if (c->M > 0)
@@ -61,30 +61,27 @@ static dg_status ensure_adjoint(Ctx* c) {
 static dg_status step_adjoint(Ctx* c, const double* Un, double* lam, double* dJdmu, double t, double dt,
                               cudaStream_t s) {
   const RkScheme rk = rk_scheme(c->prm.rk_scheme);
-  const size_t st = (size_t)c->E * 5 * c->P, bytes = sizeof(double) * st;
-  double* Ws = c->d_adj_work;           // work state
-  double* G = Ws + st;                  // RK register
+  const size_t st = (size_t)c->E * 5 * c->P;
+  double* G = c->d_adj_work + st;       // RK register
   double* Gb = G + st;                  // adjoint of the register
   double* tmp = Gb + st;                // dt * Gb, then VJP output
-  // forward recomputation of the stage states
-  ADJ_CUDA(cudaMemcpyAsync(Ws, Un, bytes, cudaMemcpyDeviceToDevice, s), c, "stage copy");
+  // stage states: the step's start state (not written), then each stage by the
+  // last one's volume kernel
+  auto state = [&](int k) { return k == 0 ? Un : c->d_adj_stage + (size_t)(k - 1) * st; };
   ADJ_CUDA(launch_set_clock(c->d_clock, t, dt, s), c, "clock");
-  for (int k = 0; k < rk.stages; ++k) {
-    ADJ_CUDA(cudaMemcpyAsync(c->d_adj_stage + (size_t)k * st, Ws, bytes, cudaMemcpyDeviceToDevice, s), c, "stage copy");
-    ADJ_CUDA(launch_lift(*c, Ws, s), c, "lift");
-    ADJ_CUDA(launch_face(*c, Ws, s), c, "face");
-    StageArgs a{Ws, Ws, G, nullptr, c->d_clock, rk.C[k], rk.A[k], rk.B[k], 1};
+  for (int k = 0; k + 1 < rk.stages; ++k) {
+    ADJ_CUDA(launch_lift(*c, state(k), s), c, "lift");
+    ADJ_CUDA(launch_face(*c, state(k), s), c, "face");
+    StageArgs a{state(k), c->d_adj_stage + (size_t)k * st, G, nullptr, c->d_clock, rk.C[k], rk.A[k], rk.B[k], 1};
     ADJ_CUDA(launch_volume(*c, a, s), c, "volume");
   }
   // reverse sweep: Gb += B_k lam;  lam += (dR/dU)^T (dt Gb);  Gb *= A_k
-  ADJ_CUDA(cudaMemsetAsync(Gb, 0, bytes, s), c, "memset");
   for (int k = rk.stages - 1; k >= 0; --k) {
-    ADJ_CUDA(launch_axpby(Gb, lam, 1.0, rk.B[k], st, s), c, "axpby");
-    ADJ_CUDA(launch_axpby(tmp, Gb, 0.0, dt, st, s), c, "axpby");
-    ADJ_CUDA(launch_vjp(*c, c->d_adj_stage + (size_t)k * st, tmp, tmp, dJdmu, 1.0, s), c, "vjp");
-    ADJ_CUDA(launch_axpby(lam, tmp, 1.0, 1.0, st, s), c, "axpby");
-    ADJ_CUDA(launch_axpby(Gb, Gb, rk.A[k], 0.0, st, s), c, "axpby");
+    const bool first = k == rk.stages - 1;
+    ADJ_CUDA(launch_adj_stage(Gb, lam, tmp, first ? 0.0 : rk.A[k + 1], rk.B[k], dt, first, st, s), c, "stage adjoint");
+    ADJ_CUDA(launch_vjp(*c, state(k), tmp, tmp, dJdmu, 1.0, s), c, "vjp");
   }
+  ADJ_CUDA(launch_axpby(lam, tmp, 1.0, 1.0, st, s), c, "axpby");
   return DG_OK;
 }
 
@@ -208,11 +205,7 @@ struct DeviceCheckpoints {
     ADJ_CUDA(cudaMemcpyAsync(W, snap[slot], bytes(), cudaMemcpyDeviceToDevice, s), c, "copy");
     dg_status st = advance(c, W, reg(), t0 + i0 * dt, dt, i - i0, s);
     if (st != DG_OK) return st;
-    // the step adjoint overwrites the work area, so it starts from a copy in
-    // stage slot 4, which it reads first and rewrites only at its fifth stage
-    double* keep = c->d_adj_stage + (size_t)4 * c->E * 5 * c->P;
-    ADJ_CUDA(cudaMemcpyAsync(keep, W, bytes(), cudaMemcpyDeviceToDevice, s), c, "copy");
-    return step_adjoint(c, keep, lam, dJdmu, t0 + i * dt, dt, s);
+    return step_adjoint(c, W, lam, dJdmu, t0 + i * dt, dt, s);
   }
 };
 

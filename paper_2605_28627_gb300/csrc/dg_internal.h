@@ -172,10 +172,10 @@ struct Ctx {
   double* d_adj_fseed = nullptr; // [F][2][5][NN]
   double* d_adj_face = nullptr;  // [F][2][17][NN]
   double* d_adj_mu = nullptr;    // block partials of d/dmu
-  double* d_adj_stage = nullptr; // [5][E][5][P] stage states of one step
+  double* d_adj_stage = nullptr; // [stages - 1][E][5][P] stage states of one step after its start state
   double* d_adj_mx = nullptr;    // [M][5][4][NN] mortar sides' lifting-transpose terms
   double* d_adj_lgf = nullptr;   // [E][6][9][NN] Gauss nodes: lifting surface sums, face-value adjoints
-  double* d_adj_work = nullptr;  // [4][E][5][P]: work state, G, G-bar, VJP scratch
+  double* d_adj_work = nullptr;  // [4][E][5][P]: recomputed state of a solve, G, G-bar, VJP scratch
   // host-buffer path
   double* d_U = nullptr;
   double* d_G = nullptr;
@@ -262,6 +262,8 @@ int adjoint_mu_partials(const Ctx& c);
 cudaError_t launch_vjp(const Ctx& c, const double* U, const double* lam, double* out, double* dJdmu, double mu_scale,
                        cudaStream_t s);
 cudaError_t launch_axpby(double* y, const double* x, double a, double b, size_t len, cudaStream_t s);
+cudaError_t launch_adj_stage(double* Gb, double* lam, double* tmp, double A, double B, double dt, bool first, size_t len,
+                             cudaStream_t s);
 cudaError_t launch_kinetic(const Ctx& c, const double* U, double* grad, double* d_out, cudaStream_t s);
 constexpr int kRedValues = 9;
 
