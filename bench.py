@@ -46,12 +46,12 @@ def build_mesh(N):
 # DRAM bytes (read + write) per launch of the volume kernel on this workload,
 # the median over the launches of one ncu capture of the current kernels
 # (profiles/volume_traffic_N7_mms16.txt); absent = not captured.
-MEASURED_TRAFFIC = {(7, "fp64"): 670.667520e6 + 217.116672e6, (7, "fp32op"): 406.712064e6 + 143.888640e6}
+MEASURED_TRAFFIC = {(7, "fp64"): 581.094656e6 + 231.395712e6, (7, "fp32op"): 406.712064e6 + 143.888640e6}
 # The other orders of the sweep, DRAM read + write per launch (medians, MB) from one capture of
 # the volume kernels of `--sweep 1,2,3,4,5,6,8,9`; up to N = 4 the working set stays in the
 # 129 MB L2 between launches, so DRAM sees less than the kernel's algorithmic bytes.
-for _N, _f64, _f32 in ((1, 11.0, 7.1), (2, 34.7, 22.7), (3, 79.7, 52.3), (4, 165.9, 102.6), (5, 302.5, 203.7),
-                       (6, 499.7, 344.3), (8, 1084.3, 800.5), (9, 1765.2, 1067.8)):
+for _N, _f64, _f32 in ((1, 11.6, 7.1), (2, 37.8, 22.7), (3, 79.7, 52.3), (4, 168.7, 104.1), (5, 306.8, 204.1),
+                       (6, 497.5, 344.9), (8, 1071.0, 799.7), (9, 1732.3, 1066.5)):
     MEASURED_TRAFFIC[(_N, "fp64")] = _f64 * 1e6
     MEASURED_TRAFFIC[(_N, "fp32op")] = _f32 * 1e6
 

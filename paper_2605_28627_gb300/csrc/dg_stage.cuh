@@ -60,10 +60,9 @@ struct VShape : Shape<N, EPB_> {
 // budget must allow.  FP32 (latency-bound): enough for about 32 warps per SM at
 // N <= 5 (+8 to +16 % at N = 2, 4, 5 over two blocks; 48 warps lost 6 to 23 %
 // there), 33 to 48 at N = 6..8, where a hundred-odd bytes of spilled registers
-// per thread pay.  FP64 at N = 6, 7: two -- a hundred-odd bytes of spilled
-// registers cost less than an SM with only 11 or 16 warps to feed its FP64
-// pipe from (+2.4 % at N = 6, +0.5 % at N = 7; at N = 4, 5 a third block did
-// not pay).
+// per thread pay.  FP64: only the shared-memory budget of this body, which runs
+// for the elements out of the fixed-point range (the kernel's registers follow
+// fx_min_blocks).
 template <int N, typename R>
 constexpr int vol_min_blocks() {
   constexpr int threads = Shape<N>::THREADS;
