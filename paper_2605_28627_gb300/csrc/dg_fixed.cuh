@@ -457,4 +457,27 @@ DG_HD void fx_pair(i64 ra, i64 rb, i64 ba, i64 bb, i64 su0, i64 su1, i64 su2, i6
   F[4] = (ea >> al.se1) + (fx_end<3>(b) >> al.se2);
 }
 
+// Lifting on LGL nodes.  Line sum D phi + jump of a field with exponent e (D and
+// the jump factor with 60 - e_D bits, fields with 60 - e): 60 - e - e_D bits,
+// below 2^62.1 for N <= 9.  Gradient component (1/J) sum_d Ja^d dd_d: the sum,
+// with metric terms of 60 - e_j bits, has 58 - e - e_D - e_j bits and stays
+// below 2^61.6, its product with 1/J (62 - e_i) 58 - e - e_D - e_j - e_i.  The
+// shifts fill the words: with 3 bits less (as the bound of the single factors
+// leaves) the products' rounding was up to 3 times the FP64 kernel's at N = 7.
+constexpr int kFxUpLift = kFxUpD + 2;
+DG_HD FxSum fx_lift_start(i64 jump) { return FxSum{jump, (i64)1 << (31 - kFxUpLift)}; }
+DG_HD i64 fx_lift_line(const FxSum& s) { return fx_end<kFxUpLift>(s); }
+DG_HD int fx_lift_bits(int eD, int ej, int ei) { return 58 - eD - ej - ei; }   // less e
+DG_HD i64 fx_lift_gradient(const Fx J[3], const Fx dd[3], Fx iJ) {
+  FxSum s = fx_zero<2>();
+  fx_add(s, J[0], dd[0]);
+  fx_add(s, J[1], dd[1]);
+  fx_add(s, J[2], dd[2]);
+  return fx_mul<2>(fx_split(fx_end<2>(s)), iJ);
+}
+
+// Weak lifting: line sums of n + 2 products of 60 bits, shifted up so that the
+// three directions' sum (59 - e - e_D - e_j bits) stays below 2^61.8 for N <= 9.
+constexpr int kFxUpWeak = kFxUpD + 1;
+
 }  // namespace dg

@@ -123,11 +123,11 @@ __device__ __forceinline__ bool lift_lg_fx(const double* __restrict__ U, const d
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int l = 0; l < 3; ++l) s[(a * 3 + l) * NN] = fx_mul<1>(st[a], ns[l]);   // 59 - e - e_j
+        for (int l = 0; l < 3; ++l) s[(a * 3 + l) * NN] = fx_mul<2>(st[a], ns[l]);   // 60 - e - e_j
     }
   }
   const int i = id % n, j = (id / n) % n, k = id / NN;
-  i64 acc[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};   // 57 - e - e_j - e_D, below 2^61
+  i64 acc[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};   // 59 - e - e_j - e_D, below 2^62
 #pragma unroll 1
   for (int d = 0; d < 3; ++d) {
     __syncthreads();
@@ -136,9 +136,9 @@ __device__ __forceinline__ bool lift_lg_fx(const double* __restrict__ U, const d
                J2 = fx_split(d == 0 ? Ja[2] : (d == 1 ? Ja[5] : Ja[8]));
 #pragma unroll
       for (int a = 0; a < 4; ++a) {   // negated: the volume term enters with a minus sign
-        sprod[(a * 3) * P + id] = -fx_mul<1>(X[a], J0);
-        sprod[(a * 3 + 1) * P + id] = -fx_mul<1>(X[a], J1);
-        sprod[(a * 3 + 2) * P + id] = -fx_mul<1>(X[a], J2);
+        sprod[(a * 3) * P + id] = -fx_mul<2>(X[a], J0);
+        sprod[(a * 3 + 1) * P + id] = -fx_mul<2>(X[a], J1);
+        sprod[(a * 3 + 2) * P + id] = -fx_mul<2>(X[a], J2);
       }
     }
     __syncthreads();
@@ -151,24 +151,24 @@ __device__ __forceinline__ bool lift_lg_fx(const double* __restrict__ U, const d
       const i64* f0 = sS + (2 * d) * 12 * NN + pq;
 #pragma unroll
       for (int al = 0; al < 12; ++al) {
-        FxSum s = fx_zero<kFxUpD>();
+        FxSum s = fx_zero<kFxUpWeak>();
         const i64* line = sprod + al * P + line0;
 #pragma unroll
         for (int m = 0; m < n; ++m) fx_add(s, Dr[m], fx_split(line[m * stride]));
         fx_add(s, t0, fx_split(f0[al * NN]));
         fx_add(s, t1, fx_split(f0[(12 + al) * NN]));
-        acc[al] += fx_end<kFxUpD>(s);
+        acc[al] += fx_end<kFxUpWeak>(s);
       }
     }
   }
   __syncthreads();   // every thread is done with sprod
-  const int qg = 57 + 62 - 64 - (int)ej.x - eD - (int)ej.z;   // less e
+  const int qg = 59 + 62 - 64 + 1 - (int)ej.x - eD - (int)ej.z;   // less e
   if (act) {
     double* go = grad + (size_t)e * 12 * P + id;
     const Fx iJx = fx_split(iJ);
 #pragma unroll
     for (int al = 0; al < 12; ++al) {
-      const i64 G = fx_mul<0>(fx_split(acc[al]), iJx);   // below 2^59
+      const i64 G = fx_mul<1>(fx_split(acc[al]), iJx);   // below 2^61
       go[al * P] = fx_to(G, qg - (al < 9 ? eu : et));
       sprod[al * P + id] = G;
     }
@@ -184,10 +184,13 @@ __device__ __forceinline__ bool lift_lg_fx(const double* __restrict__ U, const d
     const Fx* l = sT + (2 + (f & 1)) * n;
     const int stride = d == 0 ? 1 : (d == 1 ? n : NN);
     const i64* line = sprod + al * P + line_node<n>(d, 0, p, q);
-    FxSum s = fx_zero<3>();
+    FxSum s = fx_zero<4>();
 #pragma unroll
-    for (int m = 0; m < n; ++m) fx_add(s, l[m], fx_split(line[m * stride]));
-    gf[((size_t)e * 6 + f) * 12 * NN + (size_t)al * NN + pq] = fx_to(fx_end<3>(s), qg + 59 - 64 + 3 - (al < 9 ? eu : et));
+    for (int m = 0; m < n; ++m) {
+      if (n > 5 && m == n / 2) fx_fold(s);   // five terms fill c
+      fx_add(s, l[m], fx_split(line[m * stride]));
+    }
+    gf[((size_t)e * 6 + f) * 12 * NN + (size_t)al * NN + pq] = fx_to(fx_end<4>(s), qg + 59 - 64 + 4 - (al < 9 ? eu : et));
   }
   return bad;
 }
@@ -286,14 +289,16 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
   const int ej = (int)ejv.x, em = fx_expo(fx_mag(g.mu)), el = fx_expo(fx_mag(g.mu * g.kappa));
   const bool act = active && top < 90 && ej < 90;
   if (id == 0) state[le] = active ? (act ? 1 : 2) : 0;
-  // bits after the point of the mass (q0), momentum (qm + 1) and energy (qe)
-  // fluxes: below 2^59.7, so that the n + 2 terms of a line fit in FxSum
-  const int n0 = 60 - x[kR] - x[kU] - ej;                                             // rho {u . Ja}
-  const int n1 = 58 - x[kR] - 2 * x[kU] - ej, n2 = 58 - x[kP] - ej, n3 = 58 - x[kG] - em - ej;
-  const int qm = min(min(n1, n2) - 1, min(n3 - 2, 58 - x[kFm]));
-  const int n4 = 59 - x[kH] - x[kU] - ej, n5 = 57 - x[kG] - em - ej - x[kU], n6 = 60 - x[kT] - el - ej;
-  const int qe = min(min(n4, n5) - 1, min(n6 - 2, 59 - x[kFe]));
-  const int q0 = min(n0 - 1, 58 - x[kF0]);
+  // bits after the point of the mass (q0), momentum (qm) and energy (qe) fluxes:
+  // below 2^61.3, so that six of a line's n + 2 terms fit in FxSum's c (the part of
+  // the products that fx_add leaves out is the sums' largest error, and a bit
+  // more in the factors halves it)
+  const int n0 = 61 - x[kR] - x[kU] - ej;                                             // rho {u . Ja}
+  const int n1 = 61 - x[kR] - 2 * x[kU] - ej, n2 = 60 - x[kP] - ej, n3 = 59 - x[kG] - em - ej;
+  const int qm = min(min(n1 - 1, n2), min(n3 - 2, 60 - x[kFm]));
+  const int n4 = 60 - x[kH] - x[kU] - ej, n5 = n3 - 2 - x[kU], n6 = 60 - x[kT] - el - ej;
+  const int qe = min(min(n4, n5 - 1), min(n6 - 1, 60 - x[kFe]));
+  const int q0 = min(n0, 60 - x[kF0]);
   if (act) {
     const Fx U[3] = {fx_split(fx_from(u, 62 - x[kU])), fx_split(fx_from(v, 62 - x[kU])), fx_split(fx_from(w, 62 - x[kU]))};
     const Fx rho = fx_split(fx_from(q[0], 62 - x[kR])), H = fx_split(fx_from(q[4] + p, 62 - x[kH]));
@@ -318,31 +323,31 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
       FxSum s = fx_zero<3>();
       fx_add(s, U[0], J[0]); fx_add(s, U[1], J[1]); fx_add(s, U[2], J[2]);
       const Fx un = fx_split(fx_end<3>(s));                 // 61 - e_u - e_j
-      const i64 f0 = fx_mul<1>(rho, un);                    // n0
+      const i64 f0 = fx_mul<2>(rho, un);                    // n0
       const Fx X = fx_split(f0 >> fx_clamp(n1 - qm));
       FxSum w0 = fx_zero<4>(), w1 = fx_zero<4>(), w2 = fx_zero<4>();
       fx_add(w0, t00, J[0]); fx_add(w0, t01, J[1]); fx_add(w0, t02, J[2]);
       fx_add(w1, t01, J[0]); fx_add(w1, t11, J[1]); fx_add(w1, t12, J[2]);
       fx_add(w2, t02, J[0]); fx_add(w2, t12, J[1]); fx_add(w2, t22, J[2]);
-      const i64 V[3] = {fx_end<4>(w0), fx_end<4>(w1), fx_end<4>(w2)};   // n3 + 1
+      const i64 V[3] = {fx_end<4>(w0), fx_end<4>(w1), fx_end<4>(w2)};   // n3
       sF[(d * 5) * P + id] = -(f0 >> fx_clamp(n0 - q0));
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        FxSum mo = fx_zero<1>();
+        FxSum mo = fx_zero<2>();
         fx_add(mo, X, U[c]);
         fx_add(mo, Pp, J[c]);
-        sF[(d * 5 + 1 + c) * P + id] = (V[c] >> fx_clamp(n3 - qm)) - fx_end<1>(mo);   // qm + 1
+        sF[(d * 5 + 1 + c) * P + id] = (V[c] >> fx_clamp(n3 - qm)) - fx_end<2>(mo);
       }
       FxSum en = fx_zero<0>(), h = fx_zero<4>();
       fx_add(en, fx_split(V[0]), U[0]); fx_add(en, fx_split(V[1]), U[1]); fx_add(en, fx_split(V[2]), U[2]);
       fx_add(h, T[0], J[0]); fx_add(h, T[1], J[1]); fx_add(h, T[2], J[2]);
       sF[(d * 5 + 4) * P + id] = (fx_end<0>(en) >> fx_clamp(n5 - qe)) + (fx_end<4>(h) >> fx_clamp(n6 - qe)) -
-                                 (fx_mul<0>(H, un) >> fx_clamp(n4 - qe));
+                                 (fx_mul<1>(H, un) >> fx_clamp(n4 - qe));
     }
     for (int o = id; o < 30 * NN; o += P) {
       const int v2 = (o / NN) % 5;
       i64* s = sFs + o;
-      *s = fx_from(__longlong_as_double(*s), v2 == 0 ? q0 : (v2 == 4 ? qe : qm + 1));
+      *s = fx_from(__longlong_as_double(*s), v2 == 0 ? q0 : (v2 == 4 ? qe : qm));
     }
   }
   __syncthreads();
@@ -364,7 +369,10 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
       FxSum s = fx_zero<kFxUpD>();
       const i64* line = sF + (d * 5 + c) * P + line0;
 #pragma unroll
-      for (int m = 0; m < n; ++m) fx_add(s, Dr[m], fx_split(line[m * stride]));
+      for (int m = 0; m < n; ++m) {
+        if (n + 2 > 6 && m == (n + 2) / 2) fx_fold(s);
+        fx_add(s, Dr[m], fx_split(line[m * stride]));
+      }
       fx_add(s, t0, fx_split(sFs[(2 * d * 5 + c) * NN + pq]));
       fx_add(s, t1, fx_split(sFs[((2 * d + 1) * 5 + c) * NN + pq]));
       acc[c] += fx_end<kFxUpD>(s);
@@ -377,7 +385,7 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
     const size_t o = o0 + (size_t)c * P;
-    const double R = fma(-fx_to(acc[c], (c == 0 ? q0 : (c == 4 ? qe : qm + 1)) - 2 - eD), iJ, src[c]);
+    const double R = fma(-fx_to(acc[c], (c == 0 ? q0 : (c == 4 ? qe : qm)) - 2 - eD), iJ, src[c]);
     if (a.mode == 0) {
       a.Ut[o] = R;
     } else {

@@ -48,8 +48,9 @@ struct LatShape {
 // The threads of direction 0 evaluate the node's phi while the others evaluate
 // the neighbours' at the face points; the jump (phi_nbr - phi) h, h = +-1/(2
 // w_0), goes into the line sum, its own part through D's corners (D_00 + 1/(2
-// w_0) = 0 there up to rounding).  Bound by the memory latency of its two
-// dependent loads and by some 50 FP64 instructions a warp.
+// w_0) = 0 there up to rounding), the neighbour's by a fused multiply-add.  Bound
+// by the memory latency of its two dependent loads and by some 50 FP64
+// instructions a warp.
 template <int N>
 constexpr size_t lift_lat_smem_bytes() {
   constexpr int P = LatShape<N>::P, NN = LatShape<N>::NN;
@@ -66,7 +67,7 @@ k_lift_lat(const double* __restrict__ U_, const double* __restrict__ metrics, co
   __shared__ double sD[n * n];
   extern __shared__ __align__(16) unsigned char lat_raw[];
   double* sphi = reinterpret_cast<double*>(lat_raw);   // [4][P]
-  double* snb = sphi + 4 * P;                          // [6][4][NN] h phi_nbr
+  double* snb = sphi + 4 * P;                          // [6][4][NN] phi_nbr
   double* sdd = snb + 24 * NN;                         // [4][3][P]: D_d phi_a + jump_d
   const int d = threadIdx.x / P, id = threadIdx.x - d * P;
   const int e = blockIdx.x;
@@ -74,14 +75,14 @@ k_lift_lat(const double* __restrict__ U_, const double* __restrict__ metrics, co
   const double* mt = metrics + (size_t)e * 10 * P + id;
   const double J0 = mt[(0 * 3 + d) * P], J1 = mt[(1 * 3 + d) * P], J2 = mt[(2 * 3 + d) * P];
   const double iJ = mt[9 * P];
-  auto lifted = [&](const double* q, double scale, double* out, int pitch) {
+  auto lifted = [&](const double* q, double* out, int pitch) {
     const double rho = q[0], m0 = q[P], m1 = q[2 * P], m2 = q[3 * P], en = q[4 * P], ir = rcp_op(rho);
     const double u = m0 * ir, v = m1 * ir, w = m2 * ir;
     const double T = g.gm1 * (en - 0.5 * (m0 * u + m1 * v + m2 * w)) * ir * g.inv_R;
-    out[0] = scale * u;
-    out[pitch] = scale * v;
-    out[2 * pitch] = scale * w;
-    out[3 * pitch] = scale * T;
+    out[0] = u;
+    out[pitch] = v;
+    out[2 * pitch] = w;
+    out[3 * pitch] = T;
   };
   constexpr int NI = (NF + 2 * P - 1) / (2 * P);   // face points of a thread of directions 1 and 2
   int nbr[NI] = {};
@@ -104,14 +105,14 @@ k_lift_lat(const double* __restrict__ U_, const double* __restrict__ metrics, co
   wait_previous();
   const double* U = after_previous(U_);
   if (d == 0) {
-    lifted(U + (size_t)e * 5 * P + id, 1.0, sphi + id, P);
+    lifted(U + (size_t)e * 5 * P + id, sphi + id, P);
   } else {
 #pragma unroll
     for (int x = 0; x < NI; ++x) {
       const int t = threadIdx.x - P + x * 2 * P;
       if (t >= NF) break;
       const int f = t / NN, pq = t - f * NN;
-      lifted(U + nbr[x], (f & 1) ? hw : -hw, snb + f * 4 * NN + pq, NN);
+      lifted(U + nbr[x], snb + f * 4 * NN + pq, NN);
     }
   }
   __syncthreads();
@@ -120,13 +121,15 @@ k_lift_lat(const double* __restrict__ U_, const double* __restrict__ metrics, co
   const int stride = d == 0 ? 1 : (d == 1 ? n : NN);
   const int line0 = id - r * stride;
   const double* jm = nullptr;
+  const double h = r == N ? hw : -hw;
   if (r == 0 || r == N)
     jm = snb + (2 * d + (r == N ? 1 : 0)) * 4 * NN + (d == 0 ? j : i) + n * (d == 2 ? j : k);
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
-    double s = jm ? jm[a * NN] : 0.0;
+    double s = 0.0;
 #pragma unroll
     for (int m = 0; m < n; ++m) s = fma(sD[r * n + m], sphi[a * P + line0 + m * stride], s);
+    if (jm) s = fma(h, jm[a * NN], s);
     sdd[(a * 3 + d) * P + id] = s;
   }
   __syncthreads();

@@ -187,7 +187,7 @@ __device__ __forceinline__ void lift_body_fx(const double* __restrict__ U, const
     }
     return;
   }
-  // line sums D phi + jump: 58 - e - e_D bits, below 2^60.2
+  // line sums D phi + jump
   i64 dd[4][3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
@@ -196,7 +196,7 @@ __device__ __forceinline__ void lift_body_fx(const double* __restrict__ U, const
     const bool edge = r == 0 || r == N;
     FxSum s[4];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) s[a] = FxSum{edge ? jm[a * NN] : 0, 0};
+    for (int a = 0; a < 4; ++a) s[a] = fx_lift_start(edge ? jm[a * NN] : 0);
     const longlong2* line = ph + id - r * stride;
 #pragma unroll
     for (int m = 0; m < n; ++m) {
@@ -208,23 +208,19 @@ __device__ __forceinline__ void lift_body_fx(const double* __restrict__ U, const
       fx_add(s[3], D, fx_split(p1.y));
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a) dd[a][d] = fx_end<kFxUpD>(s[a]);
+    for (int a = 0; a < 4; ++a) dd[a][d] = fx_lift_line(s[a]);
   }
   // g_l = (1/J) sum_d Ja^d_l dd_d
   const i64* mt = jx + (size_t)e * 10 * P + id;
   const Fx iJ = fx_split(mt[9 * P]);
-  const int qg = 56 + 62 - 64 - eD - (int)ej.x - (int)ej.z + 1;   // less e
+  const int qg = fx_lift_bits(eD, (int)ej.x, (int)ej.z);   // less e
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
-    const Fx J0 = fx_split(mt[l * P]), J1 = fx_split(mt[(3 + l) * P]), J2 = fx_split(mt[(6 + l) * P]);
+    const Fx J[3] = {fx_split(mt[l * P]), fx_split(mt[(3 + l) * P]), fx_split(mt[(6 + l) * P])};
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
-      FxSum s = fx_zero<2>();
-      fx_add(s, J0, fx_split(dd[a][0]));
-      fx_add(s, J1, fx_split(dd[a][1]));
-      fx_add(s, J2, fx_split(dd[a][2]));
-      const i64 G = fx_mul<1>(fx_split(fx_end<2>(s)), iJ);
-      go[(a * 3 + l) * P] = fx_to(G, qg - (a < 3 ? eu : et));
+      const Fx x[3] = {fx_split(dd[a][0]), fx_split(dd[a][1]), fx_split(dd[a][2])};
+      go[(a * 3 + l) * P] = fx_to(fx_lift_gradient(J, x, iJ), qg - (a < 3 ? eu : et));
     }
   }
 }

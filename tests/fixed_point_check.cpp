@@ -113,6 +113,47 @@ void check_pairs(int count, double r0, double r1, double p0, double p1, double u
   out[7] = (double)outside;
 }
 
+// Lifted gradients of one field along a line of n nodes, D [n][n], half = 1/(2
+// w_0): g = (1/J_el) J (D phi + jump), the other two derivatives 0.  out: rms
+// error of the fixed-point and of the FP64 arithmetic over the rms gradient.
+void check_lifting(int count, int n, const double* D, int eD, double half, double* out) {
+  srand48(14);
+  double ef = 0, ed = 0, sc = 0;
+  for (int t = 0; t < count; ++t) {
+    const double J = ldexp(uniform(0.5, 1.0), -3), iJ = uniform(0.6, 1.9), base = uniform(-1, 1), amp = uniform(0.01, 0.3),
+                 ph = uniform(0, 6);
+    double phi[16], top = 0;
+    for (int m = 0; m < n; ++m) top = std::max(top, std::fabs(phi[m] = base + amp * std::sin(ph + 2.0 * m / n)));
+    const double nbr[2] = {phi[0] + uniform(-1e-3, 1e-3), phi[n - 1] + uniform(-1e-3, 1e-3)};
+    top = std::max(top, std::max(std::fabs(nbr[0]), std::fabs(nbr[1])));
+    const int e = expo(top), ej = expo(J), ei = expo(iJ);
+    const Fx Jx[3] = {fx_split(fx_from(J, kFxQ - ej)), fx_split(0), fx_split(0)}, iJx = fx_split(fx_from(iJ, 62 - ei));
+    for (int r = 0; r < n; ++r) {
+      const bool edge = r == 0 || r == n - 1;
+      const double hs = r == 0 ? -half : half, nb = nbr[r != 0];
+      const i64 own = fx_from(phi[r], kFxQ - e);
+      FxSum s = fx_lift_start(
+          edge ? fx_mul<0>(fx_split(fx_from(nb, kFxQ - e) - own), fx_split(fx_round(hs, kFxQD - eD))) : 0);
+      double d = edge ? (nb - phi[r]) * hs : 0;
+      L x = edge ? ((L)nb - phi[r]) * hs : 0;
+      for (int m = 0; m < n; ++m) {
+        fx_add(s, fx_split(fx_round(D[r * n + m], kFxQD - eD)), fx_split(fx_from(phi[m], kFxQ - e)));
+        d = std::fma(D[r * n + m], phi[m], d);
+        x += (L)D[r * n + m] * phi[m];
+      }
+      const Fx dd[3] = {fx_split(fx_lift_line(s)), fx_split(0), fx_split(0)};
+      const double f = fx_to(fx_lift_gradient(Jx, dd, iJx), fx_lift_bits(eD, ej, ei) - e);
+      x = x * J * iJ;
+      d = J * d * iJ;
+      ef += (double)((f - x) * (f - x));
+      ed += (double)((d - x) * (d - x));
+      sc += (double)(x * x);
+    }
+  }
+  out[0] = std::sqrt(ef / sc);
+  out[1] = std::sqrt(ed / sc);
+}
+
 // Largest relative error of 2^119 / S over S in [2^57, 2^61).
 double check_rcp(int count) {
   srand48(12);

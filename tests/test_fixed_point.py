@@ -4,8 +4,9 @@ conversions, reciprocal and two-point flux against long double.
 Bars: a conversion to fixed point truncates to one unit of 2^-60; back to
 FP64 it rounds to nearest (2^-53, and 2^-32 units, of the 96-bit
 sums' last word); the reciprocal is good to 2^-55; the flux stays below 2^60.5, so
-that the sums with a row of D cannot overflow, and its error is no larger than
-that of the same formula in FP64 over the whole admitted range of the data."""
+that the sums with a row of D cannot overflow; its error and that of a lifted
+gradient are no larger than those of the same formula in FP64 over the admitted
+range of the states."""
 import ctypes as C
 import os
 import subprocess
@@ -24,6 +25,7 @@ def lib(tmp_path_factory):
     L = C.CDLL(so)
     L.check_rcp.restype = C.c_double
     L.check_pairs.argtypes = [C.c_int] + [C.c_double] * 6 + [C.c_int, C.c_double, C.c_void_p]
+    L.check_lifting.argtypes = [C.c_int, C.c_int, C.c_void_p, C.c_int, C.c_double, C.c_void_p]
     return L
 
 
@@ -60,3 +62,12 @@ def test_two_point_flux(lib, r0, r1, p0, p1, um, jm, axis, gamma):
     assert out[7] < 0.8 * n
     assert out[6] < 60.5, out[6]
     assert (fixed <= fp64).all(), (fixed, fp64)
+
+
+@pytest.mark.parametrize("N", range(1, 10))
+def test_lifted_gradient(lib, orc, N):
+    x, w, D = orc.basis(N)
+    out = np.zeros(2)
+    e_D = (0, 2, 3, 3, 4, 4, 5, 5, 5)[N - 1]
+    lib.check_lifting(4000, N + 1, D.ctypes.data_as(C.c_void_p), e_D, 0.5 / w[0], out.ctypes.data_as(C.c_void_p))
+    assert out[0] <= out[1], out
