@@ -66,7 +66,7 @@ struct alignas(16) FxAdjAlign {
   int r, u, b, j;
   int l0, lm, l4, eg;
   int ky, eub, erho, ebt;
-  int ek, eD, pad[2];
+  int ek, eD, t, pad;   // t: the directions' shifts (FxMetricShifts)
 };
 // e: exponents of the state (FxExp, with lb), eg of 1/(gamma - 1); l0, lm, l4 of
 // the adjoint -lambda/J (mass, momentum, energy).
@@ -86,7 +86,7 @@ DG_HD FxAdjAlign fx_adj_align(const FxExp& e, int eg, int l0, int lm, int l4, in
   a.erho = fx_max(esr, e0 + e.u + e.j + 1) + 1 + 2;
   a.ebt = fx_max(esr + ep + 1, ebl + 1) + 1 + 2;
   a.ek = ew4 + ef0 + 2;
-  a.pad[0] = a.pad[1] = 0;
+  a.t = a.pad = 0;
   return a;
 }
 
@@ -139,7 +139,7 @@ struct FxLongD {
 // Adjoint of the two-point flux: S = D_rm lam_r + D_mr lam_m (58 - e_D - l
 // bits, below 2^59; half the adjoint of the flux).  Shares of the density
 // adjoint of both nodes (r[0], r[1], exponent er), of beta (b[0], b[1], eb), of
-// {u} (u) and of |u|^2 (k).
+// {u} (u) and of |u|^2 (k).  j: exponent of the metric terms (at most al.j).
 struct FxPairAdj {
   i64 r[2], b[2];
   int er, eb;
@@ -148,7 +148,7 @@ struct FxPairAdj {
 };
 template <class LONG>
 DG_HD FxPairAdj fx_pair_vjp(i64 ra, i64 rb, i64 ba, i64 bb, const i64 su[3], i64 sk, const i64 sn[3], Fx G,
-                            const i64 S[5], const FxAdjAlign& al, LONG slopes_long) {
+                            int j, const i64 S[5], const FxAdjAlign& al, LONG slopes_long) {
   const i64 sr = ra + rb;
   const Fx Sr = fx_split(sr), Sb = fx_split(ba + bb);
   const i64 yr = fx_rcp(Sr);
@@ -176,7 +176,7 @@ DG_HD FxPairAdj fx_pair_vjp(i64 ra, i64 rb, i64 ba, i64 bb, const i64 su[3], i64
   const int ei = -al.b - al.ky;                        // of 1/(2 beta_ln): Hi has 62 bits, and of 1/(8 (b_a + b_b))
   FxSum s = fx_zero<2>();
   fx_add(s, U[0], N[0]); fx_add(s, U[1], N[1]); fx_add(s, U[2], N[2]);
-  const FxF un = fx_norm(FxF{fx_end<2>(s), al.u + al.j});
+  const FxF un = fx_norm(FxF{fx_end<2>(s), al.u + j});
   const Fx unx = fx_split(un.m);
   const FxF f0 = fx_norm(FxF{fx_mul<3>(Rl, unx), al.r + un.e});
   const FxF ph = fx_norm(FxF{fx_mul<1>(Sr, Yb), al.r + 1 + ei});
@@ -208,10 +208,10 @@ DG_HD FxPairAdj fx_pair_vjp(i64 ra, i64 rb, i64 ba, i64 bb, const i64 su[3], i64
   o.k = FxF{-Hb.m, Hb.e};
   s = fx_zero<3>();
   fx_add(s, B[0], N[0]); fx_add(s, B[1], N[1]); fx_add(s, B[2], N[2]);
-  const FxF phb = fx_norm(FxF{fx_end<3>(s), fmb.e + al.j});
+  const FxF phb = fx_norm(FxF{fx_end<3>(s), fmb.e + j});
   // f_m = f0 {u} + p_hat n
-  const int ef = fx_max(f0.e + al.u, ph.e + al.j) + 1;
-  const Fx A1 = fx_split(fx_down(f0.m, ef - f0.e - al.u)), A2 = fx_split(fx_down(ph.m, ef - ph.e - al.j));
+  const int ef = fx_max(f0.e + al.u, ph.e + j) + 1;
+  const Fx A1 = fx_split(fx_down(f0.m, ef - f0.e - al.u)), A2 = fx_split(fx_down(ph.m, ef - ph.e - j));
   FxF3 fm;
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
@@ -224,7 +224,7 @@ DG_HD FxPairAdj fx_pair_vjp(i64 ra, i64 rb, i64 ba, i64 bb, const i64 su[3], i64
   fm = fx_norm(fm);
   // adjoint of {u}: w_4 f_m + f0 fmb + (f0b rho_ln) n
   const FxF c3 = fx_norm(FxF{fx_mul<3>(f0bx, Rl), f0b.e + al.r});
-  const int e1 = w4.e + fm.e, e2 = f0.e + fmb.e, e3 = c3.e + al.j, eu = fx_max(fx_max(e1, e2), e3) + 2;
+  const int e1 = w4.e + fm.e, e2 = f0.e + fmb.e, e3 = c3.e + j, eu = fx_max(fx_max(e1, e2), e3) + 2;
   const Fx C1 = fx_split(fx_down(w4.m, eu - e1)), C2 = fx_split(fx_down(f0.m, eu - e2)),
            C3 = fx_split(fx_down(c3.m, eu - e3 + 1));
 #pragma unroll
@@ -324,6 +324,7 @@ __device__ __forceinline__ bool adj_pairs_fx(const double* __restrict__ U, const
   __syncthreads();
   const int* mx = s_mx[le];
   const float4 ej = active ? ejx[e] : make_float4(1000.0f, 0.0f, 0.0f, 0.0f);
+  const FxMetricShifts sh = fx_shifts(ej);
   FxExp x{fx_expo(mx[kR]), fx_expo(mx[kU]), fx_expo(mx[kB]), (int)ej.x, 0.0f, 0.0f, 0.0f, 0.0f};
   x.u = max(x.u, ((-x.b) >> 1) - 40);   // 2^-40 of the speed of sound
   const int l0 = fx_expo(mx[kL0]), lm = fx_expo(mx[kLm]), l4 = fx_expo(mx[kL4]);
@@ -336,6 +337,7 @@ __device__ __forceinline__ bool adj_pairs_fx(const double* __restrict__ U, const
     if (act) {
       x.lb = fx_log_mantissa(bmin, 0) + (float)((bmin >> 20) - 1022 - x.b);
       s_al[le] = fx_adj_align(x, eg, l0, lm, l4, eD);
+      s_al[le].t = sh.w;
     }
   }
   if (act) {
@@ -347,7 +349,7 @@ __device__ __forceinline__ bool adj_pairs_fx(const double* __restrict__ U, const
     base[5 * P + id] = fx_from(w, 60 - x.u);
     const i64* mt = jx + (size_t)e * 10 * P + id;
 #pragma unroll
-    for (int r = 0; r < 9; ++r) base[(6 + r) * P + id] = mt[r * P];
+    for (int r = 0; r < 9; ++r) base[(6 + r) * P + id] = fx_up(mt[r * P], sh.t(r / 3));
     base[15 * P + id] = fx_from(lv[0], 60 - l0);
 #pragma unroll
     for (int c = 1; c < 4; ++c) base[(15 + c) * P + id] = fx_from(lv[c], 60 - lm);
@@ -374,8 +376,8 @@ __device__ __forceinline__ bool adj_pairs_fx(const double* __restrict__ U, const
       su[l] = b2[(3 + l) * P + ia] + b2[(3 + l) * P + ib];
       sn[l] = b2[(6 + 3 * d + l) * P + ia] + b2[(6 + 3 * d + l) * P + ib];
     }
-    return fx_pair_vjp(b2[ia], b2[ib], b2[P + ia], b2[P + ib], su, b2[2 * P + ia] + b2[2 * P + ib], sn, s_G, W,
-                       s_al[el], FxLongD());
+    return fx_pair_vjp(b2[ia], b2[ib], b2[P + ia], b2[P + ib], su, b2[2 * P + ia] + b2[2 * P + ib], sn, s_G,
+                       s_al[el].j - (s_al[el].t >> (4 * d) & 15), W, s_al[el], FxLongD());
   };
   // a pair's shares for one node into its exchange slot; the shifts to the
   // exponents of the sums (at most 255) as bytes

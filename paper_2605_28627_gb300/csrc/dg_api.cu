@@ -168,7 +168,7 @@ struct dg_ctx : public dg::Ctx {};
 struct InitScratch {
   cudaStream_t s = nullptr;
   double* d_xgeo = nullptr;
-  int* d_bad = nullptr;
+  int* d_bad = nullptr;   // non-positive Jacobian, stretched elements
   ~InitScratch() {
     if (d_xgeo) cudaFree(d_xgeo);
     if (d_bad) cudaFree(d_bad);
@@ -368,11 +368,11 @@ static dg_status init_impl(const dg_mesh* mesh, const dg_params* prm, int device
   const int minmask = 1 << 8;
   const size_t m3 = (size_t)(mesh->ngeo + 1) * (mesh->ngeo + 1) * (mesh->ngeo + 1);
   cudaError_t err = cudaMalloc(&tmp.d_xgeo, sizeof(double) * E * 3 * m3);
-  if (err == cudaSuccess) err = cudaMalloc(&tmp.d_bad, sizeof(int));
+  if (err == cudaSuccess) err = cudaMalloc(&tmp.d_bad, 2 * sizeof(int));
   double* d_xgeo = tmp.d_xgeo;
   int* d_bad = tmp.d_bad;
   if (err == cudaSuccess) err = cudaMemcpyAsync(d_xgeo, mesh->xgeo, sizeof(double) * E * 3 * m3, cudaMemcpyHostToDevice, s);
-  if (err == cudaSuccess) err = cudaMemsetAsync(d_bad, 0, sizeof(int), s);
+  if (err == cudaSuccess) err = cudaMemsetAsync(d_bad, 0, 2 * sizeof(int), s);
   if (err == cudaSuccess) err = cudaMemcpyAsync(c->d_D, c->D.data(), sizeof(double) * NN, cudaMemcpyHostToDevice, s);
   if (prm->nodes == DG_NODES_LG) {
     if (err == cudaSuccess)
@@ -418,16 +418,18 @@ static dg_status init_impl(const dg_mesh* mesh, const dg_params* prm, int device
   if (err == cudaSuccess) err = setup_kernels(c->N);
   if (err == cudaSuccess) err = build_geometry(*c, d_xgeo, mesh->ngeo, d_bad, s);
   if (err == cudaSuccess && prm->nodes == DG_NODES_LG) err = gauss_geometry(*c, d_bad, s);
-  if (err == cudaSuccess && c->d_jx) err = launch_fx_metrics(*c, s);
+  if (err == cudaSuccess && c->d_jx) err = launch_fx_metrics(*c, d_bad + 1, s);
   if (err == cudaSuccess && prm->source == DG_SOURCE_MMS) err = launch_mms_phase(*c, s);
   if (err == cudaSuccess && prm->precision == DG_FP32OP) {
     err = launch_to_float(c->d_metrics, c->d_metrics_f, (size_t)E * 10 * P, s);
     if (err == cudaSuccess) err = launch_to_float(c->d_facegeo, c->d_facegeo_f, (size_t)c->nfaces * 4 * NN, s);
     if (err == cudaSuccess) err = cudaStreamSynchronize(s);
   }
-  int bad = 0;
-  if (err == cudaSuccess) err = cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, s);
+  int flags[2] = {0, 0};
+  if (err == cudaSuccess) err = cudaMemcpyAsync(flags, d_bad, sizeof flags, cudaMemcpyDeviceToHost, s);
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);
+  const int bad = flags[0];
+  c->fx_stretch = flags[1] != 0;
   if (err != cudaSuccess) {
     fail(c, err == cudaErrorMemoryAllocation ? DG_ENOMEM : DG_ECUDA, "dg_init: geometry", err);
     return bail(err == cudaErrorMemoryAllocation ? DG_ENOMEM : DG_ECUDA);

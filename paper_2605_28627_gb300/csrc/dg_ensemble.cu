@@ -74,7 +74,9 @@ k_face_ens(const MemberDev<R>* __restrict__ mem, int nmem, const int2* __restric
   }
 }
 
-template <int N, typename R, int EPB>
+// STRETCH as in volume_body_fx: true if any member of the group holds stretched
+// elements.
+template <int N, typename R, int EPB, bool STRETCH>
 __global__ void __launch_bounds__(VShape<N, EPB>::THREADS)
 k_volume_ens(const MemberDev<R>* __restrict__ mem, int nmem, const int2* __restrict__ tiles, int ntiles,
              const double* __restrict__ Dg, double c_stage, double A, double B) {
@@ -83,7 +85,7 @@ k_volume_ens(const MemberDev<R>* __restrict__ mem, int nmem, const int2* __restr
     const MemberDev<R>& m = mem[dg_idx(tl.x, nmem, kSiteEnsMember)];
     StageArgs a{m.U, m.U, m.G, nullptr, m.clock, c_stage, A, B, 1};
     if constexpr (sizeof(R) == 8)
-      volume_body_f64<N, EPB>(a, m.metrics, m.jx, m.ejx, m.grad, m.fstar, m.elem_face, m.mms, Dg, m.E, m.gas, m.inv_w0,
+      volume_body_f64<N, EPB, false, STRETCH>(a, m.metrics, m.jx, m.ejx, m.grad, m.fstar, m.elem_face, m.mms, Dg, m.E, m.gas, m.inv_w0,
                               tl.y);
     else
       volume_body<N, R, EPB>(a, m.metrics, m.metrics64, m.grad, m.fstar, m.elem_face, m.mms, Dg, m.E, m.gas,
@@ -112,8 +114,12 @@ struct GroupPlan {
 
 template <int N, typename R, int EPB>
 static cudaError_t set_vol_attr() {
-  return cudaFuncSetAttribute(k_volume_ens<N, R, EPB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)volume_op_smem_bytes<N, R, EPB>());
+  const int bytes = (int)volume_op_smem_bytes<N, R, EPB>();
+  cudaError_t e = cudaFuncSetAttribute(k_volume_ens<N, R, EPB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if constexpr (sizeof(R) == 8)
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_volume_ens<N, R, EPB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return e;
 }
 
 template <int N, typename R>
@@ -130,6 +136,7 @@ struct Group {
   // elements) do not cover: Gauss nodes, mortars or FV elements at creation;
   // they run as single-member units with their own stage kernels
   bool single_only = false;
+  bool stretch = false;                // any member with stretched elements (Ctx::fx_stretch)
   std::vector<int> members;            // indices into the ensemble
   void* d_mem = nullptr;               // MemberDev<R>[members]
   int2* d_elem_tiles[2] = {nullptr, nullptr};   // per EPB choice
@@ -151,12 +158,18 @@ static cudaError_t launch_group_stage(const Group& g, int k, const double* A, co
   k_lift_ens<N, R, e0><<<g.plan.lift_grid, Shape<N, e0>::THREADS, lift_op_smem_bytes<N, R, e0>(), s>>>(
       mem, nmem, g.d_elem_tiles[0], g.n_elem_tiles[0], g.d_D);
   k_face_ens<N, R><<<g.plan.face_grid, 128, 0, s>>>(mem, nmem, g.d_face_tiles, g.n_face_tiles);
+  auto volume = [&](auto kernel, int threads, size_t smem) {
+    kernel<<<g.plan.vol_grid, threads, smem, s>>>(mem, nmem, g.d_elem_tiles[ch], g.n_elem_tiles[ch], g.d_D, C[k], A[k],
+                                                  B[k]);
+  };
+  constexpr bool both = sizeof(R) == 8;
+  const bool st = both && g.stretch;
   if (ch == 0)
-    k_volume_ens<N, R, e0><<<g.plan.vol_grid, VShape<N, e0>::THREADS, volume_op_smem_bytes<N, R, e0>(), s>>>(
-        mem, nmem, g.d_elem_tiles[0], g.n_elem_tiles[0], g.d_D, C[k], A[k], B[k]);
+    volume(st ? k_volume_ens<N, R, e0, both> : k_volume_ens<N, R, e0, false>, VShape<N, e0>::THREADS,
+           volume_op_smem_bytes<N, R, e0>());
   else
-    k_volume_ens<N, R, e1><<<g.plan.vol_grid, VShape<N, e1>::THREADS, volume_op_smem_bytes<N, R, e1>(), s>>>(
-        mem, nmem, g.d_elem_tiles[1], g.n_elem_tiles[1], g.d_D, C[k], A[k], B[k]);
+    volume(st ? k_volume_ens<N, R, e1, both> : k_volume_ens<N, R, e1, false>, VShape<N, e1>::THREADS,
+           volume_op_smem_bytes<N, R, e1>());
   return cudaGetLastError();
 }
 
@@ -557,6 +570,7 @@ static dg_status ensemble_create_impl(dg_ctx* const* members, int32_t n, const c
     Group& g = e->groups.back();
     g.N = kv.first;
     g.members = kv.second;
+    for (int r : g.members) g.stretch = g.stretch || e->members[r]->fx_stretch;
     g.d_D = e->members[g.members[0]]->d_D;
     const size_t msz = e->precision == DG_FP32OP ? sizeof(MemberDev<float>) : sizeof(MemberDev<double>);
     if (cudaMalloc(&g.d_mem, msz * g.members.size()) != cudaSuccess) return bail(DG_ENOMEM);

@@ -500,7 +500,7 @@ k_lift_lg(const double* __restrict__ U, const R* __restrict__ Uf, const R* __res
                                   n_mortar);
 }
 // FP64 operator: fixed point, then FP64 for the elements out of its range.
-template <int N, int EPB, bool MORTAR>
+template <int N, int EPB, bool MORTAR, bool STRETCH>
 __global__ void __launch_bounds__(Shape<N, EPB>::THREADS, lift_lg_fx_min_blocks<N>())
 k_lift_lg_fx(const double* __restrict__ U, const double* __restrict__ Uf, const double* __restrict__ metrics,
              const i64* __restrict__ jx, const float4* __restrict__ ejx, const double* __restrict__ facegeo,
@@ -508,8 +508,8 @@ k_lift_lg_fx(const double* __restrict__ U, const double* __restrict__ Uf, const 
              double* __restrict__ grad, double* __restrict__ gf, int E, int F, Gas g,
              const double* __restrict__ mvirt, int n_mortar) {
   __shared__ int s_state[EPB];
-  if (lift_lg_fx<N, EPB, MORTAR>(U, Uf, jx, ejx, facegeo, elem_face, elem_nbr, tab, grad, gf, E, F, g, mvirt, n_mortar,
-                                 s_state)) {
+  if (lift_lg_fx<N, EPB, MORTAR, STRETCH>(U, Uf, jx, ejx, facegeo, elem_face, elem_nbr, tab, grad, gf, E, F, g, mvirt,
+                                          n_mortar, s_state)) {
     __syncthreads();
     lift_lg_body<N, EPB, MORTAR, double>(U, Uf, metrics, facegeo, elem_face, elem_nbr, tab, grad, gf, E, F, g, mvirt,
                                          n_mortar, s_state);
@@ -723,14 +723,14 @@ k_volume_lg(StageArgs a, const R* __restrict__ metrics, const double* __restrict
             const double* __restrict__ mms, const double* __restrict__ tab, int E, Gas g) {
   volume_lg_body<N, EPB, LIST, R>(a, metrics, metrics64, grad, fstar, elem_face, mms, tab, E, g);
 }
-template <int N, int EPB, bool LIST>
+template <int N, int EPB, bool LIST, bool STRETCH>
 __global__ void __launch_bounds__(Shape<N, EPB>::THREADS, volume_lg_fx_min_blocks<N>())
 k_volume_lg_fx(StageArgs a, const double* __restrict__ metrics, const i64* __restrict__ jx,
                const float4* __restrict__ ejx, const double* __restrict__ grad, const double* __restrict__ fstar,
                const int* __restrict__ elem_face, const double* __restrict__ mms, const double* __restrict__ tab, int E,
                Gas g) {
   __shared__ int s_state[EPB];
-  if (volume_lg_fx<N, EPB, LIST>(a, metrics, jx, ejx, grad, fstar, elem_face, mms, tab, E, g, s_state)) {
+  if (volume_lg_fx<N, EPB, LIST, STRETCH>(a, metrics, jx, ejx, grad, fstar, elem_face, mms, tab, E, g, s_state)) {
     __syncthreads();
     volume_lg_body<N, EPB, LIST, double>(a, metrics, metrics, grad, fstar, elem_face, mms, tab, E, g, s_state);
   }
@@ -747,12 +747,14 @@ static cudaError_t setup_lg_NR() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_lift_lg<N, S::EPB, true, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)lift_lg_smem<N, S::EPB, R>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_volume_lg<N, S::EPB, false, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)volume_lg_smem<N, S::EPB, R>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_volume_lg<N, S::EPB, true, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)volume_lg_smem<N, S::EPB, R>());
+  if constexpr (sizeof(R) == 4) {   // FP64: k_volume_lg_fx
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_volume_lg<N, S::EPB, false, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)volume_lg_smem<N, S::EPB, R>());
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_volume_lg<N, S::EPB, true, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)volume_lg_smem<N, S::EPB, R>());
+  }
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_prolong_lg<N, S::EPB, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(sizeof(R) * S::EPB * 5 * S::P));
@@ -775,10 +777,12 @@ static cudaError_t setup_lg_fx_N() {
   using S = Shape<N>;
   const int ls = (int)lift_lg_f64_smem<N>(), vs = (int)volume_lg_f64_smem<N>();
   const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(k_lift_lg_fx<N, S::EPB, false>, at, ls);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lift_lg_fx<N, S::EPB, true>, at, ls);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_volume_lg_fx<N, S::EPB, false>, at, vs);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_volume_lg_fx<N, S::EPB, true>, at, vs);
+  cudaError_t e = cudaFuncSetAttribute(k_lift_lg_fx<N, S::EPB, false, false>, at, ls);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lift_lg_fx<N, S::EPB, false, true>, at, ls);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lift_lg_fx<N, S::EPB, true, true>, at, ls);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_volume_lg_fx<N, S::EPB, false, false>, at, vs);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_volume_lg_fx<N, S::EPB, false, true>, at, vs);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_volume_lg_fx<N, S::EPB, true, true>, at, vs);
   return e;
 }
 
@@ -833,14 +837,14 @@ static cudaError_t lift_lg_NR(const Ctx& c, const double* U, cudaStream_t s) {
   }
   if constexpr (sizeof(R) == 8) {
     if (c.d_jx) {   // absent in an FP32-operator context, whose diagnostics lift in FP64
-      if (c.M > 0)
-        k_lift_lg_fx<N, S::EPB, true><<<blocks, S::THREADS, lift_lg_f64_smem<N>(), s>>>(
+      auto launch = [&](auto kernel, const double* mvirt) {
+        kernel<<<blocks, S::THREADS, lift_lg_f64_smem<N>(), s>>>(
             U, Uf, c.d_metrics, c.d_jx, c.d_ejx, c.d_facegeo, c.d_elem_face, c.d_elem_nbr, c.d_lgb, (double*)c.d_grad,
-            gf, c.E, c.nfaces, c.gas, c.d_mortar_virt, c.M);
-      else
-        k_lift_lg_fx<N, S::EPB, false><<<blocks, S::THREADS, lift_lg_f64_smem<N>(), s>>>(
-            U, Uf, c.d_metrics, c.d_jx, c.d_ejx, c.d_facegeo, c.d_elem_face, c.d_elem_nbr, c.d_lgb, (double*)c.d_grad,
-            gf, c.E, c.nfaces, c.gas, nullptr, 0);
+            gf, c.E, c.nfaces, c.gas, mvirt, c.M);
+      };
+      if (c.M > 0) launch(k_lift_lg_fx<N, S::EPB, true, true>, c.d_mortar_virt);
+      else if (c.fx_stretch) launch(k_lift_lg_fx<N, S::EPB, false, true>, nullptr);
+      else launch(k_lift_lg_fx<N, S::EPB, false, false>, nullptr);
       return cudaGetLastError();
     }
   }
@@ -892,24 +896,23 @@ static cudaError_t volume_lg_NR(const Ctx& c, const StageArgs& a0, cudaStream_t 
   a.nfaces = c.nfaces;
   const int blocks = (c.E + S::EPB - 1) / S::EPB;
   if constexpr (sizeof(R) == 8) {
-    if (a.list != nullptr)
-      k_volume_lg_fx<N, S::EPB, true><<<blocks, S::THREADS, volume_lg_f64_smem<N>(), s>>>(
-          a, c.d_metrics, c.d_jx, c.d_ejx, (const double*)c.d_grad, (const double*)c.d_fstar, c.d_elem_face, c.d_mms,
-          c.d_lgb, c.E, c.gas);
-    else
-      k_volume_lg_fx<N, S::EPB, false><<<blocks, S::THREADS, volume_lg_f64_smem<N>(), s>>>(
-          a, c.d_metrics, c.d_jx, c.d_ejx, (const double*)c.d_grad, (const double*)c.d_fstar, c.d_elem_face, c.d_mms,
-          c.d_lgb, c.E, c.gas);
-    return cudaGetLastError();
+    auto launch = [&](auto kernel) {
+      kernel<<<blocks, S::THREADS, volume_lg_f64_smem<N>(), s>>>(a, c.d_metrics, c.d_jx, c.d_ejx, (const double*)c.d_grad,
+                                                                (const double*)c.d_fstar, c.d_elem_face, c.d_mms,
+                                                                c.d_lgb, c.E, c.gas);
+    };
+    if (a.list != nullptr) launch(k_volume_lg_fx<N, S::EPB, true, true>);
+    else if (c.fx_stretch) launch(k_volume_lg_fx<N, S::EPB, false, true>);
+    else launch(k_volume_lg_fx<N, S::EPB, false, false>);
+  } else {
+    auto launch = [&](auto kernel) {
+      kernel<<<blocks, S::THREADS, volume_lg_smem<N, S::EPB, R>(), s>>>(a, metrics_of<R>(c), c.d_metrics,
+                                                                       (const R*)c.d_grad, (const R*)c.d_fstar,
+                                                                       c.d_elem_face, c.d_mms, c.d_lgb, c.E, c.gas);
+    };
+    if (a.list != nullptr) launch(k_volume_lg<N, S::EPB, true, R>);
+    else launch(k_volume_lg<N, S::EPB, false, R>);
   }
-  if (a.list != nullptr)
-    k_volume_lg<N, S::EPB, true, R><<<blocks, S::THREADS, volume_lg_smem<N, S::EPB, R>(), s>>>(
-        a, metrics_of<R>(c), c.d_metrics, (const R*)c.d_grad, (const R*)c.d_fstar, c.d_elem_face, c.d_mms, c.d_lgb,
-        c.E, c.gas);
-  else
-    k_volume_lg<N, S::EPB, false, R><<<blocks, S::THREADS, volume_lg_smem<N, S::EPB, R>(), s>>>(
-        a, metrics_of<R>(c), c.d_metrics, (const R*)c.d_grad, (const R*)c.d_fstar, c.d_elem_face, c.d_mms, c.d_lgb,
-        c.E, c.gas);
   return cudaGetLastError();
 }
 

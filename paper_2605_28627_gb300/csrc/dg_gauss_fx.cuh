@@ -29,7 +29,9 @@ constexpr size_t lift_lg_fx_smem() {
 }
 
 // Returns whether the block holds elements left to FP64 (state[le] = 2).
-template <int N, int EPB, bool MORTAR>
+// STRETCH (both kernels): the mesh may hold elements with shifted metric terms
+// (FxMetricShifts); without it every shift is 0.
+template <int N, int EPB, bool MORTAR, bool STRETCH>
 __device__ __forceinline__ bool lift_lg_fx(const double* __restrict__ U, const double* __restrict__ Uf,
                                            const i64* __restrict__ jx, const float4* __restrict__ ejx,
                                            const double* __restrict__ facegeo, const int* __restrict__ elem_face,
@@ -105,10 +107,11 @@ __device__ __forceinline__ bool lift_lg_fx(const double* __restrict__ U, const d
   if (id == 0) state[le] = active ? (act ? 1 : 2) : 0;
   i64 Ja[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, iJ = 0;
   Fx X[4];
+  const FxMetricShifts sh{STRETCH ? __float_as_int(ej.w) : 0};
   if (act) {
     const i64* mt = jx + (size_t)e * 10 * P + id;
 #pragma unroll
-    for (int r = 0; r < 9; ++r) Ja[r] = mt[r * P];
+    for (int r = 0; r < 9; ++r) Ja[r] = fx_up(mt[r * P], sh.c(r % 3));
     iJ = mt[9 * P];
 #pragma unroll
     for (int a = 0; a < 4; ++a) X[a] = fx_split(fx_from(ph[a], 62 - (a < 3 ? eu : et)));
@@ -119,15 +122,15 @@ __device__ __forceinline__ bool lift_lg_fx(const double* __restrict__ U, const d
 #pragma unroll
       for (int a = 0; a < 4; ++a) st[a] = fx_split(fx_from(__longlong_as_double(s[a * NN]), 62 - (a < 3 ? eu : et)));
 #pragma unroll
-      for (int l = 0; l < 3; ++l) ns[l] = fx_split(fx_from(__longlong_as_double(s[(4 + l) * NN]), kFxQ - (int)ej.x));
+      for (int l = 0; l < 3; ++l) ns[l] = fx_split(fx_from(__longlong_as_double(s[(4 + l) * NN]), kFxQ - (int)ej.x + sh.c(l)));
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int l = 0; l < 3; ++l) s[(a * 3 + l) * NN] = fx_mul<2>(st[a], ns[l]);   // 60 - e - e_j
+        for (int l = 0; l < 3; ++l) s[(a * 3 + l) * NN] = fx_mul<2>(st[a], ns[l]);   // 60 - e - e_j + c_l
     }
   }
   const int i = id % n, j = (id / n) % n, k = id / NN;
-  i64 acc[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};   // 59 - e - e_j - e_D, below 2^62
+  i64 acc[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};   // 59 - e - e_j + c_l - e_D, below 2^62
 #pragma unroll 1
   for (int d = 0; d < 3; ++d) {
     __syncthreads();
@@ -162,14 +165,14 @@ __device__ __forceinline__ bool lift_lg_fx(const double* __restrict__ U, const d
     }
   }
   __syncthreads();   // every thread is done with sprod
-  const int qg = 59 + 62 - 64 + 1 - (int)ej.x - eD - (int)ej.z;   // less e
+  const int qg = 59 + 62 - 64 + 1 - (int)ej.x - eD - (int)ej.z;   // less e, + c_l
   if (act) {
     double* go = grad + (size_t)e * 12 * P + id;
     const Fx iJx = fx_split(iJ);
 #pragma unroll
     for (int al = 0; al < 12; ++al) {
       const i64 G = fx_mul<1>(fx_split(acc[al]), iJx);   // below 2^61
-      go[al * P] = fx_to(G, qg - (al < 9 ? eu : et));
+      go[al * P] = fx_to(G, qg + sh.c(al % 3) - (al < 9 ? eu : et));
       sprod[al * P + id] = G;
     }
   }
@@ -190,7 +193,7 @@ __device__ __forceinline__ bool lift_lg_fx(const double* __restrict__ U, const d
       if (n > 5 && m == n / 2) fx_fold(s);   // five terms fill c
       fx_add(s, l[m], fx_split(line[m * stride]));
     }
-    gf[((size_t)e * 6 + f) * 12 * NN + (size_t)al * NN + pq] = fx_to(fx_end<4>(s), qg + 59 - 64 + 4 - (al < 9 ? eu : et));
+    gf[((size_t)e * 6 + f) * 12 * NN + (size_t)al * NN + pq] = fx_to(fx_end<4>(s), qg + sh.c(al % 3) + 59 - 64 + 4 - (al < 9 ? eu : et));
   }
   return bad;
 }
@@ -202,7 +205,7 @@ constexpr size_t volume_lg_fx_smem() {
 }
 
 // Returns whether the block holds elements left to FP64 (state[le] = 2).
-template <int N, int EPB, bool LIST>
+template <int N, int EPB, bool LIST, bool STRETCH>
 __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* __restrict__ metrics,
                                              const i64* __restrict__ jx, const float4* __restrict__ ejx,
                                              const double* __restrict__ grad, const double* __restrict__ fstar,
@@ -234,6 +237,8 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
   for (int t = threadIdx.x; t < EPB * kCount; t += blockDim.x) s_mx[t / kCount][t % kCount] = 0;
   if (threadIdx.x == 0 && g.source == DG_SOURCE_MMS)
     sincospi(a.clock[0] + a.c_stage * a.clock[1], &s_tc[0], &s_tc[1]);
+  const float4 ejv = active ? ejx[e] : make_float4(1000.0f, 0.0f, 0.0f, 0.0f);
+  const FxMetricShifts sh{STRETCH ? __float_as_int(ejv.w) : 0};
   __syncthreads();
   double q[5] = {1, 0, 0, 0, 0}, gr[12];
   double u = 0, v = 0, w = 0, p = 0;
@@ -272,9 +277,10 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
         val = -fstar[((size_t)fid * 5 + v2) * NN + p2 + n * q2];
       }
       sFs[(f * 5 + v2) * NN + pq] = __double_as_longlong(val);
-      if (v2 == 0) m[kF0] = max(m[kF0], fx_mag(val));
-      else if (v2 == 4) m[kFe] = max(m[kFe], fx_mag(val));
-      else m[kFm] = max(m[kFm], fx_mag(val));
+      const int mv = fx_mag(val) + (sh.t(f >> 1) << 20);   // of val 2^t, as it is held below
+      if (v2 == 0) m[kF0] = max(m[kF0], mv);
+      else if (v2 == 4) m[kFe] = max(m[kFe], mv);
+      else m[kFm] = max(m[kFm], mv);
     }
     fx_maxima<kCount>(le, s_mx[le], m);
   }
@@ -285,12 +291,11 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
     x[c] = fx_expo(s_mx[le][c]);
     top = max(top, x[c]);
   }
-  const float4 ejv = active ? ejx[e] : make_float4(1000.0f, 0.0f, 0.0f, 0.0f);
   const int ej = (int)ejv.x, em = fx_expo(fx_mag(g.mu)), el = fx_expo(fx_mag(g.mu * g.kappa));
   const bool act = active && top < 90 && ej < 90;
   if (id == 0) state[le] = active ? (act ? 1 : 2) : 0;
-  // bits after the point of the mass (q0), momentum (qm) and energy (qe) fluxes:
-  // below 2^61.3, so that six of a line's n + 2 terms fit in FxSum's c (the part of
+  // bits after the point of the mass (q0), momentum (qm) and energy (qe) fluxes,
+  // + t_d in direction d: below 2^61.3, so that six of a line's n + 2 terms fit in FxSum's c (the part of
   // the products that fx_add leaves out is the sums' largest error, and a bit
   // more in the factors halves it)
   const int n0 = 61 - x[kR] - x[kU] - ej;                                             // rho {u . Ja}
@@ -319,7 +324,9 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
     const i64* mt = jx + (size_t)e * 10 * P + id;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const Fx J[3] = {fx_split(mt[(d * 3) * P]), fx_split(mt[(d * 3 + 1) * P]), fx_split(mt[(d * 3 + 2) * P])};
+      const int t = sh.t(d);
+      const Fx J[3] = {fx_split(fx_up(mt[(d * 3) * P], t)), fx_split(fx_up(mt[(d * 3 + 1) * P], t)),
+                       fx_split(fx_up(mt[(d * 3 + 2) * P], t))};
       FxSum s = fx_zero<3>();
       fx_add(s, U[0], J[0]); fx_add(s, U[1], J[1]); fx_add(s, U[2], J[2]);
       const Fx un = fx_split(fx_end<3>(s));                 // 61 - e_u - e_j
@@ -347,7 +354,7 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
     for (int o = id; o < 30 * NN; o += P) {
       const int v2 = (o / NN) % 5;
       i64* s = sFs + o;
-      *s = fx_from(__longlong_as_double(*s), v2 == 0 ? q0 : (v2 == 4 ? qe : qm));
+      *s = fx_from(__longlong_as_double(*s), (v2 == 0 ? q0 : (v2 == 4 ? qe : qm)) + sh.t(o / (10 * NN)));
     }
   }
   __syncthreads();
@@ -357,8 +364,10 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
   if (!act) return bad;
   const int i = id % n, j = (id / n) % n, k = id / NN;
   i64 acc[5] = {0, 0, 0, 0, 0};
+  const int walk = sh.walk();   // the directions by falling t: the sums are only shifted down
 #pragma unroll 1
-  for (int d = 0; d < 3; ++d) {
+  for (int pass = 0; pass < 3; ++pass) {
+    const int d = STRETCH ? walk >> (2 * pass) & 3 : pass;
     const int r = d == 0 ? i : (d == 1 ? j : k);
     const int stride = d == 0 ? 1 : (d == 1 ? n : NN);
     const int line0 = id - r * stride, pq = d == 0 ? j + n * k : (d == 1 ? i + n * k : i + n * j);
@@ -376,6 +385,10 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
       fx_add(s, t0, fx_split(sFs[(2 * d * 5 + c) * NN + pq]));
       fx_add(s, t1, fx_split(sFs[((2 * d + 1) * 5 + c) * NN + pq]));
       acc[c] += fx_end<kFxUpD>(s);
+    }
+    if (const int down = walk >> (8 + 4 * pass) & 15) {
+#pragma unroll
+      for (int c = 0; c < 5; ++c) acc[c] = (acc[c] + ((i64)1 << (down - 1))) >> down;
     }
   }
   double src[5] = {0, 0, 0, 0, 0};

@@ -126,6 +126,7 @@ struct Ctx {
   float* d_metrics_f = nullptr;  // FP32 copies for the FP32-operator path
   long long* d_jx = nullptr;     // [E][10][P] metric terms and 1/J in fixed point (FP64 operator)
   float4* d_ejx = nullptr;       // [E] their exponents (k_fx_metrics)
+  bool fx_stretch = false;       // whether any element's directions differ by a factor 2 (k_fx_metrics)
   float* d_facegeo_f = nullptr;
   FaceInfo* d_faces = nullptr;   // [F]: the conforming faces, then the mortars' small and big sides
   int nfaces_conf = 0;           // conforming faces (the face kernel's range)
@@ -217,7 +218,7 @@ cudaError_t launch_lift_lg(const Ctx& c, const double* U, cudaStream_t s, bool f
 cudaError_t launch_face_lg(const Ctx& c, cudaStream_t s);
 cudaError_t launch_volume_lg(const Ctx& c, const StageArgs& a, cudaStream_t s);
 cudaError_t setup_volume(int N);
-cudaError_t launch_fx_metrics(const Ctx& c, cudaStream_t s);   // fills d_jx, d_ejx from d_metrics
+cudaError_t launch_fx_metrics(const Ctx& c, int* d_stretch, cudaStream_t s);   // fills d_jx, d_ejx from d_metrics
 
 // FV sub-cell operator (dg_fv.cu): tables of the node set, the once-per-context
 // geometry (Jb, area vectors) and one stage (means, sub-face fluxes, the DG

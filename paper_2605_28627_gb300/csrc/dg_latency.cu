@@ -175,7 +175,8 @@ struct LatFx {
 };
 
 // False (the whole block): the element is out of the fixed-point range.
-template <int N>
+// STRETCH as in volume_body_fx.
+template <int N, bool STRETCH>
 __device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* __restrict__ metrics,
                                               const i64* __restrict__ jx, const float4* __restrict__ ejx,
                                               const double* grad_, const double* fstar_,
@@ -202,8 +203,10 @@ __device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* 
   // every operand is asked for here, what no kernel writes before the wait
   if (threadIdx.x < kMxCount) s_mx[threadIdx.x] = 0;
   const i64* mt = jx + (size_t)e * 10 * P + id;
-  const i64 Ja[3] = {mt[(d * 3) * P], mt[(d * 3 + 1) * P], mt[(d * 3 + 2) * P]};
+  const i64 Jr[3] = {mt[(d * 3) * P], mt[(d * 3 + 1) * P], mt[(d * 3 + 2) * P]};
   const float4 ej = ejx[e];
+  const int td = STRETCH ? fx_shifts(ej).t(d) : 0;
+  const i64 Ja[3] = {fx_up(Jr[0], td), fx_up(Jr[1], td), fx_up(Jr[2], td)};
   int fso[3] = {-1, -1, -1};   // surface flux of the node, per direction
   double fsg[3] = {0, 0, 0};
 #pragma unroll
@@ -281,7 +284,7 @@ __device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* 
   if (!ex.ok) return false;
   const int eg = ((__double2hiint(g.inv_gm1) >> 20) & 0x7ff) - 1022;
   const int ek = ((__double2hiint(g.kappa) >> 20) & 0x7ff) - 1022;
-  const int q1 = 56 - ex.g - ex.e.u, q2 = 59 - ex.t - ek;   // of the viscous energy flux's two terms, + (-e_j)
+  const int q1 = 56 - ex.g - ex.e.u, q2 = 59 - ex.t - ek;   // of the viscous energy flux's two terms, + (-e_j + t_d)
   if (threadIdx.x == 3 * P - 1) {
     FxElem el = ex;
     fx_element_logs(el, s_mx, ej);
@@ -374,6 +377,7 @@ __device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* 
     FxSum s{0, 0};
 #pragma unroll
     for (int m = 0; m < n; ++m) fx_add(s, sD[r * n + m], fx_split(line[m * stride]));
+    if (td) fx_visc_down(s, td);
     sS[((5 + c) * 3 + d) * P + id] = make_longlong2(s.p, s.c >> 2);
   }
   __syncthreads();
@@ -392,6 +396,7 @@ __device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* 
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
     fx_fold(acc[c]);
+    if (td) fx_shift_down(acc[c], td);
     sS[(c * 3 + d) * P + id] = make_longlong2(acc[c].p, acc[c].c);
   }
   __syncthreads();
@@ -626,7 +631,7 @@ __device__ __forceinline__ void volume_lat_f64(const StageArgs& a, const double*
   }
 }
 
-template <int N>
+template <int N, bool STRETCH>
 __global__ void __launch_bounds__(LatShape<N>::THREADS, 2)
 k_volume_lat(StageArgs a, const double* __restrict__ metrics, const i64* __restrict__ jx,
              const float4* __restrict__ ejx, const double* __restrict__ grad, const double* __restrict__ fstar,
@@ -635,7 +640,7 @@ k_volume_lat(StageArgs a, const double* __restrict__ metrics, const i64* __restr
   extern __shared__ __align__(16) unsigned char lat_raw[];
   __shared__ double s_tc[2];
   if (g.visc_law != DG_VISC_SUTHERLAND) {
-    if (volume_lat_fx<N>(a, metrics, jx, ejx, grad, fstar, elem_face, mms, Dg, E, g, inv_w0, lat_raw, s_tc)) return;
+    if (volume_lat_fx<N, STRETCH>(a, metrics, jx, ejx, grad, fstar, elem_face, mms, Dg, E, g, inv_w0, lat_raw, s_tc)) return;
     __syncthreads();
   } else {
     wait_previous();
@@ -729,12 +734,18 @@ static cudaError_t lat_setup() {
   cudaError_t e = cudaFuncSetAttribute(k_lift_lat<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)lift_lat_smem_bytes<N>());
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_volume_lat<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(k_volume_lat<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)volume_lat_smem_bytes<N>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_volume_lat<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)volume_lat_smem_bytes<N>());
   // one split of L1 for the three, so that blocks of two of them fit on an SM at a time
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lift_lat<N>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_face_lat<N>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_volume_lat<N>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_volume_lat<N, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_volume_lat<N, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   return e;
 }
 
@@ -791,7 +802,7 @@ static cudaError_t lift_lat_N(const Ctx& c, const double* U, cudaStream_t s, boo
 
 template <int N>
 static cudaError_t volume_lat_N(const Ctx& c, const StageArgs& a, cudaStream_t s) {
-  return launch_lat<N>(c, k_volume_lat<N>, true, c.E, LatShape<N>::THREADS, volume_lat_smem_bytes<N>(), s, a, c.d_metrics,
+  return launch_lat<N>(c, c.fx_stretch ? k_volume_lat<N, true> : k_volume_lat<N, false>, true, c.E, LatShape<N>::THREADS, volume_lat_smem_bytes<N>(), s, a, c.d_metrics,
                        c.d_jx, c.d_ejx, (const double*)c.d_grad, (const double*)c.d_fstar, c.d_elem_face, c.d_mms, c.d_D,
                        c.E, c.gas, 1.0 / c.w[0]);
 }

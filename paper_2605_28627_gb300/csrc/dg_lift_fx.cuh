@@ -213,10 +213,12 @@ __device__ __forceinline__ void lift_body_fx(const double* __restrict__ U, const
   // g_l = (1/J) sum_d Ja^d_l dd_d
   const i64* mt = jx + (size_t)e * 10 * P + id;
   const Fx iJ = fx_split(mt[9 * P]);
-  const int qg = fx_lift_bits(eD, (int)ej.x, (int)ej.z);   // less e
+  const FxMetricShifts sh = fx_shifts(ej);
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
-    const Fx J[3] = {fx_split(mt[l * P]), fx_split(mt[(3 + l) * P]), fx_split(mt[(6 + l) * P])};
+    const int c = sh.c(l), qg = fx_lift_bits(eD, (int)ej.x - c, (int)ej.z);   // less e
+    const Fx J[3] = {fx_split(fx_up(mt[l * P], c)), fx_split(fx_up(mt[(3 + l) * P], c)),
+                     fx_split(fx_up(mt[(6 + l) * P], c))};
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
       const Fx x[3] = {fx_split(dd[a][0]), fx_split(dd[a][1]), fx_split(dd[a][2])};

@@ -107,9 +107,17 @@ __device__ __forceinline__ void fx_element_logs(FxElem& x, const int* mx, float4
   x.e.lb = fx_log_mantissa(bmin, 0) + (float)((bmin >> 20) - 1022 - x.e.b);
 }
 
+// s / 2^t of a viscous line sum, 0 <= t <= 15.
+__device__ __forceinline__ void fx_visc_down(FxSum& s, int t) {
+  s.c = (s.c >> t) + ((s.p & ((1 << t) - 1)) << (32 - t));
+  s.p >>= t;
+}
+
 // Returns whether the block holds elements that this body left to FP64
 // (s_state[le] = 2); all threads return the same value.
-template <int N, int EPB_, bool LIST>
+// STRETCH: the mesh may hold elements whose directions' metric terms are shifted
+// by different amounts (FxMetricShifts::t); without it every t is 0.
+template <int N, int EPB_, bool LIST, bool STRETCH>
 __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double* __restrict__ metrics,
                                                const i64* __restrict__ jx, const float4* __restrict__ ejx,
                                                const double* __restrict__ grad, const double* __restrict__ fstar,
@@ -125,6 +133,7 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
   i64* const tile0 = reinterpret_cast<i64*>(smem_raw) + B::tables;
   __shared__ int s_mx[EPB][kMxCount];
   __shared__ FxAlign s_al[EPB];
+  __shared__ int s_walk[EPB], s_shift[EPB];      // FxMetricShifts
   __shared__ Fx s_G;
   __shared__ double s_tc[2];                     // sin, cos of pi t (manufactured source)
   __shared__ uint64_t s_bar[EPB];
@@ -226,6 +235,7 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
   __syncthreads();   // maxima complete; every node has its state: the staging region is free
   if (active && id == 0) bulk_bar_inval(&s_bar[le]);
   const float4 ej = active ? ejx[e] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  const FxMetricShifts sh = fx_shifts(ej);
   FxElem ex = fx_element(s_mx[le], ej);
   const bool act = active && ex.ok;
   if (id == 0) {
@@ -233,6 +243,10 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
     if (act) {
       fx_element_logs(ex, s_mx[le], ej);
       s_al[le] = fx_align(ex.e, eg, fx_log_mantissa(__double2hiint(g.inv_gm1), 1), eD);
+    }
+    if constexpr (STRETCH) {
+      s_walk[le] = sh.walk();
+      s_shift[le] = sh.w;
     }
   }
   if (act) {
@@ -254,7 +268,11 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
     Fx T[3];
 #pragma unroll
     for (int l = 0; l < 3; ++l) T[l] = fx_split(fx_mul<4>(fx_split(fx_from(gr[9 + l], kFxQ - ex.t)), kap));
-    const int q1 = 56 - ex.g - ex.e.u, q2 = 59 - ex.t - ek;   // of the energy flux's two terms, + (-e_j)
+    const int q1 = 56 - ex.g - ex.e.u, q2 = 59 - ex.t - ek;   // of the energy flux's two terms, + (-e_j + t_d)
+    if constexpr (STRETCH) {
+#pragma unroll
+      for (int r = 0; r < 9; ++r) Ja[r] = fx_up(Ja[r], sh.t(r / 3));
+    }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       Fx J[3];
@@ -265,7 +283,7 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
       fx_add(f1, t01, J[0]); fx_add(f1, t11, J[1]); fx_add(f1, t12, J[2]);
       fx_add(f2, t02, J[0]); fx_add(f2, t12, J[1]); fx_add(f2, t22, J[2]);
       fx_add(h, T[0], J[0]); fx_add(h, T[1], J[1]); fx_add(h, T[2], J[2]);
-      const i64 v0 = fx_end<3>(f0), v1 = fx_end<3>(f1), v2 = fx_end<3>(f2);   // 58 - e_g - e_j
+      const i64 v0 = fx_end<3>(f0), v1 = fx_end<3>(f1), v2 = fx_end<3>(f2);   // 58 - e_g - e_j + t_d
       fx_add(en, fx_split(v0), U[0]); fx_add(en, fx_split(v1), U[1]); fx_add(en, fx_split(v2), U[2]);
       i64 ve = fx_end<2>(en), vh = fx_end<3>(h);
       ve >>= fx_clamp(q1 - q2);
@@ -292,10 +310,15 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
         const int r = ijk[d];
         const int stride = d == 0 ? 1 : (d == 1 ? n : NN);
         const i64* line = sFv + (d * 4 + c) * P + id - r * stride;
-        FxSum s{p, 0};
+        FxSum s{STRETCH ? 0 : p, 0};
 #pragma unroll
         for (int m = 0; m < n; ++m) fx_add(s, sD[r * n + m], fx_split(line[m * stride]));
-        p = s.p;
+        if constexpr (STRETCH) {
+          if (const int t = FxMetricShifts{s_shift[le]}.t(d)) fx_visc_down(s, t);
+          p += s.p;
+        } else {
+          p = s.p;
+        }
         f += s.c >> 2;
       }
       sA[c * P + id] = fx_to2<30>(p, f, c < 3 ? qv : qe);
@@ -341,8 +364,10 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
     reinterpret_cast<longlong2*>(xs)[P + at] = make_longlong2(F[2], F[3]);
     xs[4 * P + at] = F[4];
   };
+  // the directions by falling t, so that the sums are only shifted down on the way
 #pragma unroll 1
-  for (int d = 0; d < 3; ++d) {
+  for (int x = 0; x < 3; ++x) {
+    const int d = STRETCH ? s_walk[le] >> (2 * x) & 3 : x;
     const int r = d == 0 ? i : (d == 1 ? j : k);
     const int stride = d == 0 ? 1 : (d == 1 ? n : NN);
     const int line0 = id - r * stride;
@@ -357,7 +382,7 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
     };
     // exchange buffers: a direction's first writes wait for the previous
     // direction's last reads (different lines)
-    if (d > 0) dsync(d);
+    if (x > 0) dsync(d);
 #pragma unroll 1
     for (int s = 1; s <= FULL; ++s) {
       const int m = r + s < n ? r + s : r + s - n;
@@ -391,12 +416,14 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
         le2 = t / (P / 2); w2 = t - le2 * (P / 2); take = t < EPB * (P / 2);
       }
       if (take && s_state[le2] == 1) {
-        const int hi = w2 / stride;
-        const int ia = w2 - hi * stride + stride * (hi % H + n * (hi / H));
-        const int ib = ia + H * stride;
+        const int d2 = STRETCH && SCOPE == 0 && EPB > 1 ? s_walk[le2] >> (2 * x) & 3 : d;   // the pair's own element's
+        const int st2 = d2 == 0 ? 1 : (d2 == 1 ? n : NN);
+        const int hi = w2 / st2;
+        const int ia = w2 - hi * st2 + st2 * (hi % H + n * (hi / H));
+        const int ib = ia + H * st2;
         i64* b2 = tile0 + le2 * PER_ELEM;
         i64 F[5];
-        pair(b2, le2, d, ia, ib, F);
+        pair(b2, le2, d2, ia, ib, F);
         i64* xh = b2 + 10 * P + 3 * JW + (XB > 1 ? FULL * XW : 0);
         put(xh, ia, F);
         put(xh, ib, F);
@@ -417,6 +444,12 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
     }
 #pragma unroll
     for (int c = 0; c < 5; ++c) fx_fold(acc[c]);
+    if constexpr (STRETCH) {
+      if (const int down = s_walk[le] >> (8 + 4 * x) & 15) {
+#pragma unroll
+        for (int c = 0; c < 5; ++c) fx_shift_down(acc[c], down);
+      }
+    }
   }
   int bad = 0;
 #pragma unroll
@@ -468,7 +501,7 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
 // The FP64 volume body: fixed point, then FP64 for the elements outside its
 // range (density or beta varying by more than a factor 8 to 16 inside the
 // element, non-finite or non-positive values), which the same block redoes.
-template <int N, int EPB, bool LIST = false>
+template <int N, int EPB, bool LIST = false, bool STRETCH = true>
 __device__ __forceinline__ void volume_body_f64(const StageArgs& a, const double* __restrict__ metrics,
                                                 const i64* __restrict__ jx, const float4* __restrict__ ejx,
                                                 const double* __restrict__ grad, const double* __restrict__ fstar,
@@ -476,7 +509,8 @@ __device__ __forceinline__ void volume_body_f64(const StageArgs& a, const double
                                                 const double* __restrict__ Dg, int E, const Gas& g, double inv_w0,
                                                 int blk) {
   __shared__ int s_state[EPB];   // 0: no element, 1: done in fixed point, 2: left to FP64
-  if (volume_body_fx<N, EPB, LIST>(a, metrics, jx, ejx, grad, fstar, elem_face, mms, Dg, E, g, inv_w0, blk, s_state)) {
+  if (volume_body_fx<N, EPB, LIST, STRETCH>(a, metrics, jx, ejx, grad, fstar, elem_face, mms, Dg, E, g, inv_w0, blk,
+                                            s_state)) {
     __syncthreads();
     volume_body<N, double, EPB, LIST>(a, metrics, metrics, grad, fstar, elem_face, mms, Dg, E, g, inv_w0, blk,
                                       s_state);

@@ -42,14 +42,15 @@ static void flux(T ra, T rb, const T* ua, const T* ub, T ba, T bb, const T* sn, 
 extern "C" {
 
 // Pairs with density in [r0, r1], pressure in [p0, p1], velocities below um,
-// metric terms below jm (axis: one component only), gamma.  out[0..2]: rms
+// metric terms below jm (axis: one component only) in an element whose largest
+// are 2^t0 loose times as large, gamma.  out[0..2]: rms
 // error of the fixed-point mass, momentum and energy flux over the rms flux,
 // out[3..5]: the same of FP64, out[6]: largest |F| as log2, out[7]: pairs
 // outside the range.
 void check_pairs(int count, double r0, double r1, double p0, double p1, double um, double jm, int axis, double gamma,
-                 double* out) {
+                 int t0, double loose, double* out) {
   srand48(11);
-  const double ig = 1.0 / (gamma - 1.0), jl = axis ? jm : 3 * jm, bmax = r1 / (8 * p0);
+  const double ig = 1.0 / (gamma - 1.0), jl = loose * (axis ? jm : 3 * jm), bmax = r1 / (8 * p0);
   FxExp e{expo(r1), expo(um), expo(bmax), expo(jl), 0, 0, 0, 0};
   const double bmin = std::max(r0 / (8 * p1), ldexp(1.0, e.b - 4));
   e.lr = (float)(log2(r1) - e.r + 1e-3);
@@ -82,7 +83,7 @@ void check_pairs(int count, double r0, double r1, double p0, double p1, double u
     double ka = 0, kb = 0;
     for (int a = 0; a < 3; ++a) {
       su[a] = fx_from(ua[a], 60 - e.u) + fx_from(ub[a], 60 - e.u);
-      n2[a] = fx_from(na[a], 60 - e.j) + fx_from(nb[a], 60 - e.j);
+      n2[a] = fx_up(fx_from(na[a], 60 - e.j - t0), t0) + fx_up(fx_from(nb[a], 60 - e.j - t0), t0);
       ka += ua[a] * ua[a]; kb += ub[a] * ub[a];
     }
     i64 F[5];
@@ -114,9 +115,10 @@ void check_pairs(int count, double r0, double r1, double p0, double p1, double u
 }
 
 // Lifted gradients of one field along a line of n nodes, D [n][n], half = 1/(2
-// w_0): g = (1/J_el) J (D phi + jump), the other two derivatives 0.  out: rms
+// w_0): g = (1/J_el) J (D phi + jump), the element's largest metric term 2^c
+// times as large as this one, the other two derivatives 0.  out: rms
 // error of the fixed-point and of the FP64 arithmetic over the rms gradient.
-void check_lifting(int count, int n, const double* D, int eD, double half, double* out) {
+void check_lifting(int count, int n, const double* D, int eD, double half, int c, double* out) {
   srand48(14);
   double ef = 0, ed = 0, sc = 0;
   for (int t = 0; t < count; ++t) {
@@ -127,7 +129,7 @@ void check_lifting(int count, int n, const double* D, int eD, double half, doubl
     const double nbr[2] = {phi[0] + uniform(-1e-3, 1e-3), phi[n - 1] + uniform(-1e-3, 1e-3)};
     top = std::max(top, std::max(std::fabs(nbr[0]), std::fabs(nbr[1])));
     const int e = expo(top), ej = expo(J), ei = expo(iJ);
-    const Fx Jx[3] = {fx_split(fx_from(J, kFxQ - ej)), fx_split(0), fx_split(0)}, iJx = fx_split(fx_from(iJ, 62 - ei));
+    const Fx Jx[3] = {fx_split(fx_up(fx_from(J, kFxQ - ej - c), c)), fx_split(0), fx_split(0)}, iJx = fx_split(fx_from(iJ, 62 - ei));
     for (int r = 0; r < n; ++r) {
       const bool edge = r == 0 || r == n - 1;
       const double hs = r == 0 ? -half : half, nb = nbr[r != 0];

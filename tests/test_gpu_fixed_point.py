@@ -154,3 +154,112 @@ def test_gauss_nodes(orc, N, scale):
     U = random_state(mesh.n_elems, N, seed=550 + N, rho=(0.95, 1.05), vel=0.2, p=(0.95, 1.05)) * scale
     err = _err(s.time_derivative(_cuda(U)).cpu().numpy(), o.time_derivative(U))
     assert (err < 1e-11).all(), err
+
+
+def _stretched(K, N, sizes, seed):
+    """Cartesian box of K^3 cells of the given sizes, frames turned at random."""
+    mesh = box_mesh(K, 1, rotate_seed=seed)
+    mesh.xgeo *= np.array(sizes)[None, :, None, None, None] * K / 2.0
+    return mesh
+
+
+def _axis_flow(s, mesh, N, L, ax, comp):
+    """Density, velocity component comp and pressure vary along axis ax only; the
+    same to the last bit at the nodes of different elements that coincide."""
+    X = s.node_coords().cpu().numpy().reshape(mesh.n_elems, 3, N + 1, N + 1, N + 1)
+    y = 2.0 * np.pi * np.round(X[:, ax] / L * 2.0 ** 36) * 2.0 ** -36
+    rho, vel, p = 1.0 + 0.2 * np.sin(y), 0.5 + 0.3 * np.cos(y), 1.0 + 0.2 * np.sin(y + 1.0)
+    U = np.zeros((mesh.n_elems, 5, N + 1, N + 1, N + 1))
+    U[:, 0], U[:, 1 + comp], U[:, 4] = rho, rho * vel, p / 0.4 + 0.5 * rho * vel ** 2
+    return U
+
+
+# in fixed point with the directions shifted by 1 and 4, and in FP64
+CELLS = [(3.0, 1.0, 24.0), (1.0, 10.0, 1000.0)]
+
+
+LGL = [(1, 3, 0), (1, 13, 0), (2, 3, 0), (3, 3, 0), (3, 7, 0), (4, 3, 0), (5, 3, 0), (7, 2, 0), (8, 2, 0)]
+LG = [(1, 3, 1), (3, 3, 1), (4, 2, 1), (6, 2, 1)]
+
+
+@pytest.mark.parametrize("N,K,nodes,k", [c + (k,) for c in LGL + LG for k in (1, 4, 5, 20) if not c[2] or k <= 5])
+def test_flow_along_stretched_cells(N, K, nodes, k):
+    """Cells 2^k times as long along an axis as across it and an inviscid flow
+    that varies along this axis: every term of the mass, energy and axis momentum
+    equations is 2^-k times that on cubic cells, and so is its rounding, as there
+    is no flow in the directions with the larger metric terms.  Bar 1e-13 of max
+    |R|: the rounding of both evaluations.  On Gauss nodes 3e-13 and k up to 5: the
+    face values are rounded sums, whose jumps at the long faces enter 2^k times."""
+    import paper_2605_28627_gb300 as dg
+    ax = (N + k) % 3
+    R = []
+    for long in (1.0, 2.0 ** k):
+        mesh = _stretched(K, N, [long if a == ax else 1.0 for a in range(3)], 470 + N)
+        s = dg.Solver(mesh, N, mu=0.0, nodes=nodes)
+        if long == 1.0:
+            U = _axis_flow(s, mesh, N, K, ax, ax)
+        R.append(long * s.time_derivative(_cuda(U)).cpu().numpy()[:, [0, 1 + ax, 4]])
+    d = np.abs(R[1] - R[0]).max(axis=(0, 2, 3, 4)) / np.abs(R[0]).max(axis=(0, 2, 3, 4))
+    assert (d < (3e-13 if nodes else 1e-13)).all(), d
+
+
+@pytest.mark.parametrize("N,K,nodes", LGL + [(9, 2, 0)] + LG)
+@pytest.mark.parametrize("k", [1, 4, 5, 20])
+def test_gradients_along_stretched_cells(orc, N, K, nodes, k):
+    """The same cells with a transverse velocity that varies along the axis:
+    the dissipation is a sum of squares of its lifted gradient, which the rounding
+    in the other directions enters as a square.  Bar 2e-13."""
+    import paper_2605_28627_gb300 as dg
+    ax = (N + k) % 3
+    mesh = _stretched(K, N, [2.0 ** k if a == ax else 1.0 for a in range(3)], 470 + N)
+    o, s = orc.Oracle(mesh, N, mu=0.01, nodes=nodes), dg.Solver(mesh, N, mu=0.01, nodes=nodes)
+    U = _axis_flow(s, mesh, N, K * 2.0 ** k, ax, (ax + 1) % 3)
+    got, ref = s.integrals(_cuda(U))[6], o.integrals(U)[6]
+    assert abs(got - ref) <= 2e-13 * ref, (got, ref)
+
+
+@pytest.mark.parametrize("N,K,nodes", LGL + LG)
+@pytest.mark.parametrize("cells", CELLS)
+def test_stretched_cells(orc, N, K, nodes, cells):
+    """A random state on stretched cells."""
+    import paper_2605_28627_gb300 as dg
+    mesh = _stretched(K, N, cells, 475 + N)
+    kw = dict(mu=0.02, nodes=nodes)
+    o, s = orc.Oracle(mesh, N, **kw), dg.Solver(mesh, N, **kw)
+    mild = dict(rho=(0.95, 1.05), vel=0.2, p=(0.95, 1.05)) if nodes else {}   # admissible at the face points too
+    U = random_state(mesh.n_elems, N, seed=580 + N, **mild)
+    err = _err(s.time_derivative(_cuda(U)).cpu().numpy(), o.time_derivative(U))
+    assert (err < 1e-11).all() if nodes else (err < 1e-12).all(), err
+
+
+@pytest.mark.parametrize("N", [1, 3, 5, 7])
+@pytest.mark.parametrize("cells", CELLS)
+def test_vjp_on_stretched_cells(orc, N, cells):
+    """As test_vjp."""
+    import paper_2605_28627_gb300 as dg
+    mesh = _stretched(2, N, cells, 480 + N)
+    o, s = orc.Oracle(mesh, N, mu=0.02), dg.Solver(mesh, N, mu=0.02)
+    U = random_state(mesh.n_elems, N, seed=590 + N)
+    rng = np.random.default_rng(690 + N)
+    w, v = rng.normal(size=U.shape), rng.normal(size=U.shape)
+    _, Jw = o.time_derivative_tl(U, w, 0.0)
+    JTv = s.time_derivative_vjp(_cuda(U), _cuda(v)).cpu().numpy()
+    lhs, rhs = float((JTv * w).sum()), float((v * Jw).sum())
+    assert abs(lhs - rhs) <= 1e-11 * float(np.abs(JTv * w).sum()), (lhs, rhs)
+
+
+@pytest.mark.parametrize("N", [1, 3, 4])
+def test_ensemble_with_stretched_member(N):
+    """An FP64 ensemble of a cubic and a stretched mesh: the tile-table kernels
+    against each member stepped alone."""
+    import paper_2605_28627_gb300 as dg
+    meshes = [box_mesh(4, 1), _stretched(3, N, CELLS[0], 490 + N)]
+    solvers = [dg.Solver(m, N, mu=0.01) for m in meshes]
+    U = [_cuda(random_state(m.n_elems, N, seed=600 + i)) for i, m in enumerate(meshes)]
+    ref = [u.clone() for u in U]
+    dt = 1e-3 / (N + 1) ** 2
+    for s, u in zip(solvers, ref):
+        s.rk_step(u, torch.empty_like(u), 0.0, dt, 2)
+    dg.Ensemble(solvers).step(U, [torch.empty_like(u) for u in U], [0.0] * 2, [dt] * 2, 2)
+    for a, b in zip(U, ref):
+        assert float((a - b).abs().max()) <= 1e-13 * float(b.abs().max())
