@@ -317,8 +317,10 @@ __device__ __forceinline__ bool adj_pairs_fx(const double* __restrict__ U, const
 #pragma unroll
     for (int c = 0; c < 5; ++c) lv[c] = -lam[((size_t)e * 5 + c) * P + id] * iJ;
     const int hr = max(__double2hiint(rho), 0), hb = max(__double2hiint(bt), 0);
-    int m[kCount] = {hr, 0x7fffffff - hr, hb, 0x7fffffff - hb, max(max(fx_mag(u), fx_mag(v)), fx_mag(w)), fx_mag(lv[0]),
-                     max(max(fx_mag(lv[1]), fx_mag(lv[2])), fx_mag(lv[3])), fx_mag(lv[4])};
+    // the last bit set if any of the low word is: a subnormal adjoint is not zero
+    auto mag = [](double x) { return fx_mag(x) | (__double2loint(x) != 0); };
+    int m[kCount] = {hr, 0x7fffffff - hr, hb, 0x7fffffff - hb, max(max(mag(u), mag(v)), mag(w)), mag(lv[0]),
+                     max(max(mag(lv[1]), mag(lv[2])), mag(lv[3])), mag(lv[4])};
     fx_maxima<kCount>(le, s_mx[le], m);
   }
   __syncthreads();
@@ -326,12 +328,13 @@ __device__ __forceinline__ bool adj_pairs_fx(const double* __restrict__ U, const
   const float4 ej = active ? ejx[e] : make_float4(1000.0f, 0.0f, 0.0f, 0.0f);
   const FxMetricShifts sh = fx_shifts(ej);
   FxExp x{fx_expo(mx[kR]), fx_expo(mx[kU]), fx_expo(mx[kB]), (int)ej.x, 0.0f, 0.0f, 0.0f, 0.0f};
-  x.u = max(x.u, ((-x.b) >> 1) - 40);   // 2^-40 of the speed of sound
   const int l0 = fx_expo(mx[kL0]), lm = fx_expo(mx[kLm]), l4 = fx_expo(mx[kL4]);
   const int rmin = 0x7fffffff - mx[kRmin], bmin = 0x7fffffff - mx[kBmin];
   const int dr = x.r - ((rmin >> 20) - 1023), db = x.b - ((bmin >> 20) - 1023);
-  const bool act = active && rmin > 0 && bmin > 0 && dr <= 4 && db <= 4 && x.r < 60 && x.b < 60 && x.u < 60 && x.j < 60 &&
-                   l0 < 60 && lm < 60 && l4 < 60 && x.r > -60 && x.b > -60 && x.u > -60 && x.j > -60;
+  auto in = [](int v) { return v > -60 && v < 60; };
+  const bool act = active && rmin > 0 && bmin > 0 && dr <= 4 && db <= 4 && in(x.r) && in(x.b) && in(x.j) &&
+                   fx_in_range(mx[kU], 60) && fx_in_range(mx[kL0], 60) && fx_in_range(mx[kLm], 60) &&
+                   fx_in_range(mx[kL4], 60);
   if (id == 0) {
     state[le] = active ? (act ? 1 : 2) : 0;
     if (act) {

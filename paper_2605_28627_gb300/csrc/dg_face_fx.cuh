@@ -9,7 +9,7 @@
 // -> now: N = 1 24 -> 18, 3 73 -> 47, 5 147 -> 92, 7 257 -> 149, 9 397 -> 226.
 #pragma once
 
-#include "dg_fixed.cuh"
+#include "dg_fx_metrics.cuh"
 #include "dg_stage.cuh"
 
 namespace dg {
@@ -66,8 +66,8 @@ __device__ __forceinline__ bool face_visc_fx(const double* __restrict__ gL, cons
       mu = max(mu, mag(s ? uR[l] : uL[l]));
     }
   }
-  const int eg = max((mg >> 20) - 1022, -90), et = max((mt >> 20) - 1022, -90), eu = max((mu >> 20) - 1022, -90);
-  if (eg >= 90 || et >= 90 || eu >= 90) return false;
+  if (!fx_in_range(mg, 90) || !fx_in_range(mt, 90) || !fx_in_range(mu, 90)) return false;
+  const int eg = fx_expo(mg), et = fx_expo(mt), eu = fx_expo(mu);
   Fx n[3];
 #pragma unroll
   for (int l = 0; l < 3; ++l) n[l] = fx_split(fx_from(nv[l], 60));

@@ -11,9 +11,18 @@ namespace dg {
 // corners), per degree: at most 0.5, 2.0, 4.05, 6.76, 10.2, 14.3, 19.0, 24.4, 30.5.
 constexpr int fx_eD(int N) { return N == 1 ? 0 : (N == 2 ? 2 : (N <= 4 ? 3 : (N <= 6 ? 4 : 5))); }
 
-__device__ __forceinline__ int fx_expo(int h) {   // |x| < 2^e from the high word of the largest |x|
+// |x| < 2^e from the high word of the largest |x|; a quantity that is zero all
+// over the element gets kFxLow.
+constexpr int kFxLow = -200;
+__host__ __device__ __forceinline__ int fx_expo(int h) {
   const int e = (h >> 20) - 1022;
-  return e > -90 ? e : -90;
+  return e > kFxLow ? e : kFxLow;
+}
+// Whether fixed point may hold the quantity: zero, or 2^kFxLow <= 2^e < 2^high
+// (scaled below 2^kFxLow it would lose digits).
+__host__ __device__ __forceinline__ bool fx_in_range(int h, int high) {
+  const int e = (h >> 20) - 1022;
+  return h == 0 || (e >= kFxLow && e < high);
 }
 __device__ __forceinline__ int fx_mag(double x) { return __double2hiint(x) & 0x7fffffff; }
 // maxima of v[0..C) over the lanes of element el of this warp, into mx[0..C)

@@ -103,7 +103,7 @@ __device__ __forceinline__ bool lift_lg_fx(const double* __restrict__ U, const d
   __syncthreads();
   const int eu = fx_expo(s_mx[le][0]), et = fx_expo(s_mx[le][1]);
   const float4 ej = active ? ejx[e] : make_float4(1000.0f, 0.0f, 0.0f, 0.0f);
-  const bool act = active && eu < 90 && et < 90 && ej.x < 90.0f;
+  const bool act = active && fx_in_range(s_mx[le][0], 90) && fx_in_range(s_mx[le][1], 90) && ej.x < 90.0f;
   if (id == 0) state[le] = active ? (act ? 1 : 2) : 0;
   i64 Ja[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, iJ = 0;
   Fx X[4];
@@ -277,7 +277,7 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
         val = -fstar[((size_t)fid * 5 + v2) * NN + p2 + n * q2];
       }
       sFs[(f * 5 + v2) * NN + pq] = __double_as_longlong(val);
-      const int mv = fx_mag(val) + (sh.t(f >> 1) << 20);   // of val 2^t, as it is held below
+      const int hv = fx_mag(val), mv = hv ? hv + (sh.t(f >> 1) << 20) : 0;   // of val 2^t, as it is held below
       if (v2 == 0) m[kF0] = max(m[kF0], mv);
       else if (v2 == 4) m[kFe] = max(m[kFe], mv);
       else m[kFm] = max(m[kFm], mv);
@@ -285,14 +285,16 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
     fx_maxima<kCount>(le, s_mx[le], m);
   }
   __syncthreads();
-  int x[kCount], top = -90;
+  int x[kCount];
+  bool in = true;
 #pragma unroll
   for (int c = 0; c < kCount; ++c) {
     x[c] = fx_expo(s_mx[le][c]);
-    top = max(top, x[c]);
+    in = in && fx_in_range(s_mx[le][c], 90);
   }
-  const int ej = (int)ejv.x, em = fx_expo(fx_mag(g.mu)), el = fx_expo(fx_mag(g.mu * g.kappa));
-  const bool act = active && top < 90 && ej < 90;
+  const int ej = (int)ejv.x, hm = fx_mag(g.mu), hl = fx_mag(g.mu * g.kappa);
+  const int em = fx_expo(hm), el = fx_expo(hl);
+  const bool act = active && in && ej < 90 && fx_in_range(hm, 90) && fx_in_range(hl, 90);
   if (id == 0) state[le] = active ? (act ? 1 : 2) : 0;
   // bits after the point of the mass (q0), momentum (qm) and energy (qe) fluxes,
   // + t_d in direction d: below 2^61.3, so that six of a line's n + 2 terms fit in FxSum's c (the part of

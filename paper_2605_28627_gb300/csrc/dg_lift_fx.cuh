@@ -24,7 +24,7 @@ constexpr size_t lift_fx_smem_bytes() {
 }
 
 // MORTAR as in lift_body.  Elements outside the fixed-point range (a
-// non-finite state, exponents beyond 2^90, e_j = 1000) get lift_body's FP64
+// non-finite state, velocity or temperature outside 2^kFxLow to 2^90, e_j = 1000) get lift_body's FP64
 // arithmetic from the same block.
 template <int N, int EPB, bool MORTAR = false>
 __device__ __forceinline__ void lift_body_fx(const double* __restrict__ U, const double* __restrict__ metrics,
@@ -115,10 +115,9 @@ __device__ __forceinline__ void lift_body_fx(const double* __restrict__ U, const
   }
   __syncthreads();
   // exponents of velocity and temperature; range of the element
-  auto expo = [&](int h) { const int x = (h >> 20) - 1022; return x > -90 ? x : -90; };
-  const int eu = expo(s_mx[le][0]), et = expo(s_mx[le][1]);
+  const int eu = fx_expo(s_mx[le][0]), et = fx_expo(s_mx[le][1]);
   const float4 ej = active ? ejx[e] : make_float4(1000.0f, 0.0f, 0.0f, 0.0f);
-  const bool ok = eu < 90 && et < 90 && ej.x < 90.0f;
+  const bool ok = fx_in_range(s_mx[le][0], 90) && fx_in_range(s_mx[le][1], 90) && ej.x < 90.0f;
   if (active) {
     if (ok) {
       sphi[le * 2 * P + id] = make_longlong2(fx_from(phi[0], kFxQ - eu), fx_from(phi[1], kFxQ - eu));
@@ -141,8 +140,8 @@ __device__ __forceinline__ void lift_body_fx(const double* __restrict__ U, const
       i64* sj = sjmp + (le2 * 6 + f) * 4 * NN + pq;
       const longlong2 p0 = sphi[le2 * 2 * P + node], p1 = sphi[(le2 * 2 + 1) * P + node];
       const i64 own[4] = {p0.x, p0.y, p1.x, p1.y};
-      const int eu2 = expo(s_mx[le2][0]), et2 = expo(s_mx[le2][1]);
-      if (eu2 < 90 && et2 < 90 && ejx[blk * EPB + le2].x < 90.0f) {
+      const int eu2 = fx_expo(s_mx[le2][0]), et2 = fx_expo(s_mx[le2][1]);
+      if (fx_in_range(s_mx[le2][0], 90) && fx_in_range(s_mx[le2][1], 90) && ejx[blk * EPB + le2].x < 90.0f) {
         const Fx hx = fx_split(fx_round(hs, kFxQD - eD));
 #pragma unroll
         for (int a = 0; a < 4; ++a)

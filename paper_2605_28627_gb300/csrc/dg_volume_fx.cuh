@@ -86,23 +86,21 @@ __device__ __forceinline__ FxElem fx_element(const int* mx, float4 ej) {
   x.e.r = (r >> 20) - 1022;
   x.e.b = (b >> 20) - 1022;
   const int dr = x.e.r - ((rmin >> 20) - 1023), db = x.e.b - ((bmin >> 20) - 1023);
-  const int u = (mx[kMxU] >> 20) - 1022, ufloor = ((-x.e.b) >> 1) - 40;   // 2^-40 of the speed of sound
-  x.e.u = u > ufloor ? u : ufloor;
+  x.e.u = fx_expo(mx[kMxU]);
   x.e.j = (int)ej.x;
-  const int g = (mx[kMxG] >> 20) - 1022, t = (mx[kMxT] >> 20) - 1022;
-  x.g = g > -90 ? g : -90;
-  x.t = t > -90 ? t : -90;
+  x.g = fx_expo(mx[kMxG]);
+  x.t = fx_expo(mx[kMxT]);
   auto in = [](int v) { return v > -90 && v < 90; };
-  x.ok = rmin > 0 && bmin > 0 && dr <= 4 && db <= 4 && in(x.e.r) && in(x.e.b) && in(x.e.u) && in(x.e.j) &&
-         x.g < 90 && x.t < 90;
+  x.ok = rmin > 0 && bmin > 0 && dr <= 4 && db <= 4 && in(x.e.r) && in(x.e.b) && in(x.e.j) &&
+         fx_in_range(mx[kMxU], 90) && fx_in_range(mx[kMxG], 90) && fx_in_range(mx[kMxT], 90);
   x.e.lr = x.e.lu = x.e.lj = x.e.lb = 0.0f;
   return x;
 }
 // the logarithms too (one thread per element)
 __device__ __forceinline__ void fx_element_logs(FxElem& x, const int* mx, float4 ej) {
-  const int bmin = 0x7fffffff - mx[kMxBmin], u = (mx[kMxU] >> 20) - 1022;
+  const int bmin = 0x7fffffff - mx[kMxBmin];
   x.e.lr = fx_log_mantissa(mx[kMxR], 1);
-  x.e.lu = x.e.u == u ? fx_log_mantissa(mx[kMxU], 1) : 0.0f;
+  x.e.lu = mx[kMxU] != 0 ? fx_log_mantissa(mx[kMxU], 1) : 0.0f;
   x.e.lj = ej.y;
   x.e.lb = fx_log_mantissa(bmin, 0) + (float)((bmin >> 20) - 1022 - x.e.b);
 }

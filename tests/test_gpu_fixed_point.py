@@ -263,3 +263,89 @@ def test_ensemble_with_stretched_member(N):
     dg.Ensemble(solvers).step(U, [torch.empty_like(u) for u in U], [0.0] * 2, [dt] * 2, 2)
     for a, b in zip(U, ref):
         assert float((a - b).abs().max()) <= 1e-13 * float(b.abs().max())
+
+
+@pytest.mark.parametrize("N", [1, 3, 4, 7])
+@pytest.mark.parametrize("k", [-100, -150, -400, 100])
+def test_vjp_scales_with_the_cotangent(N, k):
+    """The VJP is linear in the cotangent: scaled by a power of two it scales to
+    the last bit where the exponents move with it, and to rounding (1e-12) where
+    they leave the fixed-point range and FP64 takes over."""
+    import paper_2605_28627_gb300 as dg
+    mesh = box_mesh(2, min(N, 4), deform="sinprod", rotate_seed=600 + N)
+    s = dg.Solver(mesh, N, mu=0.02)
+    U = _cuda(random_state(mesh.n_elems, N, seed=610 + N))
+    v = _cuda(np.random.default_rng(620 + N).normal(size=tuple(U.shape)))
+    dm = [torch.zeros(1, dtype=torch.float64, device="cuda") for _ in range(2)]
+    ref = s.time_derivative_vjp(U, v, None, dm[0])
+    got = s.time_derivative_vjp(U, v * 2.0 ** k, None, dm[1]) * 2.0 ** -k
+    assert float((got - ref).abs().max()) <= (0.0 if k < 0 and k > -180 else 1e-12) * float(ref.abs().max())
+    assert abs(float(dm[1]) * 2.0 ** -k - float(dm[0])) <= 1e-10 * abs(float(dm[0]))
+
+
+@pytest.mark.parametrize("N", [1, 3, 5])
+def test_vjp_at_low_speed(orc, N):
+    """Velocities of 1e-22 of the sound speed and a cotangent of the mass equation
+    alone, equal at every node of an element face's both sides: the adjoint of the
+    density is proportional to the velocity."""
+    import paper_2605_28627_gb300 as dg
+    mesh = box_mesh(2, 1)
+    o, s = orc.Oracle(mesh, N), dg.Solver(mesh, N)
+    U = random_state(mesh.n_elems, N, seed=630 + N, rho=(1.0, 1.0), p=(1.0, 1.0), vel=1e-22)
+    X = s.node_coords().cpu().numpy().reshape(mesh.n_elems, 3, N + 1, N + 1, N + 1)
+    v, w = np.zeros_like(U), np.zeros_like(U)
+    v[:, 0] = np.sin(np.pi * np.round(X[:, 0] * 2.0 ** 40) * 2.0 ** -40)
+    w[:, 0] = np.random.default_rng(640 + N).normal(size=w[:, 0].shape)
+    w[:, 0, [0, -1]] = w[:, 0, :, [0, -1]] = w[:, 0, :, :, [0, -1]] = 0.0   # interior nodes (none at N = 1)
+    JTv = s.time_derivative_vjp(_cuda(U), _cuda(v)).cpu().numpy()
+    _, Jw = o.time_derivative_tl(U, w, 0.0)
+    lhs, rhs = float((JTv * w).sum()), float((v * Jw).sum())
+    assert abs(lhs - rhs) <= 1e-11 * float(np.abs(JTv * w).sum()), (lhs, rhs)
+
+
+@pytest.mark.parametrize("N,K,nodes", [(1, 3, 0), (3, 3, 0), (3, 7, 0), (5, 3, 0), (7, 2, 0), (1, 3, 1), (3, 3, 1), (6, 2, 1)])
+@pytest.mark.parametrize("vel", [1e-12, 1e-22, 1e-40, 1e-80])
+def test_low_speed(orc, N, K, nodes, vel):
+    """Uniform density and pressure, velocities far below the sound speed: mass
+    and energy of R(U) and the dissipation follow the velocity down to any size."""
+    import paper_2605_28627_gb300 as dg
+    mesh = box_mesh(K, min(N, 4), deform="sinprod", rotate_seed=650 + N)
+    U = random_state(mesh.n_elems, N, seed=660 + N, rho=(1.0, 1.0), p=(1.0, 1.0), vel=vel)
+    U[:, 4] = 2.5   # the kinetic energy is below the rounding of p / 0.4
+    if not nodes:
+        # inviscid, as the conduction of the temperature's rounding is larger; on Gauss
+        # nodes the face values of density and energy are rounded sums, whose jumps
+        # LLF multiplies by the sound speed
+        o, s = orc.Oracle(mesh, N), dg.Solver(mesh, N)
+        err = _err(s.time_derivative(_cuda(U)).cpu().numpy(), o.time_derivative(U))
+        assert (err[[0, 4]] < 1e-12).all(), err
+    kw = dict(mu=0.01, nodes=nodes)
+    got, ref = dg.Solver(mesh, N, **kw).integrals(_cuda(U))[6], orc.Oracle(mesh, N, **kw).integrals(U)[6]
+    assert abs(got - ref) <= 1e-12 * ref, (got, ref)
+
+
+@pytest.mark.parametrize("N,K,nodes", [(1, 3, 0), (3, 3, 0), (3, 7, 0), (5, 3, 0), (1, 3, 1), (3, 3, 1), (6, 2, 1)])
+@pytest.mark.parametrize("k", [-120, -240])
+def test_cold_gas_at_rest(orc, N, K, nodes, k):
+    """Pressure and temperature scaled by 2^k at unit density, no flow: the energy
+    equation is heat conduction alone, in proportion."""
+    import paper_2605_28627_gb300 as dg
+    mesh = box_mesh(K, 1, rotate_seed=670 + N)
+    kw = dict(mu=1.0, nodes=nodes)
+    o, s = orc.Oracle(mesh, N, **kw), dg.Solver(mesh, N, **kw)
+    U = random_state(mesh.n_elems, N, seed=680 + N, rho=(1.0, 1.0), p=(0.95, 1.05), vel=0.0)
+    U[:, 4] *= 2.0 ** k
+    R, ref = s.time_derivative(_cuda(U)).cpu().numpy()[:, 4], o.time_derivative(U)[:, 4]
+    assert np.abs(R - ref).max() < (1e-11 if nodes else 1e-12) * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("N", [1, 3, 6])
+@pytest.mark.parametrize("k", [-100, -150, -250])
+def test_gauss_nodes_scaled_down(N, k):
+    """Density, pressure and viscosity scaled by 2^k: R(U) scales to the last bit
+    where the exponents move with it, and to rounding in FP64."""
+    import paper_2605_28627_gb300 as dg
+    mesh = box_mesh(3, min(N, 4), deform="sinprod", rotate_seed=690 + N)
+    U = _cuda(random_state(mesh.n_elems, N, seed=700 + N, rho=(0.95, 1.05), vel=0.2, p=(0.95, 1.05)))
+    R = [dg.Solver(mesh, N, mu=0.01 * 2.0 ** x, nodes=dg.NODES_LG).time_derivative(U * 2.0 ** x) * 2.0 ** -x for x in (0, k)]
+    assert float((R[1] - R[0]).abs().max()) <= (0.0 if k > -180 else 1e-12) * float(R[0].abs().max())
