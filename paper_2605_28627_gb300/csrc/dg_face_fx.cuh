@@ -14,14 +14,17 @@
 
 namespace dg {
 
-// Sound speed sqrt(x), x > 0 normal: reciprocal square root by the hardware
-// approximation (2^-20) and one step of third order.
+// Sound speed sqrt(x).  For positive normal x: c = x y from the hardware's
+// approximation y of 1/sqrt(x) (2^-20), corrected to third order from the exact
+// residual x - c^2, sqrt(x) = c + (x - c^2) y/2 (1 + 3/4 e), e = 1 - c y; within 0.55
+// ulp, 6 FP64 operations.  Zero, subnormal, infinite and negative values (a gas
+// without pressure has c = 0, while y would be infinite) take sqrt().
 __device__ __forceinline__ double sqrt_op(double x) {
+  if ((unsigned)__double2hiint(x) - 0x00100000u >= 0x7fe00000u) return sqrt(x);
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double c = x * y;
-  const double e = fma(-c, y, 1.0);
-  return fma(c * e, fma(0.375, e, 0.5), c);
+  const double c = x * y, half = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));
+  return fma(fma(-c, c, x) * half, fma(0.75, fma(-c, y, 1.0), 1.0), c);
 }
 
 // Sum of the NS sides' viscous fluxes . n over mu, momentum (w[0..2]) and energy

@@ -349,3 +349,40 @@ def test_gauss_nodes_scaled_down(N, k):
     U = _cuda(random_state(mesh.n_elems, N, seed=700 + N, rho=(0.95, 1.05), vel=0.2, p=(0.95, 1.05)))
     R = [dg.Solver(mesh, N, mu=0.01 * 2.0 ** x, nodes=dg.NODES_LG).time_derivative(U * 2.0 ** x) * 2.0 ** -x for x in (0, k)]
     assert float((R[1] - R[0]).abs().max()) <= (0.0 if k > -180 else 1e-12) * float(R[0].abs().max())
+
+
+@pytest.mark.parametrize("N", [1, 3, 6])
+def test_gas_without_pressure(orc, N):
+    """No pressure, no flow: the sound speed is 0 and so is R(U) on Gauss nodes
+    (the split form on LGL nodes divides by the pressure)."""
+    import paper_2605_28627_gb300 as dg
+    mesh = box_mesh(3, min(N, 4), deform="sinprod", rotate_seed=710 + N)
+    o, s = orc.Oracle(mesh, N, mu=0.01, nodes=1), dg.Solver(mesh, N, mu=0.01, nodes=dg.NODES_LG)
+    U = random_state(mesh.n_elems, N, seed=720 + N, rho=(0.95, 1.05), vel=0.0)
+    U[:, 4] = 0.0
+    assert not o.time_derivative(U).any()
+    assert not bool(s.time_derivative(_cuda(U)).any())
+
+
+def test_sound_speed_in_the_lax_friedrichs_flux():
+    """Densities that jump at the faces, no flow, uniform pressure: R of the mass is
+    sound speed times jump over the face weight.  One plane of faces of cubic cells,
+    N = 1 (w_0 = 1, J = 1/8): bar 6 ulp, the roundings of the terms around sqrt."""
+    import paper_2605_28627_gb300 as dg
+    mesh = box_mesh(8, 1)
+    s = dg.Solver(mesh, 1, mu=0.0)
+    rng = np.random.default_rng(730)
+    r = np.exp(rng.uniform(np.log(0.25), np.log(4.0), mesh.n_elems // 64))       # per plane of constant x
+    plane = np.arange(mesh.n_elems) % 8
+    rho = np.empty((mesh.n_elems, 2, 2, 2))
+    rho[:] = r[plane][:, None, None, None]
+    p = 2.0 ** rng.integers(-8, 8) * 1.3
+    U = np.zeros((mesh.n_elems, 5, 2, 2, 2))
+    U[:, 0], U[:, 4] = rho, p / 0.4
+    R = s.time_derivative(_cuda(U)).cpu().numpy()[:, 0]
+    L = np.longdouble
+    gm1 = L(1.4 - 1.0)
+    c = np.sqrt(L(1.4) * (gm1 * L(U[0, 4, 0, 0, 0])) / r.astype(L))
+    left = np.maximum(c, np.roll(c, 1)) * (np.roll(r, 1) - r)                    # at the faces of smaller x
+    scale = 0.5 * 8.0                                                            # lambda/2 and sJ / (J w_0)
+    assert np.abs(R[:, :, :, 0] / (scale * left[plane])[:, None, None] - 1).max() < 6 * 2.0 ** -52
