@@ -4,7 +4,7 @@
 #include <cmath>
 #include <cstdlib>
 
-#include "../paper_2605_28627_gb300/csrc/dg_fixed.cuh"
+#include "../paper_2605_28627_gb300/csrc/dg_adjoint_fx.cuh"
 
 using namespace dg;
 using L = long double;
@@ -39,7 +39,152 @@ static void flux(T ra, T rb, const T* ua, const T* ub, T ba, T bb, const T* sn, 
   }
 }
 
+// Logarithmic mean (a + b)/(2 F(f)), F = atanh(f)/f, and its derivatives.
+template <class T>
+static T log_mean(T a, T b, T& La, T& Lb) {
+  const T s = a + b, f = (a - b) / s, u = f * f;
+  T F = 1, dF = 0;   // dF = F'(f)
+  if (u < T(0.05)) {
+    T p = 1;
+    for (int k = 1; k < 20; ++k) {
+      dF += 2 * k * p * f / (2 * k + 1);
+      p *= u;
+      F += p / (2 * k + 1);
+    }
+  } else {
+    F = std::log(a / b) / (2 * f);
+    dF = (1 / (1 - u) - F) / f;
+  }
+  const T c = -dF / (F * F * s);   // of f_a = 2 b / s^2, f_b = -2 a / s^2
+  La = 1 / (2 * F) + c * b;
+  Lb = 1 / (2 * F) - c * a;
+  return s / (2 * F);
+}
+// Adjoint of the two-point flux, o = {density a, b, beta a, b, {u} (3), K}, and
+// the sum of each one's terms' magnitudes.
+template <class T>
+static void flux_vjp(T ra, T rb, const T* ua, const T* ub, T ba, T bb, const T* n, T ig, const T* w, T* o, T* mag) {
+  T Lra, Lrb, Lba, Lbb, u[3], un = 0, K = 0, fm[3], fmb[3], phb = 0, f0b = w[0];
+  const T rl = log_mean(ra, rb, Lra, Lrb), bl = log_mean(ba, bb, Lba, Lbb), isb = 1 / (ba + bb), ph = (ra + rb) * isb / 2;
+  for (int l = 0; l < 3; ++l) {
+    u[l] = (ua[l] + ub[l]) / 2;
+    un += u[l] * n[l];
+    K += (ua[l] * ua[l] + ub[l] * ub[l]) / 4;
+  }
+  const T f0 = rl * un, H = ig / (2 * bl) - K;
+  T m0 = std::fabs(w[0]) + std::fabs(w[4] * H);
+  f0b += w[4] * H;
+  for (int l = 0; l < 3; ++l) {
+    fm[l] = f0 * u[l] + ph * n[l];
+    fmb[l] = w[1 + l] + w[4] * u[l];
+    phb += fmb[l] * n[l];
+    f0b += fmb[l] * u[l];
+    m0 += std::fabs(fmb[l] * u[l]);
+  }
+  const T Hb = w[4] * f0, blb = -Hb * ig / (2 * bl * bl), sr = phb * isb / 2, sb = -phb * ph * isb, rlb = f0b * un;
+  o[0] = sr + rlb * Lra; o[1] = sr + rlb * Lrb;
+  o[2] = sb + blb * Lba; o[3] = sb + blb * Lbb;
+  for (int l = 0; l < 3; ++l) {
+    o[4 + l] = w[4] * fm[l] + f0 * fmb[l] + f0b * rl * n[l];
+    mag[4 + l] = std::fabs(w[4] * fm[l]) + std::fabs(f0 * fmb[l]) + m0 * rl * std::fabs(n[l]);
+  }
+  o[7] = -Hb;
+  mag[0] = mag[1] = std::fabs(sr) + m0 * std::fabs(un);
+  mag[2] = mag[3] = std::fabs(sb) + std::fabs(blb);
+  mag[7] = std::fabs(Hb);
+}
+
 extern "C" {
+
+// Adjoint of the two-point flux, states and metric terms as in check_pairs, the
+// cotangents of mass, momentum and energy below l0, lm, l4, rows of D below
+// 2^eD.  out[0..3]: rms error of the density, beta, velocity and |u|^2 adjoints
+// over the rms magnitude of their terms, out[4..7] of FP64, out[8]: smallest
+// shift to the sums' exponents, out[9]: log2 of the largest share after it,
+// out[10]: log2 of the largest share before it, out[11]: pairs outside the range.
+void check_pair_vjp(int count, double r0, double r1, double p0, double p1, double um, double jm, int axis, double gamma,
+                    int t0, double l0, double lm, double l4, int eD, double* out) {
+  srand48(15);
+  const double ig = 1.0 / (gamma - 1.0), jl = axis ? jm : 3 * jm, bmax = r1 / (8 * p0);
+  FxExp e{expo(r1), expo(um), expo(bmax), expo(jl) + t0, 0, 0, 0, 0};
+  const double bmin = std::max(r0 / (8 * p1), ldexp(1.0, e.b - 4));
+  e.lb = (float)(log2(bmin) - e.b - 1e-3);
+  const int eg = expo(ig);
+  auto low = [](double x) { return x > 0 ? std::max(expo(x), -200) : -200; };
+  const int e0 = low(l0), em = low(lm), e4 = low(l4);
+  const FxAdjAlign al = fx_adj_align(e, eg, e0, em, e4, eD);
+  const Fx G = fx_split(fx_from(ig, 62 - eg));
+  double ef[4] = {0}, ed[4] = {0}, sc[4] = {0}, least = 1e9, after = 0, before = 0;
+  long outside = 0;
+  for (int t = 0; t < count; ++t) {
+    const double ra = uniform(r0, r1), pa = uniform(p0, p1), near = t % 3 == 1 ? 1e-2 : 1e-5;
+    double rb = t % 3 == 0 ? uniform(r0, r1) : std::min(r1, std::max(r0, ra * (1 + uniform(-near, near))));
+    double pb = t % 3 == 0 ? uniform(p0, p1) : std::min(p1, std::max(p0, pa * (1 + uniform(-near, near))));
+    if (t % 7 == 0) { rb = ra; pb = pa; }
+    const double ba = 0.125 * ra / pa, bb = 0.125 * rb / pb;
+    const i64 xr[2] = {fx_from(ra, 60 - e.r), fx_from(rb, 60 - e.r)}, xb[2] = {fx_from(ba, 60 - e.b), fx_from(bb, 60 - e.b)};
+    if (std::min(std::min(xr[0], xr[1]), std::min(xb[0], xb[1])) < (i64)1 << 56 || ba < bmin || bb < bmin) { ++outside; continue; }
+    i64 su[3], sn[3], S[5];
+    double ua[3], ub[3], n[3], ka = 0, kb = 0, w[5];
+    for (int a = 0; a < 3; ++a) {
+      const bool on = !axis || a == 0;
+      ua[a] = uniform(-um, um); ub[a] = uniform(-um, um);
+      const double na = on ? uniform(-jm, jm) : 0, nb = on ? uniform(-jm, jm) : 0;
+      n[a] = 0.5 * (na + nb);
+      su[a] = fx_from(ua[a], 60 - e.u) + fx_from(ub[a], 60 - e.u);
+      sn[a] = fx_up(fx_from(na, 60 - e.j), t0) + fx_up(fx_from(nb, 60 - e.j), t0);
+      ka += ua[a] * ua[a]; kb += ub[a] * ub[a];
+    }
+    const double dab = uniform(-1, 1) * ldexp(1.0, eD), dba = uniform(-1, 1) * ldexp(1.0, eD);
+    L wl[5];
+    for (int c = 0; c < 5; ++c) {
+      const double top = c == 0 ? l0 : (c < 4 ? lm : l4), la = uniform(-top, top), lb = uniform(-top, top);
+      const int ec = c == 0 ? e0 : (c < 4 ? em : e4);
+      FxSum s = fx_zero<kFxUpD>();
+      fx_add(s, fx_split(fx_round(dab, kFxQD - eD)), fx_split(fx_from(la, 60 - ec)));
+      fx_add(s, fx_split(fx_round(dba, kFxQD - eD)), fx_split(fx_from(lb, 60 - ec)));
+      S[c] = fx_end<kFxUpD>(s);
+      w[c] = 2 * (dab * la + dba * lb);
+      wl[c] = 2 * ((L)dab * la + (L)dba * lb);
+    }
+    const FxPairAdj o = fx_pair_vjp(xr[0], xr[1], xb[0], xb[1], su, fx_from(ka, 58 - 2 * e.u) + fx_from(kb, 58 - 2 * e.u), sn, G,
+                                    e.j - t0, S, al, [](i64 a, i64 b, i64 c, i64 d, i64 y) {
+      double La, Lb;
+      FxMeansD m;
+      m.rln2 = fx_from(2.0 * log_mean((double)a, (double)b, La, Lb), 0);
+      m.ra = fx_from(La, 61); m.rb = fx_from(Lb, 61);
+      const double x = log_mean((double)c, (double)d, La, Lb);
+      m.hib = fx_from((double)y * (0.5 * ((double)c + (double)d) / x), 0);
+      m.ba = fx_from(La, 61); m.bb = fx_from(Lb, 61);
+      return m;
+    });
+    L lua[3], lub[3], ln[3], R[8], mag[8];
+    for (int a = 0; a < 3; ++a) { lua[a] = ua[a]; lub[a] = ub[a]; ln[a] = n[a]; }
+    flux_vjp<L>(ra, rb, lua, lub, 4 * (L)ba, 4 * (L)bb, ln, ig, wl, R, mag);
+    double D[8], dm[8];
+    flux_vjp<double>(ra, rb, ua, ub, 4 * ba, 4 * bb, n, ig, w, D, dm);
+    const i64 m[8] = {o.r[0], o.r[1], o.b[0], o.b[1], o.u.m[0], o.u.m[1], o.u.m[2], o.k.m};
+    const int ex[8] = {o.er, o.er, o.eb, o.eb, o.u.e, o.u.e, o.u.e, o.k.e}, top[4] = {al.erho, al.ebt, al.eub, al.ek};
+    for (int v = 0; v < 8; ++v) {
+      const int c = v < 2 ? 0 : (v < 4 ? 1 : (v < 7 ? 2 : 3));
+      const L unit = std::ldexp((L)1, top[c] - 60);   // the sums' scale, so that squares stay in range
+      ef[c] += (double)std::pow((std::ldexp((L)m[v], ex[v] - 60) - R[v]) / unit, 2);
+      ed[c] += (double)std::pow((D[v] - R[v]) / unit, 2);
+      sc[c] += (double)std::pow(mag[v] / unit, 2);
+      least = std::min(least, (double)(top[c] - ex[v]));
+      before = std::max(before, std::fabs((double)m[v]));
+      after = std::max(after, std::ldexp(std::fabs((double)m[v]), ex[v] - top[c]));
+    }
+  }
+  for (int c = 0; c < 4; ++c) {
+    out[c] = std::sqrt(ef[c] / sc[c]);
+    out[4 + c] = std::sqrt(ed[c] / sc[c]);
+  }
+  out[8] = least;
+  out[9] = std::log2(after);
+  out[10] = std::log2(before);
+  out[11] = (double)outside;
+}
 
 // Pairs with density in [r0, r1], pressure in [p0, p1], velocities below um,
 // metric terms below jm (axis: one component only) in an element whose largest

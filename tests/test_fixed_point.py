@@ -30,6 +30,8 @@ def lib(tmp_path_factory):
     L.check_rcp.restype = C.c_double
     L.check_pairs.argtypes = [C.c_int] + [C.c_double] * 6 + [C.c_int, C.c_double, C.c_int, C.c_double, C.c_void_p]
     L.check_lifting.argtypes = [C.c_int, C.c_int, C.c_void_p, C.c_int, C.c_double, C.c_int, C.c_void_p]
+    L.check_pair_vjp.argtypes = [C.c_int] + [C.c_double] * 6 + [C.c_int, C.c_double, C.c_int] + [C.c_double] * 3 + \
+        [C.c_int, C.c_void_p]
     return L
 
 
@@ -46,7 +48,7 @@ def test_reciprocal(lib):
 # density, pressure, velocity, metric terms, one-component metrics, gamma:
 # random states of the parity tests, low Mach numbers, the density wave, Mach 2
 # and 30, densities over the whole admitted range, gamma near 1 and large
-@pytest.mark.parametrize("r0,r1,p0,p1,um,jm,axis,gamma", [
+STATES = [
     (0.8, 1.2, 0.8, 1.2, 0.5, 1.0, 0, 1.4),
     (0.99, 1.01, 71.0, 72.0, 1.0, 0.01, 1, 1.4),
     (0.9999, 1.0001, 714285.0, 714286.0, 1.0, 0.3, 0, 1.4),
@@ -57,7 +59,10 @@ def test_reciprocal(lib):
     (0.126, 1.0, 0.1, 1.0, 0.3, 50.0, 0, 1.4),
     (1e-7, 1.2e-7, 1e20, 1.1e20, 1e13, 1e6, 1, 1.05),
     (0.8, 1.2, 0.8, 1.2, 0.5, 1.0, 1, 3.0),
-])
+]
+
+
+@pytest.mark.parametrize("r0,r1,p0,p1,um,jm,axis,gamma", STATES)
 @pytest.mark.parametrize("shift,loose", [(0, 1.0), (4, 1.0), (0, 1.99)])
 def test_two_point_flux(lib, r0, r1, p0, p1, um, jm, axis, gamma, shift, loose):
     out = np.zeros(8)
@@ -79,3 +84,21 @@ def test_lifted_gradient(lib, orc, N, shift):
     e_D = (0, 2, 3, 3, 4, 4, 5, 5, 5)[N - 1]
     lib.check_lifting(4000, N + 1, D.ctypes.data_as(C.c_void_p), e_D, 0.5 / w[0], shift, out.ctypes.data_as(C.c_void_p))
     assert out[0] <= out[1], out
+
+
+@pytest.mark.parametrize("r0,r1,p0,p1,um,jm,axis,gamma", STATES)
+@pytest.mark.parametrize("cotangent", [(1.0, 1.0, 1.0), (1e-6, 1.0, 1e6), (1e8, 1.0, 1e-8), (1.0, 0.0, 0.0),
+                                       (0.0, 0.0, 1.0), (1e-45, 1e-44, 1e-45)])
+@pytest.mark.parametrize("shift,e_D", [(0, 5), (4, 0)])
+def test_two_point_flux_adjoint(lib, r0, r1, p0, p1, um, jm, axis, gamma, cotangent, shift, e_D):
+    """Adjoint of the two-point flux for densities, beta, velocity and |u|^2: errors
+    over the terms' size no larger than FP64's; no share above the exponent of its
+    sum, whose 27 terms (N = 9) stay below 2^63; mantissas below 2^60."""
+    out = np.zeros(12)
+    n = 3000
+    lib.check_pair_vjp(n, r0, r1, p0, p1, um, jm, axis, gamma, shift, *cotangent, e_D, out.ctypes.data_as(C.c_void_p))
+    assert out[11] < 0.8 * n
+    assert out[8] >= 0 and out[9] < 63 - np.log2(27) and out[10] <= 60.0, out[8:]
+    fixed, fp64 = out[:4], out[4:8]
+    some = ~np.isnan(fp64)      # no adjoint of beta and |u|^2 from the mass equation alone
+    assert some[0] and some[2] and (fixed[some] <= fp64[some]).all(), (fixed, fp64)
