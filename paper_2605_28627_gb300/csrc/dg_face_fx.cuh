@@ -69,7 +69,7 @@ __device__ __forceinline__ bool face_visc_fx(const double* __restrict__ gL, cons
       mu = max(mu, mag(s ? uR[l] : uL[l]));
     }
   }
-  if (!fx_in_range(mg, 90) || !fx_in_range(mt, 90) || !fx_in_range(mu, 90)) return false;
+  if (!(fx_in_range(mg, 90) & fx_in_range(mt, 90) & fx_in_range(mu, 90))) return false;
   const int eg = fx_expo(mg), et = fx_expo(mt), eu = fx_expo(mu);
   Fx n[3];
 #pragma unroll

@@ -21,8 +21,8 @@ __host__ __device__ __forceinline__ int fx_expo(int h) {
 // Whether fixed point may hold the quantity: zero, or 2^kFxLow <= 2^e < 2^high
 // (scaled below 2^kFxLow it would lose digits).
 __host__ __device__ __forceinline__ bool fx_in_range(int h, int high) {
-  const int e = (h >> 20) - 1022;
-  return h == 0 || (e >= kFxLow && e < high);
+  constexpr int low = (kFxLow + 1022) << 20;
+  return ((unsigned)(h - low) < (unsigned)((high - kFxLow) << 20)) | (h == 0);
 }
 __device__ __forceinline__ int fx_mag(double x) { return __double2hiint(x) & 0x7fffffff; }
 // maxima of v[0..C) over the lanes of element el of this warp, into mx[0..C)

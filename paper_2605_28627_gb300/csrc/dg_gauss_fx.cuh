@@ -237,8 +237,7 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
   for (int t = threadIdx.x; t < EPB * kCount; t += blockDim.x) s_mx[t / kCount][t % kCount] = 0;
   if (threadIdx.x == 0 && g.source == DG_SOURCE_MMS)
     sincospi(a.clock[0] + a.c_stage * a.clock[1], &s_tc[0], &s_tc[1]);
-  const float4 ejv = active ? ejx[e] : make_float4(1000.0f, 0.0f, 0.0f, 0.0f);
-  const FxMetricShifts sh{STRETCH ? __float_as_int(ejv.w) : 0};
+  const FxMetricShifts sh{STRETCH && active ? __float_as_int(ejx[e].w) : 0};
   __syncthreads();
   double q[5] = {1, 0, 0, 0, 0}, gr[12];
   double u = 0, v = 0, w = 0, p = 0;
@@ -290,11 +289,11 @@ __device__ __forceinline__ bool volume_lg_fx(const StageArgs& a, const double* _
 #pragma unroll
   for (int c = 0; c < kCount; ++c) {
     x[c] = fx_expo(s_mx[le][c]);
-    in = in && fx_in_range(s_mx[le][c], 90);
+    in = in & fx_in_range(s_mx[le][c], 90);
   }
-  const int ej = (int)ejv.x, hm = fx_mag(g.mu), hl = fx_mag(g.mu * g.kappa);
+  const int ej = active ? (int)ejx[e].x : 1000, hm = fx_mag(g.mu), hl = fx_mag(g.mu * g.kappa);
   const int em = fx_expo(hm), el = fx_expo(hl);
-  const bool act = active && in && ej < 90 && fx_in_range(hm, 90) && fx_in_range(hl, 90);
+  const bool act = active & in & (ej < 90) & fx_in_range(hm, 90) & fx_in_range(hl, 90);
   if (id == 0) state[le] = active ? (act ? 1 : 2) : 0;
   // bits after the point of the mass (q0), momentum (qm) and energy (qe) fluxes,
   // + t_d in direction d: below 2^61.3, so that six of a line's n + 2 terms fit in FxSum's c (the part of
