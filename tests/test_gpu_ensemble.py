@@ -218,3 +218,21 @@ def test_members_outside_the_tile_tables_run_as_single_units(orc, dg):
         err = np.abs(U.cpu().numpy() - ref).max() / np.abs(ref).max()
         assert err <= 1e-10, (o.N, err)
     ens.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_tuning_leaves_state_and_register_out(dg, precision):
+    """The tuning of a first step runs stages on the members' own buffers: with a
+    register full of NaN the step is the same as alone, bit for bit."""
+    runs = [_make(dg, m, precision) for m in MEMBERS if m["N"] > 3]
+    Us = [r[1].clone() for r in runs]
+    Gs = [torch.full_like(U, float("nan")) for U in Us]
+    ens = dg.Ensemble([r[0] for r in runs])
+    ens.step(Us, Gs, [0.0] * len(runs), [r[2] for r in runs], nsteps=1)
+    for (s, U0, dt), U in zip(runs, Us):
+        ref = U0.clone()
+        s.rk_step(ref, torch.empty_like(ref), 0.0, dt, 1)
+        assert torch.equal(U, ref)
+    ens.close()
+    for r in runs:
+        r[0].close()
