@@ -176,6 +176,19 @@ struct InitScratch {
   }
 };
 
+// Fixed-point metric terms, 80 B per node.  A mesh that leaves no room for them,
+// or with them none for a state, its register and a result (120 B per node), does
+// without: every element then runs in FP64.
+static void alloc_fixed_metrics(Ctx& c) {
+  const size_t nodes = (size_t)c.E * c.P;
+  size_t avail = 0, total = 0;
+  if (cudaMemGetInfo(&avail, &total) == cudaSuccess && avail >= nodes * (80 + 120) &&
+      cudaMalloc((void**)&c.d_jx, sizeof(long long) * nodes * 10) == cudaSuccess)
+    return;
+  c.d_jx = nullptr;
+  cudaGetLastError();
+}
+
 // `c` holds the context under construction, so that the caller can free it
 // if a host allocation throws half-way.
 static dg_status init_impl(const dg_mesh* mesh, const dg_params* prm, int device, dg_ctx** out, dg_ctx*& c) {
@@ -336,9 +349,7 @@ static dg_status init_impl(const dg_mesh* mesh, const dg_params* prm, int device
        (!alloc((void**)&c->d_Uf, sizeof(double) * E * 6 * 5 * NN, "alloc face states") ||
         !alloc((void**)&c->d_gf, sizeof(double) * E * 6 * 12 * NN, "alloc face gradients") ||
         !alloc((void**)&c->d_lgb, sizeof(double) * (2 * NN + 5 * c->n), "alloc Gauss basis"))) ||
-      (prm->precision != DG_FP32OP &&
-       (!alloc((void**)&c->d_jx, sizeof(long long) * E * 10 * P, "alloc metrics (fixed point)") ||
-        !alloc((void**)&c->d_ejx, sizeof(float4) * E, "alloc metric exponents"))) ||
+      (prm->precision != DG_FP32OP && !alloc((void**)&c->d_ejx, sizeof(float4) * E, "alloc metric exponents")) ||
       (prm->precision == DG_FP32OP &&
        (!alloc((void**)&c->d_metrics_f, sizeof(float) * E * 10 * P, "alloc metrics (fp32)") ||
         !alloc((void**)&c->d_facegeo_f, sizeof(float) * c->nfaces * 4 * NN, "alloc facegeo (fp32)"))))
@@ -369,6 +380,7 @@ static dg_status init_impl(const dg_mesh* mesh, const dg_params* prm, int device
   const size_t m3 = (size_t)(mesh->ngeo + 1) * (mesh->ngeo + 1) * (mesh->ngeo + 1);
   cudaError_t err = cudaMalloc(&tmp.d_xgeo, sizeof(double) * E * 3 * m3);
   if (err == cudaSuccess) err = cudaMalloc(&tmp.d_bad, 2 * sizeof(int));
+  if (err == cudaSuccess && c->d_ejx) alloc_fixed_metrics(*c);
   double* d_xgeo = tmp.d_xgeo;
   int* d_bad = tmp.d_bad;
   if (err == cudaSuccess) err = cudaMemcpyAsync(d_xgeo, mesh->xgeo, sizeof(double) * E * 3 * m3, cudaMemcpyHostToDevice, s);
@@ -418,7 +430,7 @@ static dg_status init_impl(const dg_mesh* mesh, const dg_params* prm, int device
   if (err == cudaSuccess) err = setup_kernels(c->N);
   if (err == cudaSuccess) err = build_geometry(*c, d_xgeo, mesh->ngeo, d_bad, s);
   if (err == cudaSuccess && prm->nodes == DG_NODES_LG) err = gauss_geometry(*c, d_bad, s);
-  if (err == cudaSuccess && c->d_jx) err = launch_fx_metrics(*c, d_bad + 1, s);
+  if (err == cudaSuccess && c->d_ejx) err = launch_fx_metrics(*c, d_bad + 1, s);
   if (err == cudaSuccess && prm->source == DG_SOURCE_MMS) err = launch_mms_phase(*c, s);
   if (err == cudaSuccess && prm->precision == DG_FP32OP) {
     err = launch_to_float(c->d_metrics, c->d_metrics_f, (size_t)E * 10 * P, s);

@@ -79,8 +79,9 @@ constexpr double kFxVary = 16.0;
 // Once per context: metric terms and 1/J as integers (jx [E][10][P]): rows
 // 0..8 with 60 - e_j bits, e_j of the element's largest sum over l of |J
 // a^d_l|; row 9 with 62 - e_i bits.  ej [E]: e_j, the logarithm of the largest
-// sum less e_j (rounded up), e_i, FxMetricShifts.  An element with exponents out of range, with 1/J varying
-// by more than 2^8 or stretched beyond kFxStretch gets e_j = 1000: FP64 only.
+// sum less e_j (rounded up), e_i, FxMetricShifts.  An element with exponents out
+// of range, with 1/J varying by more than 2^8 or stretched beyond kFxStretch gets
+// e_j = 1000: FP64 only; so does every element if there is no jx (null).
 // With facegeo (Gauss nodes, whose face points are not nodes) e_j and c cover
 // the surface elements of the element's faces too.  *stretch: set if any element
 // in range has a t (on Gauss nodes a t or a c) other than 0.
@@ -121,7 +122,7 @@ __global__ void __launch_bounds__(256) k_fx_metrics(const double* __restrict__ m
   auto size = [](unsigned h) { return __hiloint2double((int)h, 0); };
   const unsigned most = max(s_row[0], max(s_row[1], s_row[2])), h = max(most, s_max[0]);
   const int e = expo(h), ei = expo(s_max[1]), emin = expo(0x7fffffffu - s_max[2]);
-  bool fine = e > -90 && e < 90 && ei > -90 && ei < 90 && ei - emin <= 8;
+  bool fine = jx != nullptr && e > -90 && e < 90 && ei > -90 && ei < 90 && ei - emin <= 8;
   int t[3], w = 0;
   for (int d = 0; d < 3; ++d) {
     t[d] = expo(most) - expo(s_row[d]);
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(256) k_fx_metrics(const double* __restrict__ m
   }
   if (threadIdx.x == 0)
     ej[blockIdx.x] = make_float4(fine ? (float)e : 1000.0f, fx_log_mantissa((int)h, 1), (float)ei, __int_as_float(fine ? w : 0));
-  for (int x = threadIdx.x; x < 10 * P; x += blockDim.x)
+  for (int x = threadIdx.x; jx != nullptr && x < 10 * P; x += blockDim.x)
     jx[(size_t)blockIdx.x * 10 * P + x] = fine ? fx_from(mt[x], x < 9 * P ? kFxQ - e : 62 - ei) : 0;
 }
 

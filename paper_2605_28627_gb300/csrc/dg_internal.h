@@ -124,7 +124,7 @@ struct Ctx {
   double* d_mms = nullptr;       // [E][2][P] sin, cos of pi (x + y + z); manufactured source only
   double* d_facegeo = nullptr;   // [F][4][NN]: unit normal (3), surface element
   float* d_metrics_f = nullptr;  // FP32 copies for the FP32-operator path
-  long long* d_jx = nullptr;     // [E][10][P] metric terms and 1/J in fixed point (FP64 operator)
+  long long* d_jx = nullptr;     // [E][10][P] metric terms and 1/J in fixed point (FP64 operator, if they fit)
   float4* d_ejx = nullptr;       // [E] their exponents (k_fx_metrics)
   bool fx_stretch = false;       // whether any element's directions differ by a factor 2 (k_fx_metrics)
   float* d_facegeo_f = nullptr;

@@ -435,8 +435,8 @@ __device__ __forceinline__ bool volume_lat_fx(const StageArgs& a, const double* 
   return true;
 }
 
-// FP64 body: elements out of the fixed-point range, and Sutherland's law
-// (whose factor every thread of a node would have to apply to the gradients).
+// FP64 body: elements out of the fixed-point range, contexts without
+// fixed-point metric terms, and Sutherland's law (whose factor every thread of a node would have to apply to the gradients).
 template <int N>
 constexpr size_t volume_lat_f64_bytes() {
   constexpr int n = N + 1, P = n * n * n;
@@ -639,7 +639,7 @@ k_volume_lat(StageArgs a, const double* __restrict__ metrics, const i64* __restr
              Gas g, double inv_w0) {
   extern __shared__ __align__(16) unsigned char lat_raw[];
   __shared__ double s_tc[2];
-  if (g.visc_law != DG_VISC_SUTHERLAND) {
+  if (g.visc_law != DG_VISC_SUTHERLAND && jx != nullptr) {
     if (volume_lat_fx<N, STRETCH>(a, metrics, jx, ejx, grad, fstar, elem_face, mms, Dg, E, g, inv_w0, lat_raw, s_tc)) return;
     __syncthreads();
   } else {

@@ -182,9 +182,11 @@ __device__ __forceinline__ bool volume_body_fx(const StageArgs& a, const double*
   i64 Ja[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
   double gr[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   if (active) {
-    const i64* mt = jx + (size_t)e * 10 * P + id;
+    if (jx != nullptr) {
+      const i64* mt = jx + (size_t)e * 10 * P + id;
 #pragma unroll
-    for (int r = 0; r < 9; ++r) Ja[r] = mt[r * P];
+      for (int r = 0; r < 9; ++r) Ja[r] = mt[r * P];
+    }
     const double* gg = grad + (size_t)e * 12 * P + id;
 #pragma unroll
     for (int r = 0; r < 12; ++r) gr[r] = gg[r * P];

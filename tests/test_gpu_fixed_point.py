@@ -386,3 +386,31 @@ def test_sound_speed_in_the_lax_friedrichs_flux():
     left = np.maximum(c, np.roll(c, 1)) * (np.roll(r, 1) - r)                    # at the faces of smaller x
     scale = 0.5 * 8.0                                                            # lambda/2 and sJ / (J w_0)
     assert np.abs(R[:, :, :, 0] / (scale * left[plane])[:, None, None] - 1).max() < 6 * 2.0 ** -52
+
+
+@pytest.mark.parametrize("N,K,nodes", [(3, 40, 0), (2, 44, 1)])
+def test_mesh_that_leaves_no_room_for_fixed_point(N, K, nodes):
+    """With the device memory filled so that the fixed-point copy of the metric
+    terms (80 B per node) does not fit, a context runs in FP64 instead of failing."""
+    import paper_2605_28627_gb300 as dg
+    mesh = box_mesh(K, 1)
+    n = mesh.n_elems * (N + 1) ** 3
+    U = _cuda(random_state(mesh.n_elems, N, seed=740, rho=(0.95, 1.05), vel=0.2, p=(0.95, 1.05)))
+    out, G = torch.empty_like(U), torch.empty_like(U)
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    s = dg.Solver(mesh, N, mu=0.01, nodes=nodes)
+    used = free0 - torch.cuda.mem_get_info()[0]
+    ref = s.time_derivative(U).clone()
+    s.close()
+    torch.cuda.synchronize()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - used + 40 * n, dtype=torch.uint8, device="cuda")
+    s = dg.Solver(mesh, N, mu=0.01, nodes=nodes)
+    left = torch.cuda.mem_get_info()[0]
+    del filler
+    torch.cuda.empty_cache()
+    assert left > 20 * n          # of 40 B per node, less the allocator's granularity
+    s.time_derivative(U, out)
+    assert float((out - ref).abs().max()) <= 1e-12 * float(ref.abs().max())
+    s.rk_step(U, G, 0.0, 1e-6, 1)
+    assert bool(torch.isfinite(s.time_derivative_vjp(U, ref, out)).all())
