@@ -2,16 +2,16 @@
 //
 // Why: this GPU issues an FP64 instruction of one warp in 67.6 cycles per SM
 // sub-partition (measured with a chain of DFMAs), an integer add in 1.1 and a
-// 32 x 32 + 64-bit multiply-add (IMAD.WIDE) in about 2.2.  A product of two
-// 62-bit fixed-point numbers takes three of those and a few adds, 13 cycles
-// in all, and a sum two adds, 2.2 cycles.  So the operator's inner sums run on
-// 64-bit integers: a quantity q with |q| < 2^e over the element is held as
-// round(q 2^(Q - e)), with the exponents e taken per element from the data
+// 32 x 32 + 64-bit multiply-add (IMAD.WIDE) in 4.0.  A product of two 62-bit
+// fixed-point numbers takes three of those and a few adds, 13 cycles in all,
+// and a sum two adds, 2.2 cycles.  So the operator's inner sums run on 64-bit
+// integers: a quantity q with |q| < 2^e over the element is held as q 2^(Q - e),
+// truncated (D: rounded), with the exponents e taken per element from the data
 // (fields of one element share an exponent, as the terms that meet in one sum
 // do).  The quantisation is 2^-60 of the element's largest value where FP64
 // carries 2^-53 of each value; elements whose density or beta varies by more
-// than a factor 8 to 16, or that hold a non-finite or non-positive value, take
-// the FP64 body instead.
+// than a factor 8 to 16, whose cells are stretched by 32 or more, or that hold a
+// non-finite, non-positive or extremely small value, take the FP64 body instead.
 //
 // Every function is plain integer C++ (host and device), so that the error
 // bounds can be checked on the CPU.
