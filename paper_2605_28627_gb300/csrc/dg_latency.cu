@@ -47,10 +47,10 @@ struct LatShape {
 // g_{a,d} = (1/J) sum_d' Ja^{d'}_d (D_d' phi_a + jump_d').
 // The threads of direction 0 evaluate the node's phi while the others evaluate
 // the neighbours' at the face points; the jump (phi_nbr - phi) h, h = +-1/(2
-// w_0), goes into the line sum, its own part through D's corners (D_00 + 1/(2
-// w_0) = 0 there up to rounding), the neighbour's by a fused multiply-add.  Bound
-// by the memory latency of its two dependent loads and by some 50 FP64
-// instructions a warp.
+// w_0), starts the line sum (its shares summed one by one, the own one through
+// D's corners, gave up to 1.9 times the error in the heat flux).  Bound by the
+// memory latency of its two dependent loads and by some 55 FP64 instructions a
+// warp.
 template <int N>
 constexpr size_t lift_lat_smem_bytes() {
   constexpr int P = LatShape<N>::P, NN = LatShape<N>::NN;
@@ -97,10 +97,7 @@ k_lift_lat(const double* __restrict__ U_, const double* __restrict__ metrics, co
       apply_flip<n>(code & 7, pq % n, pq / n, p2, q2);
       nbr[x] = dg_idx(nb >> 3, E, kSiteLiftNbr) * 5 * P + face_node<n>(nb & 7, p2, q2);
     }
-    for (int t = threadIdx.x - P; t < n * n; t += 2 * P) {
-      const double dr = Dg[t];
-      sD[t] = t == 0 ? dr + hw : (t == n * n - 1 ? dr - hw : dr);
-    }
+    for (int t = threadIdx.x - P; t < n * n; t += 2 * P) sD[t] = Dg[t];
   }
   wait_previous();
   const double* U = after_previous(U_);
@@ -126,10 +123,9 @@ k_lift_lat(const double* __restrict__ U_, const double* __restrict__ metrics, co
     jm = snb + (2 * d + (r == N ? 1 : 0)) * 4 * NN + (d == 0 ? j : i) + n * (d == 2 ? j : k);
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
-    double s = 0.0;
+    double s = jm ? (jm[a * NN] - sphi[a * P + id]) * h : 0.0;
 #pragma unroll
     for (int m = 0; m < n; ++m) s = fma(sD[r * n + m], sphi[a * P + line0 + m * stride], s);
-    if (jm) s = fma(h, jm[a * NN], s);
     sdd[(a * 3 + d) * P + id] = s;
   }
   __syncthreads();
