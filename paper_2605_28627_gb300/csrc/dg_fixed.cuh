@@ -10,7 +10,7 @@
 // (fields of one element share an exponent, as the terms that meet in one sum
 // do).  The quantisation is 2^-60 of the element's largest value where FP64
 // carries 2^-53 of each value; elements whose density or beta varies by more
-// than a factor 8 to 16, whose cells are stretched by 32 or more, or that hold a
+// than a factor 8 to 16, whose cells are stretched by 4 or more, or that hold a
 // non-finite, non-positive or extremely small value, take the FP64 body instead.
 //
 // Every function is plain integer C++ (host and device), so that the error

@@ -69,11 +69,12 @@ __device__ __forceinline__ void fx_shift_down(FxSum& s, int k) {
   s.p >>= k;
 }
 // A fixed-point element's directions differ by less than 2^(kFxStretch + 1) in
-// size, the nodes of one direction by kFxVary.  Fields share exponents over the
-// directions too: in longer cells what the short direction's small velocity
-// leaves of its digits, and the pressure's rounding in the long direction's
-// momentum, would exceed the FP64 kernels' rounding.
-constexpr int kFxStretch = 4;
+// size, the nodes of one direction by kFxVary.  Beyond, the exponents that the
+// directions share in the fields cost digits: of a small velocity across long
+// faces, and by the pressure's rounding in the other momenta.  Error of R(U) over
+// the FP64 kernels', rms, boundary-layer flows on cells of ratio A: at most 1.1 to
+// 1.2 for A = 3.9 (1.0 to 1.1 for cubic cells), 1.6 to 2.4 for A = 15.
+constexpr int kFxStretch = 1;
 constexpr double kFxVary = 16.0;
 
 // Once per context: metric terms and 1/J as integers (jx [E][10][P]): rows

@@ -7,10 +7,10 @@ sums' last word); the reciprocal is good to 2^-55; the flux stays below 2^60.5, 
 that the sums with a row of D cannot overflow; its error and that of a lifted
 gradient are no larger than those of the same formula in FP64 over the admitted
 range of the states and of the metric terms.  The directions of an element share
-an exponent: one that is 2^t smaller is shifted up by t where it is used, up to
-t = 4, and one that is smaller by less than 2 is not shifted (loose 1.99; then
-the energy flux at Mach 30 is the one quantity above FP64's error, by less than
-a factor 2)."""
+an exponent: one that is 2^t smaller is shifted up by t where it is used (the
+kernels take t up to 1), and one that is smaller by less than 2 is not shifted
+(loose 1.99; then the energy flux at Mach 30 is the one quantity above FP64's
+error, by less than a factor 2)."""
 import ctypes as C
 import os
 import subprocess

@@ -174,15 +174,15 @@ def _axis_flow(s, mesh, N, L, ax, comp):
     return U
 
 
-# in fixed point with the directions shifted by 1 and 4, and in FP64
-CELLS = [(3.0, 1.0, 24.0), (1.0, 10.0, 1000.0)]
+# in fixed point with two directions shifted, and in FP64
+CELLS = [(3.0, 1.2, 3.5), (3.0, 1.0, 24.0), (1.0, 10.0, 1000.0)]
 
 
 LGL = [(1, 3, 0), (1, 13, 0), (2, 3, 0), (3, 3, 0), (3, 7, 0), (4, 3, 0), (5, 3, 0), (7, 2, 0), (8, 2, 0)]
 LG = [(1, 3, 1), (3, 3, 1), (4, 2, 1), (6, 2, 1)]
 
 
-@pytest.mark.parametrize("N,K,nodes,k", [c + (k,) for c in LGL + LG for k in (1, 4, 5, 20) if not c[2] or k <= 5])
+@pytest.mark.parametrize("N,K,nodes,k", [c + (k,) for c in LGL + LG for k in (1, 2, 5, 20) if not c[2] or k <= 5])
 def test_flow_along_stretched_cells(N, K, nodes, k):
     """Cells 2^k times as long along an axis as across it and an inviscid flow
     that varies along this axis: every term of the mass, energy and axis momentum
@@ -204,7 +204,7 @@ def test_flow_along_stretched_cells(N, K, nodes, k):
 
 
 @pytest.mark.parametrize("N,K,nodes", LGL + [(9, 2, 0)] + LG)
-@pytest.mark.parametrize("k", [1, 4, 5, 20])
+@pytest.mark.parametrize("k", [1, 2, 5, 20])
 def test_gradients_along_stretched_cells(orc, N, K, nodes, k):
     """The same cells with a transverse velocity that varies along the axis:
     the dissipation is a sum of squares of its lifted gradient, which the rounding
