@@ -46,7 +46,7 @@ def build_mesh(N):
 # DRAM bytes (read + write) per launch of the volume kernel on this workload,
 # the median over the launches of one ncu capture of the current kernels
 # (profiles/volume_traffic_N7_mms16.txt); absent = not captured.
-MEASURED_TRAFFIC = {(7, "fp64"): 581.094656e6 + 231.395712e6, (7, "fp32op"): 406.712064e6 + 143.888640e6}
+MEASURED_TRAFFIC = {(7, "fp64"): 576.639232e6 + 200.861824e6, (7, "fp32op"): 406.712064e6 + 143.888640e6}
 # The other orders of the sweep, DRAM read + write per launch (medians, MB) from one capture of
 # the volume kernels of `--sweep 1,2,3,4,5,6,8,9`; up to N = 4 the working set stays in the
 # 129 MB L2 between launches, so DRAM sees less than the kernel's algorithmic bytes.
@@ -54,6 +54,10 @@ for _N, _f64, _f32 in ((1, 11.6, 7.1), (2, 37.8, 22.7), (3, 79.7, 52.3), (4, 168
                        (6, 497.5, 344.9), (8, 1071.0, 799.7), (9, 1732.3, 1066.5)):
     MEASURED_TRAFFIC[(_N, "fp64")] = _f64 * 1e6
     MEASURED_TRAFFIC[(_N, "fp32op")] = _f32 * 1e6
+# What holds the FP64 volume kernel at N = 7: shares of the cycles in which each unit is busy,
+# 12^3 elements (profiles/fixed_point_kernels.md); a captured figure, not one of this run.
+VOLUME_BUSY = {"issue": 49.2, "integer_multiplier": 50.1, "alu": 45.0, "fp64_pipe": 28.0,
+               "source": "ncu capture, profiles/fixed_point_kernels.md"}
 
 
 # ---------------------------------------------------------------------------
@@ -1181,6 +1185,7 @@ def main():
                 "kernel": "k_volume2<%d> (split-form volume + surface + Jacobian + LSERK update)" % N,
                 "peak_source": hbm_src,
                 "limited_by": "integer multiplier and issue slots (block fixed point), not HBM",
+                "busy_pct": VOLUME_BUSY if N == 7 else None,
                 "fp64_equivalent": {"tflops": achieved, "fp64_pipe_tflops": fp64_peak, "ratio": achieved / fp64_peak,
                                     "peak_source": "measured FP64 DFMA chain throughput on this GPU (dg_probe_peaks)"},
                 "stage_ms": {"lift": ms3[0], "face": ms3[1], "volume": ms3[2]}}

@@ -14,9 +14,10 @@
 // Bound and measured: the FP64 pairs (about 135 FP64 instructions each) held the
 // FP64 pipe 87 % busy; a pair here costs some 900 integer instructions, and the
 // viscous part's 250 FP64 instructions a node run beside them.  One
-// vector-Jacobian product on 16^3 elements, before -> now (us): N = 3 976 -> 717,
-// 5 3787 -> 2124, 7 10464 -> 5666; its error against 64 bits is 0.8 to 1.0 of
-// the FP64 pairs'.
+// vector-Jacobian product on 16^3 elements, FP64 pairs -> these (us): N = 3 976 ->
+// 717, 5 3787 -> 2124, 7 10464 -> 5666 (with the face and viscous parts as they
+// are now 505, 1468, 4306); its error against 64 bits is 0.7 to 1.1 of the FP64
+// pairs'.
 #pragma once
 
 #include "dg_fixed.cuh"

@@ -6,7 +6,7 @@
 // Bound and measured: the FP64 pipe, as before, with half the instructions.  128
 // threads, 168 registers; five or six blocks per SM (with fewer registers) took 1
 // to 9 % longer.  Manufactured solution, 16^3 elements, LLF, us per launch before
-// -> now: N = 1 24 -> 18, 3 73 -> 47, 5 147 -> 92, 7 257 -> 149, 9 397 -> 226.
+// -> now: N = 1 24 -> 18, 3 73 -> 50, 5 147 -> 93, 7 257 -> 150, 9 397 -> 225.
 #pragma once
 
 #include "dg_fx_metrics.cuh"

@@ -6,11 +6,11 @@
 // Bound and measured: the FP64 kernels held the FP64 pipe 87 to 92 % busy (421
 // FP64 instructions a node in the lifting at N = 3, 233 in the volume kernel).
 // Now the lifting's 156 multiply-adds a node and direction (12 cycles each on
-// the quarter-rate integer multiplier; ALU and multiplier 53 and 49 % busy at N
+// the quarter-rate integer multiplier; ALU and multiplier 56 and 50 % busy at N
 // = 3) and the volume kernel's remaining FP64 work and loads hold them.
 // Manufactured solution, 16^3 elements, us per launch before -> now: lifting
-// with prolongation N = 3 226 -> 118, 5 792 -> 354, 7 1985 -> 898; volume N = 3
-// 134 -> 68, 5 466 -> 195, 7 1225 -> 486.
+// with prolongation N = 3 226 -> 119, 5 792 -> 356, 7 1985 -> 900; volume N = 3
+// 134 -> 74, 5 466 -> 199, 7 1225 -> 500.
 #pragma once
 
 #include "dg_fx_metrics.cuh"

@@ -759,8 +759,8 @@ cudaError_t setup_latency(int N) {
 // Whether the context takes the latency kernels: FP64, LGL nodes, N <= 3 and
 // at most kLatencyNodes nodes.  They pay where the one-thread-per-node kernels
 // leave sub-partitions idle and lose where the mesh fills the GPU (Taylor-Green,
-// us per stage, one-thread-per-node -> these: 4^3 N = 1 32.1 -> 15.2, N = 2 35.8
-// -> 14.9, N = 3 32.5 -> 16.2; 6^3 N = 3 32.7 -> 23.5; 7^3 36.9 -> 33.7; but 8^3
+// us per stage, one-thread-per-node -> these: 4^3 N = 1 32.1 -> 15.1, N = 2 35.8
+// -> 15.0, N = 3 32.5 -> 16.6; 6^3 N = 3 32.7 -> 24.1; 7^3 36.9 -> 33.7; but 8^3
 // 39.2 -> 40.1, 11^3 N = 2 46.0 -> 45.0, 16^3 N = 1 43.8 -> 57.9).
 bool use_latency_kernels(const Ctx& c) {
   return c.prm.precision == DG_FP64 && c.prm.nodes == DG_NODES_LGL && c.N <= 3 && c.M == 0 &&

@@ -6,10 +6,10 @@
 // Bound and measured: lift_body<N, double> held the FP64 pipe 93 % busy (150
 // FP64 instructions a node at N = 7); here about 25 are left, and the integer
 // part takes some 1300 issue slots a node.  Two 512-thread blocks per SM (64
-// registers, no spills) at N = 7: three (42 registers) 251 us, one 331.
+// registers, a word spilled) at N = 7: three (42 registers) 251 us, one 331.
 // Manufactured solution, 16^3 elements, us per launch before -> now: N = 1 18 ->
-// 17, 2 42 -> 31, 3 73 -> 39, 4 144 -> 70, 5 250 -> 104, 6 415 -> 175, 7 627 ->
-// 243, 8 970 -> 468, 9 1393 -> 628.
+// 17, 2 42 -> 29, 3 73 -> 39, 4 144 -> 70, 5 250 -> 104, 6 415 -> 189, 7 627 ->
+// 243, 8 970 -> 472, 9 1393 -> 639.
 #pragma once
 
 #include "dg_fx_metrics.cuh"

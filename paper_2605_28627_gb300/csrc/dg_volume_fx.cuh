@@ -12,10 +12,10 @@
 // instructions a node at N = 7, 67.6 cycles each); here a pair costs about 330
 // instructions and 445 cycles of the integer multiplier (quarter rate), and a
 // node about 70 FP64 instructions.  Neither pipe is full (issue slots and
-// multiplier 47 % busy at N = 7): barriers and the latency of the FP64 prologue
+// multiplier 49 and 50 % busy at N = 7): barriers and the latency of the FP64 prologue
 // and epilogue hold it.  Manufactured solution, 16^3 elements, us per launch
-// before -> now: N = 1 41 -> 25, 2 146 -> 55, 3 295 -> 90, 4 655 -> 180, 5 1293
-// -> 356, 6 2239 -> 604, 7 3533 -> 1010, 8 5822 -> 1845, 9 8806 -> 3106.
+// before -> now: N = 1 41 -> 25, 2 146 -> 55, 3 295 -> 92, 4 655 -> 182, 5 1293
+// -> 356, 6 2239 -> 607, 7 3533 -> 1010, 8 5822 -> 1843, 9 8806 -> 3130.
 #pragma once
 
 #include "dg_fx_metrics.cuh"
